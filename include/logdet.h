@@ -101,7 +101,9 @@ typedef struct {
     double lambda_max;        /* > 0: user upper spectral bound; else library bound */
     void *cuda_stream;        /* cudaStream_t to run on; NULL = a stream the context owns */
     const int32_t *colouring; /* optional host colouring (n ints >= 0); NULL = greedy */
-    int32_t engine;           /* 0 auto, 1 multi-CTA grid engine, 2 one-CTA-per-tile engine */
+    int32_t engine;           /* 0 auto, 1 multi-CTA grid engine, 2 one-CTA-per-tile engine.
+                                 Auto runs a grid kind's solve on chip (the resident engine)
+                                 where that is estimated faster than streaming its vectors */
     int32_t chunk_iters;      /* iterations per captured CUDA graph chunk; 0 = auto */
     double reliable_delta;    /* > 0: reliable-update residual replacement (grid engine).  The
                                  seed solution is split into an FP64 part x_hi and a vector-
@@ -126,7 +128,8 @@ typedef struct {
     int32_t n_shifts;         /* quadrature nodes N */
     int32_t iters;            /* CG iterations (maximum over tiles) */
     int32_t tile_width;
-    int32_t engine;           /* 1 multi-CTA grid engine, 2 one-CTA-per-tile, 3 matrix-free driver */
+    int32_t engine;           /* 1 multi-CTA grid engine, 2 one-CTA-per-tile, 3 matrix-free driver,
+                                 4 resident engine (the solve state stays on the SMs) */
     double lambda_min, lambda_max; /* interval enclosing the spectrum used for the nodes */
     double quad_cert;         /* max |f_N(lambda) - log lambda| on [lambda_min, lambda_max] */
     double ms;                /* device time of the solve (CUDA events) */

@@ -140,6 +140,10 @@ struct ld_ctx {
     int ngroups = 0;
     cudaStream_t gstream[kMaxGroups] = {};
     cudaEvent_t gfork = nullptr, gjoin[kMaxGroups] = {};
+    // resident engine (options.engine = 0 on a grid kind): plan per keep_x0, exchange buffers
+    int res_state[2] = {0, 0};    // 0 not planned yet, 1 planned, 2 not applicable
+    ld::ResPlan res_plan[2] = {};
+    DevBuf d_res_rec, d_res_halo;
     int32_t *h_pinned = nullptr;  // remaining, status
     bool have_x0 = false;
     int last_cb = 0, last_ce = 0;
@@ -622,6 +626,8 @@ ld_status matfree_grad(ld_ctx *c, int n_params, const int *ids, double *grad) {
     return LD_OK;
 }
 
+std::mutex g_coop_mu;   // cooperative resident solves of this process
+
 // One probed solve over colours [cb, ce).  On LD_OK, result[0..1] hold
 // sum of terms and sum of seed projections on the device and in *out.
 ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_info *info) {
@@ -659,10 +665,25 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         c->s.keep_x0 = want_x0;
         invalidate_graph(c);
     }
+    std::unique_lock<std::mutex> coop;
+    // the resident engine takes what it has a plan for unless the caller chose an engine or a pass
+    bool resident = false;
+    if (c->opt.engine == 0 && c->opt.lattice_pass == 0 && !ru && c->kind != LD_CSR) {
+        int &state = c->res_state[want_x0];
+        if (state == 0)
+            state = ld::engine_resident_plan(c->s, c->ncolours, keep_x0, c->engine == 1, &c->res_plan[want_x0]) == 0 ? 1 : 2;
+        if (state == 1) {
+            const size_t rb = ld::engine_resident_rec_bytes(c->res_plan[want_x0]);
+            const size_t hb = ld::engine_resident_halo_bytes(c->res_plan[want_x0]);
+            if (rb > c->d_res_rec.bytes) CUDA_TRY(c->d_res_rec.alloc(rb));
+            if (hb > c->d_res_halo.bytes) CUDA_TRY(c->d_res_halo.alloc(hb));
+            resident = true;
+        }
+    }
     // the lean lattice pass (four state words per vertex and column) wherever it applies;
     // the stored-w pass otherwise (FP64, other kinds, the Matern kind with a kept x0)
-    const int want_lean = c->engine == 1 && c->opt.lattice_pass == 0 ? ld::engine_lean_x(c->s, keep_x0) : 0;
-    if (c->s.lean != want_lean || (want_lean && c->lean_plan_x0 != want_x0)) {
+    const int want_lean = c->engine == 1 && c->opt.lattice_pass == 0 && !resident ? ld::engine_lean_x(c->s, keep_x0) : 0;
+    if (!resident && (c->s.lean != want_lean || (want_lean && c->lean_plan_x0 != want_x0))) {
         c->s.lean = want_lean;
         ld::engine_plan(c->s);           // the lean plan's occupancy depends on keep_x0
         c->lean_plan_x0 = want_x0;
@@ -679,11 +700,30 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
     c->solved = false;
     const int max_iter = c->opt.max_iter > 0 ? c->opt.max_iter : 100000;
     CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
-    ENGINE_TRY(ld::engine_init(c->s, cb, ce, c->stream));
-    launches += 3;
     ld_status st = LD_OK;
     double iter_ms = 0.0;
-    if (c->engine == 2) {
+    if (!resident) {
+        ENGINE_TRY(ld::engine_init(c->s, cb, ce, c->stream));
+        launches += 3;
+    }
+    if (resident) {
+        ld::ResArgs ra{};
+        ra.cb = cb;
+        ra.ce = ce;
+        // the iteration cap of the engine this context would otherwise run (whole chunks)
+        ra.cap = c->engine == 2 ? max_iter : (max_iter + c->chunk - 1) / c->chunk * c->chunk;
+        ra.rec = c->d_res_rec.as<ulonglong2>();
+        ra.halo = c->d_res_halo.p;
+        // Teams of a cooperative launch wait on one another, so two such launches must not share
+        // the SMs half each: one at a time in this process, until its results are here.
+        // (A cluster's CTAs are scheduled together: clustered plans need no such rule.)
+        if (!c->res_plan[want_x0].clustered) coop = std::unique_lock<std::mutex>(g_coop_mu);
+        CUDA_TRY(cudaEventRecord(c->ev2, c->stream));
+        ENGINE_TRY(ld::engine_resident(c->s, c->res_plan[want_x0], ra, c->stream));
+        CUDA_TRY(cudaEventRecord(c->ev3, c->stream));
+        launches += 2;
+        CUDA_TRY(cudaMemcpyAsync(c->h_pinned, c->s.remaining, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    } else if (c->engine == 2) {
         CUDA_TRY(cudaEventRecord(c->ev2, c->stream));
         ENGINE_TRY(ld::engine_cta_solve(c->s, max_iter, c->stream));
         CUDA_TRY(cudaEventRecord(c->ev3, c->stream));
@@ -768,12 +808,12 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
             }
         }
     }
-    const int dev_status = c->h_pinned[1];
-    const int remaining = c->h_pinned[0];
     double rel_resid = -1.0;
     if (c->s.keep_x0) {
-        ENGINE_TRY(ld::engine_flush_x(c->s, c->stream));
-        launches += 1;
+        if (!resident) {
+            ENGINE_TRY(ld::engine_flush_x(c->s, c->stream));
+            launches += 1;
+        }
         // true seed residuals (folding x_lo into x_hi first under reliable updates)
         ENGINE_TRY(ld::engine_true_residual(c->s, 0, cb, ce, 0, c->d_norm2.as<double>(), c->stream));
         launches += ru ? 3 : 2;
@@ -787,6 +827,13 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
     CUDA_TRY(cudaMemcpyAsync(it.data(), c->s.col_iters, c->ncols * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     CUDA_TRY(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
+    if (resident) {
+        float e = 0.f;
+        CUDA_TRY(cudaEventElapsedTime(&e, c->ev2, c->ev3));
+        iter_ms = e;
+    }
+    const int dev_status = c->h_pinned[1];
+    const int remaining = c->h_pinned[0];
     for (int v : it) iters = std::max(iters, v);
     int64_t tile_iters = 0;
     for (int t = 0; t < c->ntiles; ++t) {
@@ -810,6 +857,11 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
     if (info) {
         info->reliable_updates = updates;
         info->rel_resid_max = rel_resid;
+        if (resident) {
+            info->engine = 4;
+            info->pass_words = -1;
+            info->bulk_rows = -1;
+        }
     }
     if (st == LD_OK) {
         c->have_x0 = keep_x0;

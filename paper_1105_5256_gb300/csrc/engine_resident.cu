@@ -1,0 +1,242 @@
+// Resident engine, host side: plan (how many CTAs share a probing vector, and how they
+// exchange) and launch.
+#include "engine_resident.cuh"
+
+#include <algorithm>
+
+namespace ld {
+
+namespace {
+
+// items (16 bytes of a line) a thread owns at most: two private vectors in its 128 words of
+// tensor memory, and a 64-bit mask of its own-colour vertices
+constexpr int RES_ITEMS = 16;
+
+template <typename V, int KIND, int NT, bool KX>
+const void *res_fn() {
+    return reinterpret_cast<const void *>(&k_resident<V, KIND, NT, KX>);
+}
+
+template <typename V>
+const void *res_fn_for(int kind, int nt, bool kx) {
+    if (kind == KIND_2D5) return nt == 256 ? res_fn<V, KIND_2D5, 256, false>() : res_fn<V, KIND_2D5, 512, false>();
+    if (kind == KIND_3D7) return nt == 256 ? res_fn<V, KIND_3D7, 256, false>() : res_fn<V, KIND_3D7, 512, false>();
+    if (kx) return nt == 256 ? res_fn<V, KIND_2D13_SQ, 256, true>() : res_fn<V, KIND_2D13_SQ, 512, true>();
+    return nt == 256 ? res_fn<V, KIND_2D13_SQ, 256, false>() : res_fn<V, KIND_2D13_SQ, 512, false>();
+}
+
+const void *res_kernel(const Solve &s, int nt, bool keep_x0) {
+    return s.precision == 0 ? res_fn_for<double>(s.op.kind, nt, keep_x0) : res_fn_for<float>(s.op.kind, nt, keep_x0);
+}
+
+// geometry of a team of M CTAs; false when it does not fit
+bool res_geometry(const Solve &s, bool keep_x0, int nt, int M, bool clustered, ResPlan &p) {
+    const int word = s.precision == 0 ? 8 : 4, E = 16 / word;
+    const bool mat = s.op.kind == KIND_2D13_SQ, d3 = s.op.kind == KIND_3D7;
+    const int H = mat ? 2 : 1;
+    p.M = M;
+    p.nt = nt;
+    p.clustered = clustered;
+    p.G = (s.op.nx + E - 1) / E;
+    if (p.G > nt) return false;
+    p.pitch = (p.G + 2) * E;
+    int best = -1;
+    long best_cost = 0;
+    for (int My = 1; My <= M; ++My) {       // y x z split of a 3D lattice with the fewest lines a CTA
+        if (M % My || (!d3 && My != M)) continue;
+        const int Mz = M / My;
+        if (s.op.ny / My < H || (d3 && s.op.nz / Mz < 1)) continue;
+        const long Ly = (s.op.ny + My - 1) / My, Lz = d3 ? (s.op.nz + Mz - 1) / Mz : 1;
+        const long cost = 4 * Ly * Lz + (d3 ? 2 * (Ly + Lz) : 0);
+        if (best < 0 || cost < best_cost) {
+            best = My;
+            best_cost = cost;
+            p.My = My;
+            p.Ly = (int)Ly;
+            p.Lz = (int)Lz;
+        }
+    }
+    if (best < 0) return false;
+    const int L = p.Ly * p.Lz;
+    p.nseg = std::min(nt / p.G, L);
+    p.cmax = (L + p.nseg - 1) / p.nseg;
+    if (p.cmax > RES_ITEMS) return false;
+    p.slots = 2 * H * p.Lz + (d3 ? 2 * p.Ly : 0);
+    const ResSmem lay = res_smem(p, word, s.op.kind, s.nshift, keep_x0, !mat && s.op.field_d != nullptr);
+    p.smem = lay.bytes;
+    return lay.bytes <= 227 * 1024;
+}
+
+// Clocks of one iteration of a team, from measured parts: a warp's 16-byte item in the
+// vector phases (FP64: its FP64 instructions at 19 clocks each; FP32: issue), and the
+// exchange with the scalar chain (grows with the warps whose partials are summed, and
+// between cooperative CTAs with the records each reads).  Fits the measured iterations of
+// 48 x 40 to 1024 x 1024 and 40^3 to 128^3 lattices within about 20 %.
+double res_clocks(const Solve &s, const ResPlan &p, bool keep_x0) {
+    const bool f64 = s.precision == 0;
+    double item = s.op.kind == KIND_2D13_SQ ? (f64 ? 560 : 80) : s.op.kind == KIND_3D7 ? (f64 ? 470 : 110) : (f64 ? 390 : 62);
+    if (keep_x0) item += f64 ? (s.op.kind == KIND_2D13_SQ ? 120 : 60) : 18;
+    if (s.op.kind != KIND_2D13_SQ && s.op.field_d) item += f64 ? 10 : 15;
+    if (!f64 && p.nt == 256) item *= 1.3;      // half the warps to cover the latencies
+    const double warps = p.nt / 32.0, halo = (double)p.slots * p.G / p.nt;
+    const double active = (p.G * p.nseg + 31) / 32;            // warps that own lines
+    const double work = item * (active * p.cmax + 0.35 * warps * halo);
+    const double fixed = p.clustered ? 5000 + (f64 ? 330 : 170) * warps : (f64 ? 8000 + 330 * warps : 8500 + 60 * warps) + 50.0 * p.M;
+    return work + fixed;
+}
+
+// Clocks of one streamed pass over the same vectors (grid engine): its launches and end of
+// pass, and its state words at the rate measured for the kind (FP32: bytes; FP64: 13 or 18
+// FP64 instructions a vertex and column).
+double stream_clocks(const Solve &s, int ncolours, bool keep_x0) {
+    const double vc = (double)s.op.n * ncolours;
+    const double launch = 15.0 * 1950;
+    if (s.precision == 0) {
+        const double instr = s.op.kind == KIND_2D13_SQ ? 18 : s.op.kind == KIND_3D7 ? 15 : 13;
+        return std::max(launch, vc * (instr + (keep_x0 ? 3 : 0)) / (152 * 1.5));
+    }
+    const int words = (s.op.kind == KIND_2D13_SQ && keep_x0 ? 8 : 4) + (keep_x0 && s.op.kind != KIND_2D13_SQ ? 2 : 0);
+    const double rate = s.op.kind == KIND_3D7 ? 2350 : 3000;    // bytes a clock
+    return 0.5 * launch + vc * words * 4 / rate;
+}
+
+template <class F>
+cudaError_t res_launch(const ResPlan &p, cudaStream_t st, F &&fn) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(p.J * p.M));
+    cfg.blockDim = dim3((unsigned)(p.nt + 64));
+    cfg.dynamicSmemBytes = p.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    if (p.clustered) {
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = (unsigned)p.M;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    } else {
+        at[0].id = cudaLaunchAttributeCooperative;
+        at[0].val.cooperative = 1;
+    }
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return fn(cfg);
+}
+
+}  // namespace
+
+int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, ResPlan *out) {
+    const int k = s.op.kind;
+    if ((k != KIND_2D5 && k != KIND_2D13_SQ && k != KIND_3D7) || s.asig || ncolours < 1) return 1;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return (int)cudaGetLastError();
+    double best = 1e300;
+    for (int nt : {256, 512}) {
+        const void *fn = res_kernel(s, nt, keep_x0);
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess ||
+            cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)
+            return (int)cudaGetLastError();
+        // one cluster a vector
+        for (int M : {1, 2, 3, 4, 6, 8, 10, 12, 16}) {
+            ResPlan p{};
+            if (!res_geometry(s, keep_x0, nt, M, true, p)) continue;
+            p.J = ncolours;
+            int act = 0;
+            cudaError_t e = res_launch(p, nullptr, [&](cudaLaunchConfig_t &cfg) {
+                return cudaOccupancyMaxActiveClusters(&act, fn, &cfg);
+            });
+            if (e != cudaSuccess || act < 1) {
+                cudaGetLastError();
+                continue;
+            }
+            const int rounds = (ncolours + act - 1) / act;
+            const double t = rounds * res_clocks(s, p, keep_x0);
+            if (t < best) {
+                best = t;
+                *out = p;
+            }
+        }
+        // teams over L2, all resident at once (one CTA an SM)
+        for (int J = 1; J <= std::min(ncolours, sms); ++J) {
+            const int rounds = (ncolours + J - 1) / J;
+            if (J > 1 && (ncolours + J - 2) / (J - 1) == rounds) continue;   // fewer teams, as many rounds
+            int M = sms / J;
+            if (k != KIND_3D7) M = std::min(M, s.op.ny / (k == KIND_2D13_SQ ? 2 : 1));
+            ResPlan p{}, q{};
+            bool ok = false;
+            for (int tries = 0; M >= 1 && tries < 24; --M, ++tries) {   // a 3D split wants a composite M
+                if (!res_geometry(s, keep_x0, nt, M, false, q)) {
+                    if (k != KIND_3D7) break;
+                    continue;
+                }
+                q.J = J;
+                if (!ok || res_clocks(s, q, keep_x0) < res_clocks(s, p, keep_x0)) p = q;
+                ok = true;
+                if (k != KIND_3D7) break;
+            }
+            const double t = ok ? rounds * res_clocks(s, p, keep_x0) : 1e300;
+            int occ = 0;
+            if (t < best &&
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, p.nt + 64, p.smem) == cudaSuccess &&
+                (long)occ * sms >= (long)J * p.M) {
+                best = t;
+                *out = p;
+            }
+        }
+    }
+    cudaGetLastError();
+    // contexts the grid engine would run: only where the passes would take longer
+    if (streams && best >= stream_clocks(s, ncolours, keep_x0)) return 1;
+    return best < 1e300 ? 0 : 1;
+}
+
+size_t engine_resident_rec_bytes(const ResPlan &p) {
+    return p.clustered ? 0 : (size_t)p.J * 2 * p.M * 8 * sizeof(ulonglong2);
+}
+size_t engine_resident_halo_bytes(const ResPlan &p) {
+    return p.clustered ? 0 : (size_t)p.J * p.M * 2 * p.slots * p.G * 16;
+}
+
+// state of the columns the engine does not solve, and the counters
+__global__ void k_resident_init(Solve s, int cb, int ce) {
+    __shared__ int cnt;
+    if (threadIdx.x == 0) cnt = 0;
+    __syncthreads();
+    for (int q = threadIdx.x; q < s.ncols * s.nshift; q += blockDim.x) s.pi[q] = make_double2(0.0, 0.0);
+    for (int c = threadIdx.x; c < s.ncols; c += blockDim.x) {
+        s.pi0[c] = 0.0;
+        s.col_iters[c] = 0;
+        s.rho[c] = s.class_size[c];
+        s.col_active[c] = 0;
+        if (c >= cb && c < ce && s.class_size[c] > 0.0) atomicAdd(&cnt, 1);
+    }
+    for (int t = threadIdx.x; t < s.ntiles; t += blockDim.x) {
+        s.tile_done[t] = 1;
+        s.tile_ctr[t] = 0;
+        s.tile_par[t] = 0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        *s.remaining = cnt;
+        *s.status = 0;
+    }
+}
+
+int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    k_resident_init<<<1, 1024, 0, st>>>(s, a.cb, a.ce);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return (int)e;
+    if (a.rec && (e = cudaMemsetAsync(a.rec, 0, engine_resident_rec_bytes(p), st)) != cudaSuccess) return (int)e;
+    const bool kx = s.keep_x0 != 0;
+    const void *fn = res_kernel(s, p.nt, kx);
+    Solve sv = s;
+    ResPlan pv = p;
+    ResArgs av = a;
+    void *args[] = {&sv, &pv, &av};
+    e = res_launch(p, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
+    if (e != cudaSuccess) cudaGetLastError();
+    return (int)e;
+}
+
+}  // namespace ld

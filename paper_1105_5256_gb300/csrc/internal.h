@@ -113,6 +113,31 @@ struct Solve {
     double *result;        // [0] = sum of terms, [1] = sum of seed projections
 };
 
+// Resident engine (engine_resident.cu): the whole solve of a probing vector on chip.
+struct ResPlan {
+    int M, My;            // CTAs of a team; of them along y (the rest along z)
+    int J;                // teams: team j solves columns j, j + J, ...
+    int clustered;        // a team is one thread-block cluster; else a cooperative launch
+    int nt;               // vector threads of a CTA
+    int G, nseg, cmax;    // 16-byte groups of a line; line segments; lines a thread owns at most
+    int pitch;            // shared-memory line pitch (elements)
+    int Ly, Lz;           // lines of a CTA at most
+    int slots;            // halo lines of a CTA at most
+    size_t smem;
+};
+struct ResArgs {
+    int cb, ce;           // colour range
+    int cap;              // iterations at most
+    ulonglong2 *rec;      // cooperative teams: partial-sum records [J][2][M][8]
+    void *halo;           // cooperative teams: boundary rows [J][M][2][slots][G]
+};
+// 0 and a plan when the engine takes the solve; nonzero otherwise.  streams: the context
+// would otherwise run the grid engine, so the plan must beat its passes
+int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, ResPlan *out);
+size_t engine_resident_rec_bytes(const ResPlan &p);
+size_t engine_resident_halo_bytes(const ResPlan &p);
+int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *stream);
+
 // dot products per column reduced each pass: r.r, p.w, r.w, w.w, v.r, v.w
 constexpr int NDOT = 6;
 

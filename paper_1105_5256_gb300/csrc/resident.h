@@ -1,0 +1,57 @@
+// Plan and shared-memory layout of the resident engine, common to its kernel
+// (engine_resident.cuh) and its host side (engine_resident.cu).
+#pragma once
+#include <cstddef>
+#include <cstdint>
+
+#include "internal.h"
+
+namespace ld {
+
+constexpr int RES_CTL_BYTES = 288;
+
+// bytes of one CTA's shared memory by purpose (offsets from the dynamic base)
+struct ResSmem {
+    size_t part, bc, shift, a, b, rh, hb, x, d, bytes;
+    size_t zero_bytes;      // from `a`: what a new column starts from zero
+    bool x_tm, d_tm;        // x, diagonal in tensor memory (else in shared memory)
+};
+
+__host__ __device__ inline ResSmem res_smem(const ResPlan &p, int word, int kind, int nshift, int keepx, bool field) {
+    const bool mat = kind == KIND_2D13_SQ, d3 = kind == KIND_3D7;
+    const int E = 16 / word, H = mat ? 2 : 1, NW = p.nt / 32;
+    const size_t ge = (size_t)p.G * E * word, pitch = (size_t)p.pitch * word;
+    const size_t np = p.clustered ? (size_t)NW * p.M : NW;
+    const size_t priv = (size_t)p.cmax * p.nt * 16;
+    ResSmem s;
+    // private vectors in tensor memory, 128 words a thread: w; r or (Matern with x) p; then
+    // x and the diagonal while they fit
+    int room = 32 - p.cmax * (mat && !keepx ? 1 : 2);
+    s.x_tm = keepx && room >= p.cmax;
+    if (s.x_tm) room -= p.cmax;
+    s.d_tm = field && room >= p.cmax;
+    size_t o = 0;
+    s.part = o;
+    o += (2 * 5 * np * 8 + 15) / 16 * 16;
+    s.bc = o;
+    o += RES_CTL_BYTES;
+    s.shift = o;
+    o += ((size_t)nshift * 65 + 15) / 16 * 16;
+    s.a = o;
+    o += (size_t)(d3 ? (p.Ly + 2) * (p.Lz + 2) : p.Ly + 2 * H) * pitch;
+    s.b = o;
+    if (mat) o += (size_t)(p.Ly + 2) * pitch;
+    s.rh = o;
+    if (!mat) o += (size_t)p.slots * ge;
+    s.x = o;
+    if (keepx && !s.x_tm) o += priv;
+    s.zero_bytes = o - s.a;
+    s.hb = o;
+    if (p.clustered) o += 2 * (size_t)p.slots * ge;
+    s.d = o;
+    if (field && !s.d_tm) o += priv;
+    s.bytes = o;
+    return s;
+}
+
+}  // namespace ld

@@ -1,0 +1,104 @@
+"""GPU parity of the resident engine (options.engine = 0 on grid kinds: a probing vector's
+whole solve on chip, info engine 4) with the streaming grid engine on the same problem,
+over geometries where its blocks, teams and exchanges can go wrong: lines that are no
+multiple of 16 bytes, one line or one group a CTA, torus wraps onto the same CTA, teams of
+one to sixteen CTAs in a cluster and cooperative teams over L2, blocks of a 3D lattice with
+uneven sides, kappa^2 fields and masks, the kept seed solution, more shifts than lanes.
+
+Both engines run the same recurrences to the same stopping rule (each shifted residual
+<= tol), so terms and seed projections differ by rounding and by at most an iteration at
+the stop: FP64 to 50 tol relative, FP32 vectors to 2e-5 (the bounds of the other parity
+tests); seed solutions enter the gradient linearly, at the same bounds.
+"""
+import numpy as np
+import pytest
+
+import paper_1105_5256_gb300 as L
+import synth
+
+pytestmark = pytest.mark.gpu
+
+K = {5: L.LD_STENCIL_2D5, 13: L.LD_STENCIL_2D13_SQ, 7: L.LD_STENCIL_3D7}
+CASES = [
+    # points, dims, periodic, kappa2, distance, form, gradient ids, shifts
+    (5, (1, 40), False, 0.5, 2, "", (), 16),               # one column of vertices
+    (5, (5, 3), True, 0.5, 1, "mask", (0, 1), 16),         # wraps within one CTA, partial item
+    (13, (6, 5), True, 0.5, 1, "", (2,), 16),              # two halo lines that wrap onto own lines
+    (13, (33, 7), False, 0.4, 1, "", (), 40),              # more shifts than a warp has lanes
+    (5, (127, 61), False, 0.3, 2, "field", (0, 2), 20),
+    (13, (126, 61), True, 0.3, 1, "", (0, 2), 20),         # torus ghosts in a partial item
+    (13, (130, 90), False, 0.2, 2, "", (), 20),
+    (5, (400, 260), True, 0.3, 4, "mask", (1,), 20),       # several CTAs a vector, mask bits
+    (5, (1030, 12), False, 0.4, 2, "field", (0,), 20),     # wide lines: 258 groups of four
+    (13, (301, 203), False, 0.3, 2, "", (0, 2), 20),
+    (7, (9, 8, 7), True, 0.4, 2, "field", (0,), 20),
+    (7, (21, 20, 19), False, 0.4, 2, "mask", (1, 2), 20),
+    (7, (40, 33, 35), False, 0.4, 2, "", (), 20),
+]
+
+
+def build(case, prec, engine, col, tol, **kw):
+    points, dims, per, k2, d, form, _, shifts = case
+    n = int(np.prod(dims))
+    field = synth.kappa2_field(7, dims) if form == "field" else None
+    mask = synth.obs_mask(8, n, 0.2) if form == "mask" else None
+    m = L.grid_matrix(K[points], dims, 1.0 if form == "field" else k2, periodic=per, kappa2_field=field,
+                      tau=3.0 if form == "mask" else 0.0, obs_mask=mask, scale=1.7)
+    return L.ld_create(m, d, shifts, tol, L.options(precision=prec, engine=engine, colouring=col, **kw))
+
+
+def evaluate(ctx, ids):
+    if ids:
+        v, g, info = L.ld_logdet_grad(ctx, list(ids))
+    else:
+        (v, info), g = L.ld_logdet(ctx), np.zeros(0)
+    return v, g, info, *L.ld_column_terms(ctx)
+
+
+@pytest.mark.parametrize("prec", [L.LD_FP64, L.LD_MIXED])
+@pytest.mark.parametrize("case", CASES, ids=lambda c: "%d-%s%s%s" % (c[0], "x".join(map(str, c[1])), "t" if c[2] else "", c[5]))
+def test_resident_matches_streaming_engine(case, prec):
+    points, dims, per, k2, d, form, ids, shifts = case
+    tol = 1e-9 if prec == L.LD_FP64 else 1e-6
+    col, _ = L.ld_colour_grid(K[points], dims, per, d)
+    ref = evaluate(build(case, prec, 1, col, tol, tile_width=2), ids)
+    ctx = build(case, prec, 0, col, tol, tile_width=2)
+    got = evaluate(ctx, ids)
+    # FP64 lattices large enough to keep every SM's FP64 units busy either way may stream
+    assert ref[2]["engine"] == 1 and (got[2]["engine"] == 4 or (prec == L.LD_FP64 and np.prod(dims) > 12000))
+    bar = 50 * tol if prec == L.LD_FP64 else 2e-5
+    for k in (3, 4):                                       # per-colour terms, seed projections
+        err = np.linalg.norm(got[k] - ref[k]) / np.linalg.norm(ref[k])
+        assert err <= bar, (k, err)
+    assert abs(got[0] - ref[0]) <= bar * np.abs(ref[3]).sum()
+    assert np.allclose(got[1], ref[1], rtol=bar, atol=0)
+    assert abs(got[2]["iters"] - ref[2]["iters"]) <= max(3, ref[2]["iters"] // 10)
+    if ids and prec == L.LD_FP64:                          # (in FP32 both are rounding, eps x condition)
+        assert 0 <= got[2]["rel_resid_max"] <= 2 * max(tol, ref[2]["rel_resid_max"])
+    again = evaluate(ctx, ids)                             # the same bits on every call
+    assert again[0] == got[0] and np.array_equal(again[3], got[3]) and np.array_equal(again[1], got[1])
+
+
+def test_partial_colour_ranges_keep_each_column():
+    case = (13, (130, 90), False, 0.2, 2, "", (), 20)
+    col, nc = L.ld_colour_grid(K[13], case[1], False, 2)
+    ctx = build(case, L.LD_FP64, 0, col, 1e-8)
+    whole, info = L.ld_logdet(ctx)
+    assert info["engine"] == 4
+    terms, _ = L.ld_column_terms(ctx)
+    parts = [L.ld_logdet_partial(ctx, a, b)[0] for a, b in ((0, 5), (5, 5), (5, nc))]
+    assert parts[1] == 0.0 and abs(sum(parts) - whole) <= 1e-13 * np.abs(terms).sum()
+
+
+def test_iteration_cap_and_new_parameters():
+    case = (5, (127, 61), False, 1e-4, 2, "", (), 20)
+    col, _ = L.ld_colour_grid(K[5], case[1], False, 2)
+    ctx = build(case, L.LD_FP64, 0, col, 1e-10, max_iter=20)
+    with pytest.raises(L.LogDetError) as e:
+        L.ld_logdet(ctx)
+    assert e.value.status == L.LD_ENOTCONV
+    L.ld_set_params(ctx, 50.0, 0.0, 1.7)                   # well conditioned: converges within the cap
+    v, info = L.ld_logdet(ctx)
+    other = build((5, (127, 61), False, 50.0, 2, "", (), 20), L.LD_FP64, 1, col, 1e-10)
+    w, _ = L.ld_logdet(other)
+    assert info["engine"] == 4 and abs(v - w) <= 50e-10 * abs(w)
