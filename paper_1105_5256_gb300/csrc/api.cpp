@@ -718,6 +718,8 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         // the SMs half each: one at a time in this process, until its results are here.
         // (A cluster's CTAs are scheduled together: clustered plans need no such rule.)
         if (!c->res_plan[want_x0].clustered) coop = std::unique_lock<std::mutex>(g_coop_mu);
+        // the engine writes the seed solutions of the colours it solves; the others' are zero
+        if (keep_x0 && (cb > 0 || ce < c->ncolours)) CUDA_TRY(cudaMemsetAsync(c->d_x.p, 0, c->d_x.bytes, c->stream));
         CUDA_TRY(cudaEventRecord(c->ev2, c->stream));
         ENGINE_TRY(ld::engine_resident(c->s, c->res_plan[want_x0], ra, c->stream));
         CUDA_TRY(cudaEventRecord(c->ev3, c->stream));

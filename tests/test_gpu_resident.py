@@ -90,6 +90,19 @@ def test_partial_colour_ranges_keep_each_column():
     assert parts[1] == 0.0 and abs(sum(parts) - whole) <= 1e-13 * np.abs(terms).sum()
 
 
+def test_partial_ranges_leave_zero_seed_solutions_elsewhere():
+    """ld_grad after a partial solve sums over the colours of the range alone."""
+    case = (5, (127, 61), False, 0.3, 2, "mask", (), 20)
+    col, nc = L.ld_colour_grid(K[5], case[1], False, 2)
+    grads = []
+    for engine in (1, 0):
+        ctx = build(case, L.LD_FP64, engine, col, 1e-10, keep_x0=1)
+        L.ld_logdet(ctx)                                   # every colour's x on the device
+        L.ld_logdet_partial(ctx, 2, nc - 1)
+        grads.append(L.ld_grad(ctx, [L.LD_P_TAU, L.LD_P_SCALE]))
+    assert np.allclose(grads[0], grads[1], rtol=50e-10, atol=0)
+
+
 def test_iteration_cap_and_new_parameters():
     case = (5, (127, 61), False, 1e-4, 2, "", (), 20)
     col, _ = L.ld_colour_grid(K[5], case[1], False, 2)
