@@ -331,6 +331,8 @@ ld_status set_nodes(ld_ctx *c) {
             c->nshift = N;
             c->s.nshift = N;
             invalidate_graph(c);
+            // a resident plan's shared memory holds the shift state: plan again
+            if (c->kind != LD_CSR) c->res_state[0] = c->res_state[1] = 0;
         }
         if (N > c->nshift_cap)
             if (ld_status st = bind_shift_state(c, std::max(N, 2 * c->nshift_cap))) return st;
