@@ -144,6 +144,8 @@ struct ld_ctx {
     int res_state[2] = {0, 0};    // 0 not planned yet, 1 planned, 2 not applicable
     ld::ResPlan res_plan[2] = {};
     DevBuf d_res_rec, d_res_halo;
+    ld::CsrPlan csr_plan{};       // CSR contexts: laid out at creation (res_state 1) or absent (2)
+    DevBuf d_csr_row0, d_csr_ext0, d_csr_ext, d_csr_lcol;
     int32_t *h_pinned = nullptr;  // remaining, status
     bool have_x0 = false;
     int last_cb = 0, last_ce = 0;
@@ -670,7 +672,14 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
     std::unique_lock<std::mutex> coop;
     // the resident engine takes what it has a plan for unless the caller chose an engine or a pass
     bool resident = false;
-    if (c->opt.engine == 0 && c->opt.lattice_pass == 0 && !ru && c->kind != LD_CSR) {
+    if (c->kind == LD_CSR) {
+        if (c->res_state[0] == 1 && c->nshift <= (c->auto_shift ? 64 : c->nshift)) {
+            const size_t hb = (size_t)c->csr_plan.J * 2 * c->n * c->csr_plan.T * (c->opt.precision == LD_FP64 ? 8 : 4);
+            if (!c->d_res_rec.p) CUDA_TRY(c->d_res_rec.alloc(ld::engine_csr_rec_bytes(c->csr_plan)));
+            if (!c->d_res_halo.p) CUDA_TRY(c->d_res_halo.alloc(hb));
+            resident = true;
+        }
+    } else if (c->opt.engine == 0 && c->opt.lattice_pass == 0 && !ru) {
         int &state = c->res_state[want_x0];
         if (state == 0)
             state = ld::engine_resident_plan(c->s, c->ncolours, keep_x0, c->engine == 1, &c->res_plan[want_x0]) == 0 ? 1 : 2;
@@ -719,11 +728,12 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         // Teams of a cooperative launch wait on one another, so two such launches must not share
         // the SMs half each: one at a time in this process, until its results are here.
         // (A cluster's CTAs are scheduled together: clustered plans need no such rule.)
-        if (!c->res_plan[want_x0].clustered) coop = std::unique_lock<std::mutex>(g_coop_mu);
+        if (c->kind == LD_CSR || !c->res_plan[want_x0].clustered) coop = std::unique_lock<std::mutex>(g_coop_mu);
         // the engine writes the seed solutions of the colours it solves; the others' are zero
         if (keep_x0 && (cb > 0 || ce < c->ncolours)) CUDA_TRY(cudaMemsetAsync(c->d_x.p, 0, c->d_x.bytes, c->stream));
         CUDA_TRY(cudaEventRecord(c->ev2, c->stream));
-        ENGINE_TRY(ld::engine_resident(c->s, c->res_plan[want_x0], ra, c->stream));
+        if (c->kind == LD_CSR) ENGINE_TRY(ld::engine_resident_csr(c->s, c->csr_plan, ra, c->stream));
+        else ENGINE_TRY(ld::engine_resident(c->s, c->res_plan[want_x0], ra, c->stream));
         CUDA_TRY(cudaEventRecord(c->ev3, c->stream));
         launches += 2;
         CUDA_TRY(cudaMemcpyAsync(c->h_pinned, c->s.remaining, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
@@ -1184,6 +1194,28 @@ ld_status ld_create(const ld_matrix *Q, int colouring_distance, int n_shifts, do
         if (f32) {
             CUDA_TRY(c->d_val_f.alloc(std::max<int64_t>(nnz, 1) * sizeof(float)));
             CUDA_TRY(cudaMemcpy(c->d_val_f.p, vf.data(), nnz * sizeof(float), cudaMemcpyHostToDevice));
+        }
+    }
+    if (c->kind == LD_CSR && opt.engine == 0 && opt.reliable_delta == 0.0) {
+        // the resident engine's row split and local column numbers
+        std::vector<int32_t> row0, ext0, ext;
+        std::vector<uint16_t> lcol;
+        const bool fits = ld::engine_csr_plan(c->n, Q->rowptr, Q->colidx, f32 ? 1 : 0, c->ncolours,
+                                              c->auto_shift ? 64 : c->nshift, &c->csr_plan, row0, ext0, ext, lcol) == 0;
+        c->res_state[0] = c->res_state[1] = fits ? 1 : 2;
+        if (fits) {
+            auto put = [](DevBuf &d, const void *src, size_t bytes) {
+                cudaError_t e = d.alloc(std::max<size_t>(bytes, 16));
+                return e != cudaSuccess || bytes == 0 ? e : cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice);
+            };
+            CUDA_TRY(put(c->d_csr_row0, row0.data(), row0.size() * 4));
+            CUDA_TRY(put(c->d_csr_ext0, ext0.data(), ext0.size() * 4));
+            CUDA_TRY(put(c->d_csr_ext, ext.data(), ext.size() * 4));
+            CUDA_TRY(put(c->d_csr_lcol, lcol.data(), lcol.size() * 2));
+            c->csr_plan.row0 = c->d_csr_row0.as<int32_t>();
+            c->csr_plan.ext0 = c->d_csr_ext0.as<int32_t>();
+            c->csr_plan.ext = c->d_csr_ext.as<int32_t>();
+            c->csr_plan.lcol = c->d_csr_lcol.as<uint16_t>();
         }
     }
     // work buffers

@@ -222,9 +222,13 @@ __global__ void k_resident_init(Solve s, int cb, int ce) {
     }
 }
 
+void resident_init(const Solve &s, int cb, int ce, cudaStream_t st) {
+    k_resident_init<<<1, 1024, 0, st>>>(s, cb, ce);
+}
+
 int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *stream) {
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    k_resident_init<<<1, 1024, 0, st>>>(s, a.cb, a.ce);
+    resident_init(s, a.cb, a.ce, st);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return (int)e;
     if (a.rec && (e = cudaMemsetAsync(a.rec, 0, engine_resident_rec_bytes(p), st)) != cudaSuccess) return (int)e;
@@ -233,8 +237,9 @@ int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *st
     Solve sv = s;
     ResPlan pv = p;
     ResArgs av = a;
+    pv.smem = res_smem(p, s.precision == 0 ? 8 : 4, s.op.kind, s.nshift, kx, s.op.kind != KIND_2D13_SQ && s.op.field_d).bytes;
     void *args[] = {&sv, &pv, &av};
-    e = res_launch(p, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
+    e = res_launch(pv, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
 }

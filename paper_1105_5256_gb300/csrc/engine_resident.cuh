@@ -415,8 +415,10 @@ struct ResBlock {
 };
 
 // ------------------------------------------------------------------ shift warp
-__device__ __noinline__ void res_shift_role(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team,
-                                            ResCtl *ctl, double2 *shm) {
+// columns first, first + stride, ...
+static __device__ __noinline__ void res_shift_role(const Solve &s, int stride, int first, const ResArgs &ar,
+                                                   ResCtl::Entry *queue, volatile int *head, volatile int *tail_out,
+                                                   volatile int *done_out, double2 *shm) {
     const int lane = threadIdx.x & 31;
     ResShift sh;
     sh.z = shm;
@@ -425,7 +427,7 @@ __device__ __noinline__ void res_shift_role(const Solve &s, const ResPlan &pl, c
     sh.phi = sh.pi + s.nshift;
     sh.act = reinterpret_cast<uint8_t *>(sh.phi + s.nshift);
     int tail = 0;
-    for (int c = ar.cb + team; c < ar.ce; c += pl.J) {
+    for (int c = first; c < ar.ce; c += stride) {
         const double vv = s.class_size[c];
         if (!(vv > 0.0)) continue;
         for (int l = lane; l < s.nshift; l += 32) {
@@ -440,13 +442,13 @@ __device__ __noinline__ void res_shift_role(const Solve &s, const ResPlan &pl, c
         int iters = 0;
         bool done = false;
         for (;;) {
-            while (ctl->head == tail) __nanosleep(20);     // the scalar warp always posts an end
+            while (*head == tail) __nanosleep(20);     // the scalar warp always posts an end
             __threadfence_block();
-            const ResCtl::Entry e = ctl->q[tail & 3];
+            const ResCtl::Entry e = queue[tail & 3];
             if (e.code < 0) {
                 __syncwarp();
                 ++tail;
-                if (lane == 0) ctl->tail = tail;
+                if (lane == 0) *tail_out = tail;
                 if (e.code == -2) return;                // a wait ran out
                 break;
             }
@@ -471,12 +473,12 @@ __device__ __noinline__ void res_shift_role(const Solve &s, const ResPlan &pl, c
                     }
                     if (done && lane == 0) s.rho[c] = e.rho;
                 }
-                if (done && lane == 0) ctl->done = tail + 1;
+                if (done && lane == 0) *done_out = tail + 1;
             }
             __threadfence_block();
             __syncwarp();
             ++tail;
-            if (lane == 0) ctl->tail = tail;
+            if (lane == 0) *tail_out = tail;
         }
         for (int l = lane; l < s.nshift; l += 32) s.pi[(size_t)c * s.nshift + l] = sh.pi[l];
         if (lane == 0) {
@@ -1168,7 +1170,8 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__
     else if (wid == NW)
         res_scalar_role<NT>(s, pl, ar, team, m, ctl, reinterpret_cast<const double *>(smem + lay.part), NP, in_bytes);
     else if (m == 0)
-        res_shift_role(s, pl, ar, team, ctl, reinterpret_cast<double2 *>(smem + lay.shift));
+        res_shift_role(s, pl.J, ar.cb + team, ar, ctl->q, &ctl->head, &ctl->tail, &ctl->done,
+                       reinterpret_cast<double2 *>(smem + lay.shift));
     __syncwarp();
     __syncthreads();
     if (pl.clustered) cluster_sync_all();          // no CTA leaves while another may still store to it

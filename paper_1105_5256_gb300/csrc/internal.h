@@ -138,6 +138,28 @@ size_t engine_resident_rec_bytes(const ResPlan &p);
 size_t engine_resident_halo_bytes(const ResPlan &p);
 int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *stream);
 
+// Resident engine for CSR matrices (engine_resident_csr.cu): cooperative teams of M CTAs, T
+// probing vectors a team, a row range with its matrix part a CTA.
+struct CsrPlan {
+    int M, J, T;                   // CTAs of a team, teams, vectors of a team
+    int nt;                        // vector threads of a CTA
+    int own_max, ext_max, nnz_max; // rows, external columns, matrix entries of a CTA at most
+    int items_own, items_ext;      // of them per thread
+    size_t rec_team;               // records of a team
+    size_t smem;
+    int split, T2;                 // colours from `split` on run T2 at a time (0: none)
+    // device: first row / first external column of each CTA (M + 1), the external columns,
+    // and every matrix entry's local column
+    const int32_t *row0, *ext0, *ext;
+    const uint16_t *lcol;
+};
+// host layout of a CSR plan (engine_resident_csr.cu): 0 when one fits
+int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int ncolours, int nshift,
+                    CsrPlan *out, std::vector<int32_t> &row0, std::vector<int32_t> &ext0, std::vector<int32_t> &ext,
+                    std::vector<uint16_t> &lcol);
+size_t engine_csr_rec_bytes(const CsrPlan &p);
+int engine_resident_csr(const Solve &s, const CsrPlan &p, const ResArgs &a, void *stream);
+
 // dot products per column reduced each pass: r.r, p.w, r.w, w.w, v.r, v.w
 constexpr int NDOT = 6;
 

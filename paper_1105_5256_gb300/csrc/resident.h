@@ -54,4 +54,38 @@ __host__ __device__ inline ResSmem res_smem(const ResPlan &p, int word, int kind
     return s;
 }
 
+// ---- CSR (engine_resident_csr.cuh)
+constexpr int RES_CSR_T = 16;            // vectors of a team at most
+constexpr int RES_CSR_CTL_BYTES = 24 + 4 * 40 + 16 * RES_CSR_T + 8;
+
+struct CsrSmem {
+    size_t part, ctl, shift, val, col, row, colour, coef, p, bytes;
+};
+
+__host__ __device__ inline CsrSmem csr_smem(const CsrPlan &p, int word, int nshift) {
+    const size_t a16 = 15;
+    CsrSmem s;
+    size_t o = 0;
+    s.p = o;
+    o += (size_t)(p.own_max + p.ext_max) * p.T * word;
+    s.part = o;
+    o += (size_t)2 * 5 * p.T * (p.nt / 32) * 8;
+    s.ctl = o;
+    o += (RES_CSR_CTL_BYTES + a16) / 16 * 16;
+    s.shift = o;
+    o += ((size_t)nshift * 65 + a16) / 16 * 16;
+    s.coef = o;
+    o += (size_t)3 * p.T * word;
+    s.val = o;
+    o += ((size_t)p.nnz_max * word + a16) / 16 * 16;
+    s.col = o;
+    o += ((size_t)p.nnz_max * 2 + a16) / 16 * 16;
+    s.row = o;
+    o += ((size_t)(p.own_max + 1) * 4 + a16) / 16 * 16;
+    s.colour = o;
+    o += ((size_t)p.own_max * 4 + a16) / 16 * 16;
+    s.bytes = o;
+    return s;
+}
+
 }  // namespace ld

@@ -115,3 +115,58 @@ def test_iteration_cap_and_new_parameters():
     other = build((5, (127, 61), False, 50.0, 2, "", (), 20), L.LD_FP64, 1, col, 1e-10)
     w, _ = L.ld_logdet(other)
     assert info["engine"] == 4 and abs(v - w) <= 50e-10 * abs(w)
+
+
+# ------------------------------------------------------------------ CSR
+def csr_problem(name):
+    if name.startswith("mesh"):                            # mesh<alpha>-<nx>x<ny>
+        alpha, size = name[4:].split("-")
+        nx, ny = map(int, size.split("x"))
+        p, t = synth.perturbed_triangulation(6, nx, ny)
+        from paper_1105_5256_gb300 import mesh
+        rp, ci, vv = mesh.spde_csr(p, t, 0.3 * (nx - 1) * (ny - 1), int(alpha), 1.0)
+    else:
+        n = int(name[4:])
+        rp, ci, vv = synth.csr_from_edges(n, *synth.random_sparse_spd_pattern(9, n), 0.3)
+    lo, hi, _ = *L.ld_csr_bounds(rp, ci, vv), None
+    return rp, ci, vv, lo, hi
+
+
+@pytest.mark.parametrize("prec", [L.LD_FP64, L.LD_MIXED])
+@pytest.mark.parametrize("name,shifts", [
+    ("rand9", 16),                # fewer rows than a warp, one or two a CTA
+    ("rand333", 40),              # more shifts than lanes
+    ("rand3001", 20),
+    ("mesh1-31x27", 20),
+    ("mesh2-40x33", 20),          # long rows, external columns on both sides
+    ("mesh2-141x97", 20),         # several vectors a team and a remainder
+])
+def test_resident_csr_matches_streaming_engine(name, shifts, prec):
+    rp, ci, vv, lo, hi = csr_problem(name)
+    tol = 1e-9 if prec == L.LD_FP64 else 1e-6
+    out = []
+    for engine in (1, 0):
+        ctx = L.ld_create(L.csr_matrix(rp, ci, vv, scale=1.3), 2, shifts, tol,
+                          L.options(precision=prec, engine=engine, lambda_min=1.3 * lo, lambda_max=1.3 * hi, tile_width=2))
+        out.append((ctx, evaluate(ctx, (L.LD_P_SCALE,))))
+    ref, got = out[0][1], out[1][1]
+    assert ref[2]["engine"] == 1 and got[2]["engine"] == 4
+    bar = 50 * tol if prec == L.LD_FP64 else 2e-5
+    for k in (3, 4):
+        assert np.linalg.norm(got[k] - ref[k]) <= bar * np.linalg.norm(ref[k])
+    assert np.allclose(got[1], ref[1], rtol=bar, atol=0)
+    ctx = out[1][0]
+    again = evaluate(ctx, (L.LD_P_SCALE,))
+    assert again[0] == got[0] and np.array_equal(again[3], got[3]) and np.array_equal(again[1], got[1])
+    nc = len(got[3])                                       # each column alike in any range
+    split = [L.ld_logdet_partial(ctx, a, b)[0] for a, b in ((0, nc // 3), (nc // 3, nc))]
+    assert abs(sum(split) - got[0]) <= 1e-13 * np.abs(got[3]).sum()
+
+
+def test_resident_csr_reports_not_spd():
+    n = 600
+    rp, ci, vv = synth.csr_from_edges(n, *synth.random_sparse_spd_pattern(9, n), 0.3)
+    ctx = L.ld_create(L.csr_matrix(rp, ci, -vv), 1, 16, 1e-8, L.options(lambda_min=0.1, lambda_max=50.0))
+    with pytest.raises(L.LogDetError) as e:
+        L.ld_logdet(ctx)
+    assert e.value.status == L.LD_ENOTSPD
