@@ -284,7 +284,8 @@ ld_status ld_apply(ld_ctx *ctx, int ncols, const double *x, double *y);
  * plus one complex search direction per shift, accumulating y directly.  V, Y host arrays,
  * row-major n x ncols, FP64 (the vectors run in the context's precision).  Uses the
  * context's operator, nodes and tolerance; needs about (6 w + 16 N + 8) n ncols bytes of
- * device memory for the call (a matrix-free context: the caller's product, FP64 vectors,
+ * device memory for the call, at least 64 MB where the solve runs on chip (engine option 0 on
+ * a grid kind; up to 256 MB of it stays with the context) (a matrix-free context: the caller's product, FP64 vectors,
  * (16 N + 40) n ncols bytes).  Errors as ld_logdet. */
 ld_status ld_logmv(ld_ctx *ctx, int ncols, const double *V, double *Y, ld_info *info);
 

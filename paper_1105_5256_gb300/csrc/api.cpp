@@ -146,6 +146,10 @@ struct ld_ctx {
     DevBuf d_res_rec, d_res_halo;
     ld::CsrPlan csr_plan{};       // CSR contexts: laid out at creation (res_state 1) or absent (2)
     DevBuf d_csr_row0, d_csr_ext0, d_csr_ext, d_csr_lcol;
+    DevBuf d_vec;                 // vector form on chip: one workspace, kept while it is small
+    ld::ResPlan vec_plan{};       // its plan for vec_ncols columns and vec_nshift nodes (0: none yet)
+    int vec_ncols = 0, vec_nshift = 0;
+    bool vec_fits = false;
     int32_t *h_pinned = nullptr;  // remaining, status
     bool have_x0 = false;
     int last_cb = 0, last_ce = 0;
@@ -1544,6 +1548,127 @@ ld_status ld_apply(ld_ctx *c, int ncols, const double *x, double *y) {
     return LD_OK;
 }
 
+// Vector form on chip (see engine_resident_funmv): false in *taken leaves the call to the
+// streaming form (no plan, or more iterations than the records hold).
+static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y, ld_info *info,
+                                const double2 *weight_dev, bool *taken) {
+    *taken = false;
+    if (c->opt.engine != 0 || c->opt.lattice_pass != 0 || c->kind == LD_CSR) return LD_OK;
+    const int N = c->nshift;
+    const int64_t n = c->n;
+    Solve s = c->s;
+    s.T = 1;
+    s.ntiles = s.ncols = ncols;
+    s.keep_x0 = 0;
+    s.x = nullptr;
+    s.xhi = nullptr;
+    s.weight = weight_dev;
+    if (c->vec_ncols != ncols || c->vec_nshift != N) {
+        c->vec_fits = ld::engine_resident_plan_vec(s, ncols, &c->vec_plan) == 0;
+        c->vec_ncols = ncols;
+        c->vec_nshift = N;
+    }
+    if (!c->vec_fits) return LD_OK;
+    const ld::ResPlan &plan = c->vec_plan;
+    const int max_iter = c->opt.max_iter > 0 ? c->opt.max_iter : 100000;
+    // records of every iteration's shift scalars: within the streaming form's shifted directions
+    const size_t per_iter = (size_t)ncols * N * 3 * sizeof(double2);
+    const size_t budget = std::max<size_t>((size_t)16 * N * n * ncols, (size_t)64 << 20);
+    const int hcap = (int)std::min<size_t>(budget / per_iter, (size_t)max_iter);
+    if (hcap < 1) return LD_OK;
+    // one workspace
+    size_t off = 0;
+    auto take = [&off](size_t bytes) {
+        const size_t o = off;
+        off += (bytes + 255) / 256 * 256;
+        return o;
+    };
+    const size_t C = ncols;
+    const size_t o_rhs = take((size_t)n * C * 8), o_y = take((size_t)n * C * 8), o_hist = take(per_iter * hcap);
+    const size_t o_ab = take(C * hcap * sizeof(double2)), o_coef = take(C * hcap * 8), o_pi = take(C * N * sizeof(double2));
+    const size_t o_sc = take(3 * C * 8), o_int = take((2 * C + 3 * C + 2) * 4);
+    const size_t o_rec = take(ld::engine_resident_rec_bytes(plan)), o_halo = take(ld::engine_resident_halo_bytes(plan));
+    if (c->d_vec.bytes < off && c->d_vec.alloc(off) != cudaSuccess) {
+        cudaGetLastError();
+        return LD_OK;
+    }
+    unsigned char *w = c->d_vec.as<unsigned char>();
+    s.pi = reinterpret_cast<double2 *>(w + o_pi);
+    double *sc = reinterpret_cast<double *>(w + o_sc);
+    s.rho = sc;
+    s.pi0 = sc + C;
+    s.class_size = sc + 2 * C;
+    int32_t *ii = reinterpret_cast<int32_t *>(w + o_int);
+    s.col_iters = ii;
+    s.col_active = ii + C;
+    s.tile_done = ii + 2 * C;
+    s.tile_ctr = ii + 3 * C;
+    s.tile_par = ii + 4 * C;
+    s.remaining = ii + 5 * C;
+    s.status = s.remaining + 1;
+    std::vector<double> norm2(C, 0.0);
+    for (int64_t i = 0; i < n; ++i)
+        for (size_t k = 0; k < C; ++k) norm2[k] += V[i * C + k] * V[i * C + k];
+    ld::ResArgs ra{};
+    ra.cb = 0;
+    ra.ce = ncols;
+    ra.cap = max_iter;
+    ra.rec = plan.clustered ? nullptr : reinterpret_cast<ulonglong2 *>(w + o_rec);
+    ra.halo = w + o_halo;
+    ra.rhs = reinterpret_cast<double *>(w + o_rhs);
+    ra.y = reinterpret_cast<double *>(w + o_y);
+    ra.ld = ncols;
+    ra.hcap = hcap;
+    ra.hist = reinterpret_cast<double2 *>(w + o_hist);
+    ra.ab = reinterpret_cast<double2 *>(w + o_ab);
+    ra.coef = reinterpret_cast<double *>(w + o_coef);
+    std::unique_lock<std::mutex> coop;
+    if (!plan.clustered) coop = std::unique_lock<std::mutex>(g_coop_mu);
+    CUDA_TRY(cudaMemcpyAsync(const_cast<double *>(s.class_size), norm2.data(), C * 8, cudaMemcpyHostToDevice, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(w + o_rhs, V, (size_t)n * C * 8, cudaMemcpyHostToDevice, c->stream));
+    CUDA_TRY(cudaMemsetAsync(w + o_y, 0, (size_t)n * C * 8, c->stream));
+    CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
+    ENGINE_TRY(ld::engine_resident(s, plan, ra, c->stream));
+    std::vector<int32_t> it(C);
+    CUDA_TRY(cudaMemcpyAsync(c->h_pinned, s.remaining, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(it.data(), s.col_iters, C * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    int remaining = c->h_pinned[0], status = c->h_pinned[1];
+    if (status == ld::DEV_OVERFLOW && hcap < max_iter) return LD_OK;      // nothing written: the streaming form
+    if (status == ld::DEV_OVERFLOW) status = 0;                            // max_iter itself
+    *taken = true;
+    int64_t launches = 2;
+    if (status == 0 && remaining == 0) {
+        ENGINE_TRY(ld::engine_resident_funmv(s, plan, ra, ncols, c->stream));
+        launches += 3;
+    }
+    CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
+    CUDA_TRY(cudaMemcpyAsync(c->h_pinned, s.remaining, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
+    const bool good = status == 0 && remaining == 0;
+    if (good) CUDA_TRY(cudaStreamSynchronize(c->stream));
+    if (good && c->h_pinned[1] == 0)
+        CUDA_TRY(cudaMemcpyAsync(Y, ra.y, (size_t)n * C * 8, cudaMemcpyDeviceToHost, c->stream));
+    CUDA_TRY(cudaStreamSynchronize(c->stream));
+    if (good) status = c->h_pinned[1];
+    float ms = 0.f;
+    CUDA_TRY(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
+    ld_status st = LD_OK;
+    if (status == ld::DEV_NOTSPD) st = fail(LD_ENOTSPD, "p^T Q p <= 0: Q is not SPD");
+    else if (status == ld::DEV_TIMEOUT) st = fail(LD_ETIMEOUT, "device wait timed out");
+    else if (status != 0) st = fail(LD_ENUMERIC, "non-finite CG scalar");
+    else if (remaining > 0) st = fail(LD_ENOTCONV, "max_iter reached");
+    int iters = 0;
+    for (int v : it) iters = std::max(iters, v);
+    fill_info(c, info, st, iters, ms, launches, ms, 0);
+    if (info) {
+        info->engine = 4;
+        info->pass_words = -1;
+        info->bulk_rows = -1;
+    }
+    if (c->d_vec.bytes > ((size_t)256 << 20)) CUDA_TRY(c->d_vec.alloc(0));
+    return st;
+}
+
 // f(Q) V by the vector form of CG-M, for the rational f whose weights (N double2, on the
 // device) pair with the context's shifts: log (the context's weights) or z^{-1/2}
 static ld_status funmv(ld_ctx *c, int ncols, const double *V, double *Y, ld_info *info,
@@ -1552,6 +1677,9 @@ static ld_status funmv(ld_ctx *c, int ncols, const double *V, double *Y, ld_info
     if (!c || !V || !Y || ncols < 1) return fail(LD_EINVAL, "bad arguments");
     if (c->is_batch) return fail(LD_EINVAL, "batched context");
     REJECT_MATFREE(c);
+    bool taken = false;
+    if (ld_status st = funmv_resident(c, ncols, V, Y, info, weight_dev, &taken)) return st;
+    if (taken) return LD_OK;
     const int T = c->T, N = c->nshift;
     const int nt = (ncols + T - 1) / T, C = nt * T;
     const int64_t n = c->n;

@@ -14,7 +14,7 @@ constexpr int RES_ITEMS = 16;
 
 template <typename V, int KIND, int NT, bool KX>
 const void *res_fn() {
-    return reinterpret_cast<const void *>(&k_resident<V, KIND, NT, KX>);
+    return reinterpret_cast<const void *>(&k_resident<V, KIND, NT, KX, false>);
 }
 
 template <typename V>
@@ -30,13 +30,14 @@ const void *res_kernel(const Solve &s, int nt, bool keep_x0) {
 }
 
 // geometry of a team of M CTAs; false when it does not fit
-bool res_geometry(const Solve &s, bool keep_x0, int nt, int M, bool clustered, ResPlan &p) {
+bool res_geometry(const Solve &s, bool keep_x0, int yw, int nt, int M, bool clustered, ResPlan &p) {
     const int word = s.precision == 0 ? 8 : 4, E = 16 / word;
     const bool mat = s.op.kind == KIND_2D13_SQ, d3 = s.op.kind == KIND_3D7;
     const int H = mat ? 2 : 1;
     p.M = M;
     p.nt = nt;
     p.clustered = clustered;
+    p.yw = yw;
     p.G = (s.op.nx + E - 1) / E;
     if (p.G > nt) return false;
     p.pitch = (p.G + 2) * E;
@@ -60,7 +61,7 @@ bool res_geometry(const Solve &s, bool keep_x0, int nt, int M, bool clustered, R
     const int L = p.Ly * p.Lz;
     p.nseg = std::min(nt / p.G, L);
     p.cmax = (L + p.nseg - 1) / p.nseg;
-    if (p.cmax > RES_ITEMS) return false;
+    if (p.cmax > RES_ITEMS || p.cmax * (4 * (mat && !keep_x0 ? 1 : 2) + yw) > 128) return false;
     p.slots = 2 * H * p.Lz + (d3 ? 2 * p.Ly : 0);
     const ResSmem lay = res_smem(p, word, s.op.kind, s.nshift, keep_x0, !mat && s.op.field_d != nullptr);
     p.smem = lay.bytes;
@@ -123,7 +124,7 @@ cudaError_t res_launch(const ResPlan &p, cudaStream_t st, F &&fn) {
 
 }  // namespace
 
-int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, ResPlan *out) {
+static int resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, int yw, ResPlan *out) {
     const int k = s.op.kind;
     if ((k != KIND_2D5 && k != KIND_2D13_SQ && k != KIND_3D7) || s.asig || ncolours < 1) return 1;
     int dev = 0, sms = 0;
@@ -139,7 +140,7 @@ int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
         // one cluster a vector
         for (int M : {1, 2, 3, 4, 6, 8, 10, 12, 16}) {
             ResPlan p{};
-            if (!res_geometry(s, keep_x0, nt, M, true, p)) continue;
+            if (!res_geometry(s, keep_x0, yw, nt, M, true, p)) continue;
             p.J = ncolours;
             int act = 0;
             cudaError_t e = res_launch(p, nullptr, [&](cudaLaunchConfig_t &cfg) {
@@ -165,7 +166,7 @@ int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
             ResPlan p{}, q{};
             bool ok = false;
             for (int tries = 0; M >= 1 && tries < 24; --M, ++tries) {   // a 3D split wants a composite M
-                if (!res_geometry(s, keep_x0, nt, M, false, q)) {
+                if (!res_geometry(s, keep_x0, yw, nt, M, false, q)) {
                     if (k != KIND_3D7) break;
                     continue;
                 }
@@ -188,6 +189,14 @@ int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
     // contexts the grid engine would run: only where the passes would take longer
     if (streams && best >= stream_clocks(s, ncolours, keep_x0)) return 1;
     return best < 1e300 ? 0 : 1;
+}
+
+int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, ResPlan *out) {
+    return resident_plan(s, ncolours, keep_x0, streams, 0, out);
+}
+
+int engine_resident_plan_vec(const Solve &s, int ncols, ResPlan *out) {
+    return resident_plan(s, ncols, false, false, s.precision == 0 ? 4 : 8, out);
 }
 
 size_t engine_resident_rec_bytes(const ResPlan &p) {
@@ -238,6 +247,81 @@ int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *st
     ResPlan pv = p;
     ResArgs av = a;
     pv.smem = res_smem(p, s.precision == 0 ? 8 : 4, s.op.kind, s.nshift, kx, s.op.kind != KIND_2D13_SQ && s.op.field_d).bytes;
+    void *args[] = {&sv, &pv, &av};
+    e = res_launch(pv, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
+    if (e != cudaSuccess) cudaGetLastError();
+    return (int)e;
+}
+
+// ------------------------------------------------------------------ vector form
+// y = Re sum_l w_l x^{sigma_l}, every x^{sigma_l} a combination of the seed residuals r_k:
+// with p_0 = r_0, p_{k+1} = zeta_{k+1} r_{k+1} + beta_k p_k, x += alpha_k p_k per shift, the
+// weight of p_k in x is G_k = alpha_k + beta_k G_{k+1}, so y = sum_k coef_k r_k with
+// coef_k = Re sum_l w_l zeta_k G_k.  The solve records the shift scalars of every iteration,
+// the coefficients follow backwards, and the same CG runs again (its alpha and beta known: no
+// dots) adding coef_k r_k: one FP64 update a vertex and iteration in place of one complex
+// direction per shift.
+__global__ void k_funmv_back(Solve s, ResArgs a) {
+    const int c = blockIdx.x, l = threadIdx.x;
+    const int J = s.col_iters[c];
+    if (l >= s.nshift || !(s.class_size[c] > 0.0)) return;
+    double2 *h = a.hist + (size_t)c * a.hcap * s.nshift * 3 + 3 * l;
+    const size_t step = (size_t)s.nshift * 3;
+    const double2 w = s.weight[l];
+    double2 G = make_double2(0.0, 0.0);
+    constexpr int U = 4;        // records in flight
+    for (int k0 = J - 1; k0 >= 0; k0 -= U) {
+        double2 as[U], bs[U], z[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const double2 *q = h + (size_t)max(k0 - u, 0) * step;
+            as[u] = q[0];
+            bs[u] = q[1];
+            z[u] = q[2];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (k0 - u < 0) break;
+            G = cadd(as[u], cmul(bs[u], G));
+            const double2 f = cmul(w, z[u]);
+            h[(size_t)(k0 - u) * step].x = f.x * G.x - f.y * G.y;
+        }
+    }
+}
+
+// coef of every iteration: the shifts' parts in order
+__global__ void k_funmv_coef(Solve s, ResArgs a) {
+    const int c = blockIdx.y, J = s.col_iters[c];
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < J; k += gridDim.x * blockDim.x) {
+        const double2 *h = a.hist + ((size_t)c * a.hcap + k) * s.nshift * 3;
+        double v = 0.0;
+        for (int l = 0; l < s.nshift; ++l) v += h[3 * l].x;
+        a.coef[(size_t)c * a.hcap + k] = v;
+    }
+}
+
+template <typename V, int NT>
+static const void *replay_fn(int kind) {
+    if (kind == KIND_2D5) return reinterpret_cast<const void *>(&k_resident<V, KIND_2D5, NT, false, true>);
+    if (kind == KIND_3D7) return reinterpret_cast<const void *>(&k_resident<V, KIND_3D7, NT, false, true>);
+    return reinterpret_cast<const void *>(&k_resident<V, KIND_2D13_SQ, NT, false, true>);
+}
+
+int engine_resident_funmv(const Solve &s, const ResPlan &p, const ResArgs &a, int ncols, void *stream) {
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    k_funmv_back<<<ncols, (s.nshift + 31) / 32 * 32, 0, st>>>(s, a);
+    k_funmv_coef<<<dim3(8, ncols), 128, 0, st>>>(s, a);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return (int)e;
+    if (a.rec && (e = cudaMemsetAsync(a.rec, 0, engine_resident_rec_bytes(p), st)) != cudaSuccess) return (int)e;
+    const void *fn = s.precision == 0 ? (p.nt == 256 ? replay_fn<double, 256>(s.op.kind) : replay_fn<double, 512>(s.op.kind))
+                                      : (p.nt == 256 ? replay_fn<float, 256>(s.op.kind) : replay_fn<float, 512>(s.op.kind));
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+        return (int)e;
+    Solve sv = s;
+    ResPlan pv = p;
+    ResArgs av = a;
     void *args[] = {&sv, &pv, &av};
     e = res_launch(pv, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
     if (e != cudaSuccess) cudaGetLastError();

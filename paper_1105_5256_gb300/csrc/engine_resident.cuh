@@ -256,12 +256,15 @@ struct ResShift {
 // Shift recurrences of one finished iteration (alpha, beta, predicted rho = |r_{k+1}|^2,
 // measured vrn = v^T r_{k+1}); one warp.  Returns whether the column is still active.
 __device__ __forceinline__ bool res_tail(const Solve &s, const ResShift &h, double alpha, double beta, double rho,
-                                         double vrn, double ap, double bp, double lim2, bool &bad) {
+                                         double vrn, double ap, double bp, double lim2, double2 *hist, bool &bad) {
     const int lane = threadIdx.x & 31;
     bool any = rho > lim2;
     bad = !isfinite(vrn) || !isfinite(alpha) || !isfinite(beta);
     for (int l = lane; l < s.nshift; l += 32) {
-        if (!h.act[l]) continue;
+        if (!h.act[l]) {
+            if (hist) hist[3 * l] = hist[3 * l + 1] = hist[3 * l + 2] = make_double2(0.0, 0.0);
+            continue;
+        }
         const double2 sl = s.shift[l];
         const double2 z = h.z[l], zp = h.zp[l], phi = h.phi[l];
         // zeta_{k+1} / zeta_k as one complex quotient (see fused_tail)
@@ -273,6 +276,11 @@ __device__ __forceinline__ bool res_tail(const Solve &s, const ResShift &h, doub
         const double2 as = cscale(alpha, ratio);
         const double2 bs = cscale(beta, cmul(ratio, ratio));
         h.pi[l] = cadd(h.pi[l], cmul(as, phi));
+        if (hist) {
+            hist[3 * l] = as;
+            hist[3 * l + 1] = bs;
+            hist[3 * l + 2] = z;
+        }
         h.phi[l] = cadd(cscale(vrn, zn), cmul(bs, phi));
         h.zp[l] = z;
         h.z[l] = zn;
@@ -453,12 +461,14 @@ static __device__ __noinline__ void res_shift_role(const Solve &s, int stride, i
                 break;
             }
             if (!done) {
-                if (e.code) {
-                    if (lane == 0) set_status(s.status, e.code);
+                if (e.code || (ar.hist && iters >= ar.hcap)) {
+                    if (lane == 0) set_status(s.status, e.code ? e.code : DEV_OVERFLOW);
                     done = true;
                 } else {
                     bool bad;
-                    const bool still = res_tail(s, sh, e.alpha, e.beta, e.rho, e.vr, alpha_p, beta_p, lim2, bad);
+                    double2 *const hist = ar.hist ? ar.hist + ((size_t)c * ar.hcap + iters) * s.nshift * 3 : nullptr;
+                    if (hist && lane == 0) ar.ab[(size_t)c * ar.hcap + iters] = make_double2(e.alpha, e.beta);
+                    const bool still = res_tail(s, sh, e.alpha, e.beta, e.rho, e.vr, alpha_p, beta_p, lim2, hist, bad);
                     pi0 += e.alpha * phi0;
                     phi0 = e.vr + e.beta * phi0;
                     ++iters;
@@ -650,8 +660,57 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
     }
 }
 
+// The scalar warp of a replay: waits for the boundary rows, hands out the recorded alpha and
+// beta.  A CTA waits for its neighbours only.
+template <int NT, int KIND>
+__device__ __noinline__ void res_replay_role(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team, int m,
+                                             ResCtl *ctl, unsigned in_bytes) {
+    const int lane = threadIdx.x & 31, M = pl.M;
+    const bool clustered = pl.clustered;
+    const ResBlock<KIND> bk(s, pl, m);
+    ulonglong2 *const rec = clustered ? nullptr : ar.rec + (size_t)team * 2 * M * 8;
+    unsigned long long tick = 0;
+    for (int c = ar.cb + team; c < ar.ce; c += pl.J) {
+        if (!(s.class_size[c] > 0.0)) continue;
+        const int last = s.col_iters[c] - 1;
+        int stop = 0;
+        for (int it = 0; it < last; ++it, ++tick) {
+            const int par = (int)(tick & 1);
+            const double2 ab = ar.ab[(size_t)c * ar.hcap + it];
+            bool ok = true;
+            if (clustered) {
+                ok = res_bar_wait(smem_u32(&ctl->bar[par]), (unsigned)(tick >> 1) & 1u);
+                __syncwarp();
+                if (lane == 0) mbar_arrive_tx(&ctl->bar[par], in_bytes);      // armed for tick + 2
+            } else {
+                bar_sync(3, NT + 32);
+                __threadfence();
+                ulonglong2 *rp = rec + (size_t)par * M * 8;
+                if (lane == 0) rec_st(rp + (size_t)m * 8, 0.0, tick + 1);
+                double v;
+                if (lane < 4 && bk.has[lane]) ok = rec_wait(rp + (size_t)bk.nb(lane) * 8, tick + 1, v);
+                __threadfence();
+            }
+            if (!__all_sync(0xffffffffu, ok)) {
+                set_status(s.status, DEV_TIMEOUT);
+                stop = 2;
+            }
+            if (lane == 0) {
+                ctl->alpha = ab.x;
+                ctl->beta = ab.y;
+                ctl->stop = stop;
+            }
+            bar_sync(2, NT + 32);
+            if (stop) return;
+        }
+        tick += 2;      // the last iteration exchanges nothing: its parity's buffers are free, see below
+    }
+}
+
 // ------------------------------------------------------------------ vector warps
-template <typename V, int KIND, int NT, bool KX>
+// RP: replay of a finished solve (vector form): alpha, beta from its records, no dots,
+// y += coef_k r_k
+template <typename V, int KIND, int NT, bool KX, bool RP>
 __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team, int m,
                                                 unsigned char *smem, const ResSmem &lay, ResCtl *ctl) {
     constexpr int E = res_epi<V>(), NW = NT / 32;
@@ -679,7 +738,9 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
     // columns of this warp (two warps of a CTA of 256 share a lane quarter, four of 512)
     const uint32_t tmw = ctl->tm + ((uint32_t)(wid & 3) << 21) + (uint32_t)(wid >> 2) * 128u;    // w
     const uint32_t tma = tmw + 4u * cmax;                                                        // r or p
-    const uint32_t tmx = tma + (PRIV ? 4u * cmax : 0u), tmd = tmx + (lay.x_tm ? 4u * cmax : 0u);
+    constexpr uint32_t YW = sizeof(V) == 8 ? 4 : 8;            // words of an item's y (FP64)
+    const uint32_t tmy = tma + (PRIV ? 4u * cmax : 0u);
+    const uint32_t tmx = tmy + (uint32_t)pl.yw * cmax, tmd = tmx + (lay.x_tm ? 4u * cmax : 0u);
     const bool x_tm = lay.x_tm, d_tm = lay.d_tm, keepx = s.keep_x0;
     const size_t hstride = (size_t)pl.slots * GE;   // one parity of one CTA's halo buffer
     V *const hglob = clustered ? nullptr : static_cast<V *>(ar.halo) + (size_t)team * M * 2 * hstride;
@@ -775,6 +836,10 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
         for (int q = tid; q < (int)(lay.zero_bytes / 16); q += NT)
             reinterpret_cast<float4 *>(smem + lay.a)[q] = make_float4(0.f, 0.f, 0.f, 0.f);
         bar_sync(1, NT);
+        // the column's starting vector: its colour's indicator, or (vector form) a right-hand side
+        auto start = [&](int64_t v) -> V {
+            return ar.rhs ? (V)ar.rhs[v * ar.ld + c] : (s.colour[v] == c ? (V)1 : (V)0);
+        };
         uint64_t vbits = 0;                         // own-colour bits of the thread's vertices
         for (int i = 0, jy = jy0, jz = jz0; i < items; ++i, next_line(jy, jz)) {
             It r = zero_pack<V, E>();
@@ -782,9 +847,9 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                 const int64_t v0 = own_vertex(jy, jz);
 #pragma unroll
                 for (int e = 0; e < E; ++e)
-                    if (e < ev && s.colour[v0 + e] == c) {
-                        vbits |= 1ull << (i * E + e);
-                        r.v[e] = (V)1;
+                    if (e < ev) {
+                        r.v[e] = start(v0 + e);
+                        if (!ar.rhs && r.v[e] != (V)0) vbits |= 1ull << (i * E + e);
                     }
                 if constexpr (MAT) put(A + (size_t)sline(jy, jz) * pitch, g, r);
             }
@@ -793,6 +858,10 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
             tm_st<V>(tmw + 4u * i, zz);
             if constexpr (PRIV) tm_st<V>(tma + 4u * i, MAT ? zz : r);
             if (keepx && x_tm) tm_st<V>(tmx + 4u * i, zz);
+            if constexpr (RP) {
+#pragma unroll
+                for (uint32_t k = 0; k < YW; k += 4) tm_st<V>(tmy + YW * i + k, zz);
+            }
         }
         tm_wait_st();
         for (int q = tid; q < bk.slots * G; q += NT) {
@@ -808,15 +877,47 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
             It r = zero_pack<V, E>();
 #pragma unroll
             for (int e = 0; e < E; ++e)
-                if (gg * E + e < nx && s.colour[v0 + e] == c) r.v[e] = (V)1;
+                if (gg * E + e < nx) r.v[e] = start(v0 + e);
             if constexpr (MAT) put(A + (size_t)line * pitch, gg, r);
             else ri_st(RH + (size_t)sl * GE + gg * E, r);
         }
         V al = (V)0, be = (V)0;
         int stop = 0;
+        double al64 = 0.0, ck = 0.0;
+        int last = -1;
+        if constexpr (RP) {
+            last = s.col_iters[c] - 1;
+            ck = ar.coef[(size_t)c * ar.hcap];
+        }
+        // y += coef (r - alpha w) with r, w of the last iteration, in FP64 before rounding
+        auto y_add = [&](int i, const It &rold, const It &wv) {
+            if constexpr (sizeof(V) == 8) {
+                TmItem t;
+                tm_ld(t, tmy + YW * i);
+                const It r = PM::fma(PM::splat(-al * sc), wv, rold);
+                tm_wait(t);
+                tm_st<V>(tmy + YW * i, PM::fma(PM::splat((V)ck), r, tm_get<V>(t)));
+            } else {
+                TmItem t[2];
+                tm_ld(t[0], tmy + YW * i);
+                tm_ld(t[1], tmy + YW * i + 4);
+                const double a64 = -al64 * (double)sc;
+                tm_wait(t);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    ResItem<double> yv = tm_get<double>(t[h]);
+#pragma unroll
+                    for (int e = 0; e < 2; ++e)
+                        yv.v[e] = ::fma(ck, ::fma(a64, (double)wv.v[2 * h + e], (double)rold.v[2 * h + e]), yv.v[e]);
+                    tm_st<double>(tmy + YW * i + 4 * h, yv);
+                }
+            }
+        };
         for (int it = 0;; ++it, ++tick) {
             const int par = (int)(tick & 1);
             const It bb = PM::splat(be);
+            double ckn = 0.0;
+            if constexpr (RP) ckn = it < last ? ar.coef[(size_t)c * ar.hcap + it + 1] : 0.0;
             {
                 // ---- update r (and p, x) on own and halo lines
                 const It nas = PM::splat(-al * sc), aa = PM::splat(al);
@@ -844,6 +945,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         if (i >= items) break;
                         const bool act = i < cnt;
                         const It wv = tm_get<V>(tw[k]);
+                        if constexpr (RP) y_add(i, MAT ? old[k] : tm_get<V>(ta[PRIV ? k : 0]), wv);
                         if constexpr (MAT) {
                             const It r = PM::fma(nas, wv, old[k]);
                             if constexpr (KX) {
@@ -861,6 +963,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     }
                 }
                 tm_wait_st();
+                if (RP && it == last) break;          // y has its last term
                 const V *in = clustered ? HB + (size_t)(par ^ 1) * hstride : hglob + (size_t)(2 * m + (par ^ 1)) * hstride;
                 for (int q = tid; q < bk.slots * G; q += NT) {
                     const int sl = q / G, gg = q - sl * G;
@@ -913,7 +1016,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     u = PM::fma(bb, uo, u);
                     clip(u);
                     if (i < cnt) {
-                        d_pw = PM::fma(u, u, d_pw);
+                        if constexpr (!RP) d_pw = PM::fma(u, u, d_pw);
                         put(ul, g, u);
                     }
                     up = mid;
@@ -1029,13 +1132,15 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     if constexpr (MAT) clip(rv);   // a torus ghost inside a partial item is not r
                     tm_st<V>(tmw + 4u * i, wv);
                     if (act) {
-                        d_rr = PM::fma(rv, rv, d_rr);
-                        if constexpr (!MAT) d_pw = PM::fma(mid, wv, d_pw);
-                        d_rw = PM::fma(rv, wv, d_rw);
-                        d_ww = PM::fma(wv, wv, d_ww);
+                        if constexpr (!RP) {
+                            d_rr = PM::fma(rv, rv, d_rr);
+                            if constexpr (!MAT) d_pw = PM::fma(mid, wv, d_pw);
+                            d_rw = PM::fma(rv, wv, d_rw);
+                            d_ww = PM::fma(wv, wv, d_ww);
 #pragma unroll
-                        for (int e = 0; e < E; ++e)
-                            if ((unsigned)vb & (1u << e)) d_vr += rv.v[e];
+                            for (int e = 0; e < E; ++e)
+                                if ((unsigned)vb & (1u << e)) d_vr += rv.v[e];
+                        }
                         // boundary rows to the neighbours' halo slots
                         if constexpr (D3) {
                             if (jyc == 0 && bk.has[0]) send(0, bk.Lz + jzc, wv);
@@ -1071,6 +1176,12 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     else tm_wait(ta);
                 }
                 tm_wait_st();
+                if constexpr (RP) {
+                    if (!clustered) {
+                        __threadfence();
+                        bar_arrive(3, NT + 32);
+                    }
+                } else {
                 V flat[8] = {(V)0, (V)0, (V)0, (V)0, d_vr, (V)0, (V)0, (V)0};
 #pragma unroll
                 for (int e = 0; e < E; ++e) {
@@ -1091,14 +1202,49 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     __threadfence();       // boundary rows before the record of the scalar warp
                     bar_arrive(3, NT + 32);
                 }
+                }
             }
             bar_sync(2, NT + 32);
             al = (V)ctl->alpha;
             be = (V)ctl->beta;
             stop = ctl->stop;
+            if constexpr (RP) {
+                al64 = ctl->alpha;
+                ck = ckn;
+            }
             if (stop) break;
         }
         ++tick;
+        if constexpr (RP) {
+            // The next column starts on the parity the last iteration did not send: a neighbour
+            // may still read the other one.
+            ++tick;
+            for (int i = 0, jy = jy0, jz = jz0; i < items; ++i, next_line(jy, jz)) {
+                double yv[E];
+                if constexpr (sizeof(V) == 8) {
+                    TmItem t;
+                    tm_ld(t, tmy + YW * i);
+                    tm_wait(t);
+                    const It q = tm_get<V>(t);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) yv[e] = q.v[e];
+                } else {
+                    TmItem t[2];
+                    tm_ld(t[0], tmy + YW * i);
+                    tm_ld(t[1], tmy + YW * i + 4);
+                    tm_wait(t);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) yv[e] = tm_get<double>(t[e >> 1]).v[e & 1];
+                }
+                if (i < cnt) {
+                    const int64_t v0 = own_vertex(jy, jz);
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        if (e < ev) ar.y[(v0 + e) * ar.ld + c] = yv[e];
+                }
+                __syncwarp();
+            }
+        }
         if (keepx) {
             const int tile = c / s.T, t = c - tile * s.T;
             V *x = static_cast<V *>(s.x) + (int64_t)tile * s.op.n * s.T + t;
@@ -1128,7 +1274,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
 
 // ------------------------------------------------------------------ kernel
 // NT vector threads, then the scalar warp and the shift warp
-template <typename V, int KIND, int NT, bool KX>
+template <typename V, int KIND, int NT, bool KX, bool RP>
 __global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__ Solve s, const __grid_constant__ ResPlan pl,
                                                          const __grid_constant__ ResArgs ar) {
     constexpr int NW = NT / 32;
@@ -1143,7 +1289,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__
     if (pl.clustered) {
         const ResBlock<KIND> bk(s, pl, m);
         for (int d = 0; d < 4; ++d) in_bytes += (unsigned)(bk.halo_lines(d) * pl.G * 16);
-        in_bytes += (unsigned)(NP * RES_NDOT * 8) + 8u;
+        if (!RP) in_bytes += (unsigned)(NP * RES_NDOT * 8) + 8u;
     }
     if (wid == NW) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(&ctl->tm)),
@@ -1166,10 +1312,12 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__
     __syncthreads();
     if (pl.clustered) cluster_sync_all();          // barriers armed before any remote store
     if (wid < NW)
-        res_vector_role<V, KIND, NT, KX>(s, pl, ar, team, m, smem, lay, ctl);
+        res_vector_role<V, KIND, NT, KX, RP>(s, pl, ar, team, m, smem, lay, ctl);
+    else if (RP && wid == NW)
+        res_replay_role<NT, KIND>(s, pl, ar, team, m, ctl, in_bytes);
     else if (wid == NW)
         res_scalar_role<NT>(s, pl, ar, team, m, ctl, reinterpret_cast<const double *>(smem + lay.part), NP, in_bytes);
-    else if (m == 0)
+    else if (m == 0 && !RP)
         res_shift_role(s, pl.J, ar.cb + team, ar, ctl->q, &ctl->head, &ctl->tail, &ctl->done,
                        reinterpret_cast<double2 *>(smem + lay.shift));
     __syncwarp();

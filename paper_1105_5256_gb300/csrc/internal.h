@@ -61,7 +61,7 @@ inline void set_f32_coefs(Operator &op) {
 }
 
 // Status codes written by kernels into the device status word.
-enum { DEV_OK = 0, DEV_NOTSPD = 4, DEV_NUMERIC = 6, DEV_TIMEOUT = 7 };
+enum { DEV_OK = 0, DEV_NOTSPD = 4, DEV_NUMERIC = 6, DEV_TIMEOUT = 7, DEV_OVERFLOW = 100 };
 
 // Everything one solve's kernels need (passed by value).
 struct Solve {
@@ -123,6 +123,7 @@ struct ResPlan {
     int pitch;            // shared-memory line pitch (elements)
     int Ly, Lz;           // lines of a CTA at most
     int slots;            // halo lines of a CTA at most
+    int yw;               // vector form: words of y per item in tensor memory (4 FP64, 8 FP32), else 0
     size_t smem;
 };
 struct ResArgs {
@@ -130,7 +131,19 @@ struct ResArgs {
     int cap;              // iterations at most
     ulonglong2 *rec;      // cooperative teams: partial-sum records [J][2][M][8]
     void *halo;           // cooperative teams: boundary rows [J][M][2][slots][G]
+    // vector form (engine_resident_funmv): right-hand sides and results row-major, n x ld
+    const double *rhs;
+    double *y;
+    int ld;
+    int hcap;             // iterations the records below hold
+    double2 *hist;        // [column][iteration][shift][3]: alpha^sigma, beta^sigma, zeta
+    double2 *ab;          // [column][iteration]: alpha, beta
+    double *coef;         // [column][iteration]: y = sum_k coef_k r_k
 };
+// vector form on chip: y = Re sum_l weight_l (Q - sigma_l)^{-1} v for the columns of a.rhs;
+// plan with engine_resident_plan_vec.  DEV_OVERFLOW in *s.status: more than hcap iterations
+int engine_resident_plan_vec(const Solve &s, int ncols, ResPlan *out);
+int engine_resident_funmv(const Solve &s, const ResPlan &p, const ResArgs &a, int ncols, void *stream);
 // 0 and a plan when the engine takes the solve; nonzero otherwise.  streams: the context
 // would otherwise run the grid engine, so the plan must beat its passes
 int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, ResPlan *out);

@@ -26,7 +26,7 @@ __host__ __device__ inline ResSmem res_smem(const ResPlan &p, int word, int kind
     ResSmem s;
     // private vectors in tensor memory, 128 words a thread: w; r or (Matern with x) p; then
     // x and the diagonal while they fit
-    int room = 32 - p.cmax * (mat && !keepx ? 1 : 2);
+    int room = 32 - p.cmax * ((mat && !keepx ? 1 : 2) + p.yw / 4);
     s.x_tm = keepx && room >= p.cmax;
     if (s.x_tm) room -= p.cmax;
     s.d_tm = field && room >= p.cmax;

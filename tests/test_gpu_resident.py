@@ -170,3 +170,49 @@ def test_resident_csr_reports_not_spd():
     with pytest.raises(L.LogDetError) as e:
         L.ld_logdet(ctx)
     assert e.value.status == L.LD_ENOTSPD
+
+
+# ------------------------------------------------------------------ vector form
+@pytest.mark.parametrize("prec", [L.LD_FP64, L.LD_MIXED])
+@pytest.mark.parametrize("points,dims,per,form,ncols,shifts", [
+    (5, (1, 9), False, "", 1, 16),
+    (5, (33, 21), True, "mask", 3, 40),       # more shifts than a warp has lanes
+    (5, (62, 51), False, "field", 5, 20),
+    (13, (30, 34), True, "", 4, 20),          # one CTA a column, torus ghosts
+    (13, (130, 90), False, "", 2, 20),        # teams of many CTAs
+    (13, (48, 40), False, "", 160, 20),       # more columns than SMs
+    (7, (13, 11, 10), False, "field", 3, 20),
+])
+def test_resident_vector_form_matches_streaming_engine(points, dims, per, form, ncols, shifts, prec):
+    """log(Q) V and Q^{-1/2} V: the coefficient form on chip against the shifted directions.
+    Both stop each shift at a relative residual tol: 50 tol relative (FP32 vectors: 2e-5)."""
+    tol = 1e-9 if prec == L.LD_FP64 else 1e-6
+    n = int(np.prod(dims))
+    V = synth.random_probe_block(3, n, ncols)
+    V[:, -1] = 0.0 if ncols > 1 else V[:, -1]              # a zero column stays zero
+    out = []
+    for engine in (1, 0):
+        ctx = build((points, dims, per, 0.3, 1, form, (), shifts), prec, engine, None, tol)
+        Y, info = L.ld_logmv(ctx, V)
+        Z, _ = L.ld_invsqrt_mv(ctx, V)
+        out.append((Y, Z, info, L.ld_logmv(ctx, V)[0]))
+    assert out[0][2]["engine"] != 4 and out[1][2]["engine"] == 4
+    bar = 50 * tol if prec == L.LD_FP64 else 2e-5
+    for k in (0, 1):
+        assert np.linalg.norm(out[1][k] - out[0][k]) <= bar * np.linalg.norm(out[0][k])
+    assert np.array_equal(out[1][0], out[1][3])
+    if ncols > 1:
+        assert not out[1][0][:, -1].any()
+
+
+def test_vector_form_errors_leave_the_context_usable():
+    V = synth.random_probe_block(3, 40 * 30, 2)
+    ctx = build((5, (40, 30), False, 1e-4, 1, "", (), 20), L.LD_FP64, 0, None, 1e-10, max_iter=20)
+    Y = np.zeros_like(V)
+    with pytest.raises(L.LogDetError) as e:
+        L.ld_logmv(ctx, V)
+    assert e.value.status == L.LD_ENOTCONV
+    L.ld_set_params(ctx, 50.0, 0.0, 1.7)
+    Y, info = L.ld_logmv(ctx, V)
+    W, _ = L.ld_logmv(build((5, (40, 30), False, 50.0, 1, "", (), 20), L.LD_FP64, 1, None, 1e-10), V)
+    assert info["engine"] == 4 and np.linalg.norm(Y - W) <= 50e-10 * np.linalg.norm(W)
