@@ -382,8 +382,9 @@ ld_status ld_grid_bounds(const ld_matrix *Q, double *lmin, double *lmax);
 /* Batched evaluation of many independent grid GMRFs of uneven size in one persistent
  * launch (each (instance, tile) a work item).  Qs[count] (grid kinds), distances[count]
  * as in ld_create; every instance gets its own colouring, spectral bounds and nodes.
- * opt: precision, max_iter, tile_width (0 = chosen by timing short runs of the persistent
- * launch per candidate, cached per batch shape), cuda_stream.  An instance whose one-CTA
+ * opt: precision, max_iter, tile_width (0: instances whose columns a thread-block cluster can
+ * hold run on the resident engine; the width of any others is chosen by timing short runs of
+ * the persistent launch per candidate, cached per batch shape), cuda_stream.  An instance whose one-CTA
  * solve would outlast the batch (estimated from its size, its condition number and the
  * measured time of a CTA step) runs on the multi-CTA grid engine instead, several at once
  * on their own streams from host threads; for those to overlap, the process should set

@@ -162,6 +162,14 @@ struct ld_ctx {
     // batch: instances in the persistent launch (small) and on the multi-CTA engine (large)
     std::vector<int> small_idx, large_idx;
     cudaGraphExec_t bgraph = nullptr;
+    // batch: instances on the resident engine, by kind and cluster size (launch order)
+    struct ResClass {
+        int kind, M, first, count;
+        size_t smem;
+    };
+    std::vector<int> res_idx;
+    std::vector<ResClass> res_class;
+    DevBuf d_rb_solves, d_rb_plans, d_rb_items, d_rb_ncol, d_rb_out, d_rb_int;
     // matrix-free operator (ld_create_matfree): the caller's W = Q P drives the solve
     ld::Matfree *mf = nullptr;
     std::vector<double> mf_terms, mf_seeds;
@@ -1060,8 +1068,10 @@ ld_status ld_default_options(ld_options *opt) {
     return LD_OK;
 }
 
-ld_status ld_create(const ld_matrix *Q, int colouring_distance, int n_shifts, double tol,
-                    const ld_options *opt_in, ld_ctx **out) {
+// ld_create; vectors = false leaves the streaming engines' CG vectors out (batch instances of
+// the resident engine)
+static ld_status create_context(const ld_matrix *Q, int colouring_distance, int n_shifts, double tol,
+                                const ld_options *opt_in, bool vectors, ld_ctx **out) {
     if (!out) return fail(LD_EINVAL, "out is NULL");
     *out = nullptr;
     if (ld_status v = validate_matrix(Q)) return v;
@@ -1225,7 +1235,7 @@ ld_status ld_create(const ld_matrix *Q, int colouring_distance, int n_shifts, do
     // work buffers
     const size_t w = f32 ? 4 : 8;
     const size_t vb = (size_t)c->ntiles * c->n * c->T * w;
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < 2 && vectors; ++k) {
         CUDA_TRY(c->d_r[k].alloc(vb));
         CUDA_TRY(c->d_w[k].alloc(vb));
         CUDA_TRY(c->d_p[k].alloc(vb));
@@ -1295,6 +1305,11 @@ ld_status ld_create(const ld_matrix *Q, int colouring_distance, int n_shifts, do
     if (ld_status nd = set_nodes(c)) return nd;
     *out = guard.release();
     return LD_OK;
+}
+
+ld_status ld_create(const ld_matrix *Q, int colouring_distance, int n_shifts, double tol,
+                    const ld_options *opt_in, ld_ctx **out) {
+    return create_context(Q, colouring_distance, n_shifts, tol, opt_in, true, out);
 }
 
 ld_status ld_create_matfree(int64_t n, ld_matvec_fn matvec, void *user, const int32_t *colouring,
@@ -2006,8 +2021,117 @@ ld_status ld_grid_bounds(const ld_matrix *Q, double *lmin, double *lmax) {
 // host threads driving a batch's grid-engine instances at once
 constexpr int kBatchLargeThreads = 8;
 
+// cluster sizes a batch's columns run on
+constexpr int kClusterSizes[] = {1, 2, 3, 4, 6, 8, 10, 12, 16};
+
+// whether some cluster holds a column of the instance (host only)
+bool resident_batch_fits(const ld_matrix &Q, int n_shifts, int precision) {
+    Solve s{};
+    s.op.kind = Q.kind;
+    s.op.nx = Q.dims[0];
+    s.op.ny = Q.dims[1];
+    s.op.nz = Q.kind == LD_STENCIL_3D7 ? Q.dims[2] : 1;
+    s.op.field_d = Q.kappa2_field;      // only whether there is one
+    s.precision = precision == LD_MIXED ? 1 : 0;
+    s.nshift = n_shifts;
+    ld::ResPlan p;
+    double t;
+    for (int M : kClusterSizes)
+        if (ld::engine_resident_cluster(s, M, &p, &t)) return true;
+    return false;
+}
+
+// Cluster size of every resident instance, and the tables and launch classes.  A column on M
+// CTAs costs M t(M) SM-clocks an iteration: each instance takes the cheapest M, unless its
+// columns would then run longer than half of what the whole batch keeps the SMs busy; those
+// take the smallest M that does not (or the fastest).
+ld_status resident_batch_plan(ld_ctx *c, const ld_options &opt) {
+    const int nr = (int)c->res_idx.size();
+    struct Choice { ld::ResPlan p; double t; };
+    std::vector<std::vector<Choice>> all(nr);
+    std::vector<int> pick(nr, 0);
+    std::vector<double> iters(nr);
+    double busy = 0.0;
+    auto column = [&](int k, int o) { return iters[k] * all[k][o].t; };                   // clocks of one column
+    auto cost = [&](int k, int o) { return column(k, o) * all[k][o].p.M * c->subs[c->res_idx[k]]->ncolours; };
+    for (int k = 0; k < nr; ++k) {
+        const ld_ctx *sc = c->subs[c->res_idx[k]];
+        iters[k] = 0.55 * std::sqrt(sc->lmax / sc->lmin) * std::log(2.0 / c->tol) + 3.0;
+        for (int M : kClusterSizes) {
+            Choice ch;
+            if (ld::engine_resident_cluster(sc->s, M, &ch.p, &ch.t)) all[k].push_back(ch);
+        }
+        for (int o = 1; o < (int)all[k].size(); ++o)
+            if (cost(k, o) < cost(k, pick[k])) pick[k] = o;
+        busy += cost(k, pick[k]);
+    }
+    for (int round = 0; round < 3; ++round) {
+        const double limit = 0.5 * busy / 152.0;
+        busy = 0.0;
+        for (int k = 0; k < nr; ++k) {
+            int best = pick[k];
+            if (column(k, best) > limit) {
+                int fast = best, ok = -1;
+                for (int o = 0; o < (int)all[k].size(); ++o) {
+                    if (column(k, o) < column(k, fast)) fast = o;
+                    if (column(k, o) <= limit && (ok < 0 || cost(k, o) < cost(k, ok))) ok = o;
+                }
+                best = ok >= 0 ? ok : fast;
+            }
+            pick[k] = best;
+            busy += cost(k, best);
+        }
+    }
+    std::vector<Solve> solves(nr);
+    std::vector<ld::ResPlan> plans(nr);
+    std::vector<int> ncol(nr);
+    std::map<std::pair<int, int>, std::vector<int>> classes;        // (kind, M) -> instances
+    for (int k = 0; k < nr; ++k) {
+        const ld_ctx *sc = c->subs[c->res_idx[k]];
+        solves[k] = sc->s;
+        plans[k] = all[k][pick[k]].p;
+        ncol[k] = sc->ncolours;
+        classes[{sc->kind, plans[k].M}].push_back(k);
+    }
+    std::vector<int2> items;
+    std::vector<std::pair<double, ld_ctx::ResClass>> order;
+    for (auto &cl : classes) {
+        std::vector<int> &v = cl.second;
+        std::stable_sort(v.begin(), v.end(), [&](int a, int b) { return column(a, pick[a]) > column(b, pick[b]); });
+        ld_ctx::ResClass rc{cl.first.first, cl.first.second, (int)items.size(), 0, 0};
+        for (int k : v) {
+            rc.smem = std::max(rc.smem, plans[k].smem);
+            for (int q = 0; q < ncol[k]; ++q) items.push_back(make_int2(k, q));
+        }
+        rc.count = (int)items.size() - rc.first;
+        order.push_back({column(v[0], pick[v[0]]), rc});
+    }
+    // the longest columns first
+    std::stable_sort(order.begin(), order.end(), [](const auto &a, const auto &b) { return a.first > b.first; });
+    for (const auto &o : order) c->res_class.push_back(o.second);
+    auto put = [](DevBuf &d, const void *src, size_t bytes) {
+        cudaError_t e = d.alloc(bytes);
+        return e != cudaSuccess ? e : cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice);
+    };
+    CUDA_TRY(put(c->d_rb_solves, solves.data(), sizeof(Solve) * nr));
+    CUDA_TRY(put(c->d_rb_plans, plans.data(), sizeof(ld::ResPlan) * nr));
+    CUDA_TRY(put(c->d_rb_items, items.data(), sizeof(int2) * items.size()));
+    CUDA_TRY(put(c->d_rb_ncol, ncol.data(), sizeof(int) * nr));
+    CUDA_TRY(c->d_rb_out.alloc(sizeof(double) * 2 * nr));
+    CUDA_TRY(c->d_rb_int.alloc(sizeof(int) * 3 * nr));
+    const int ns = std::min((int)c->res_class.size(), (int)ld_ctx::kMaxGroups);
+    CUDA_TRY(cudaEventCreateWithFlags(&c->gfork, cudaEventDisableTiming));
+    for (int g = 0; g < ns; ++g) {
+        CUDA_TRY(cudaStreamCreateWithFlags(&c->gstream[g], cudaStreamNonBlocking));
+        CUDA_TRY(cudaEventCreateWithFlags(&c->gjoin[g], cudaEventDisableTiming));
+    }
+    (void)opt;
+    return LD_OK;
+}
+
+// resident: instances that a cluster holds run on the resident engine
 ld_status batch_build(int count, const ld_matrix *Qs, const int *distances, int n_shifts, double tol,
-                      const ld_options &opt, int T, double step_s, ld_ctx **out) {
+                      const ld_options &opt, int T, double step_s, bool resident, ld_ctx **out) {
     ld_ctx *c = new (std::nothrow) ld_ctx();
     if (!c) return fail(LD_ENOMEM, "host allocation");
     std::unique_ptr<ld_ctx> guard(c);
@@ -2040,19 +2164,22 @@ ld_status batch_build(int count, const ld_matrix *Qs, const int *distances, int 
         if (ld_status st = ld_grid_bounds(&Qs[i], &lo, &hi)) return st;
         int32_t dd[3] = {Qs[i].dims[0], Qs[i].dims[1], Qs[i].kind == LD_STENCIL_3D7 ? Qs[i].dims[2] : 1};
         const double est_s = 8.0 * std::sqrt(hi / lo) * ((double)grid_n(dd) / 128.0) * step_s;
-        const bool large = step_s > 0.0 && est_s > 0.8 && grid_n(dd) >= 32768;
+        const bool res = resident && resident_batch_fits(Qs[i], n_shifts, opt.precision);
+        const bool large = !res && step_s > 0.0 && est_s > 0.8 && grid_n(dd) >= 32768;
         ld_options o = sub;
         o.engine = large ? 1 : 2;
         o.cuda_stream = large ? nullptr : c->stream;
         ld_ctx *sc = nullptr;
-        ld_status st = ld_create(&Qs[i], distances[i], n_shifts, tol, &o, &sc);
+        ld_status st = create_context(&Qs[i], distances[i], n_shifts, tol, &o, !res, &sc);
         if (st != LD_OK) {
             std::string msg = g_err;
             return fail(st, "instance %d: %s", i, msg.c_str());
         }
         c->subs.push_back(sc);
-        (large ? c->large_idx : c->small_idx).push_back(i);
+        (res ? c->res_idx : large ? c->large_idx : c->small_idx).push_back(i);
     }
+    if (!c->res_idx.empty())
+        if (ld_status st = resident_batch_plan(c, opt)) return st;
     // the grid-engine instances run kBatchLargeThreads at a time: each plans for its share
     const int share = std::min((int)c->large_idx.size(), kBatchLargeThreads);
     for (int i : c->large_idx) {
@@ -2163,7 +2290,12 @@ ld_status ld_batch_create(int count, const ld_matrix *Qs, const int *distances, 
         if (distances[i] < 0) return fail(LD_EINVAL, "instance %d: colouring_distance must be >= 0", i);
     }
     const double default_step = 1.2e-6;   // one CTA step before any measurement
-    int T = opt.tile_width;
+    // no tile width asked for: instances that fit run on the resident engine, and only the
+    // others need a tuned width
+    const bool resident = opt.tile_width == 0 && opt.engine == 0;
+    bool all_resident = resident;
+    for (int i = 0; i < count && all_resident; ++i) all_resident = resident_batch_fits(Qs[i], n_shifts, opt.precision);
+    int T = all_resident ? (opt.precision == LD_MIXED ? 2 : 1) : opt.tile_width;
     double step_s = default_step;
     const std::string key = batch_key(count, Qs, distances, n_shifts, opt.precision);
     {
@@ -2183,7 +2315,7 @@ ld_status ld_batch_create(int count, const ld_matrix *Qs, const int *distances, 
             ld_options o = opt;
             o.max_iter = 16;
             ld_ctx *t = nullptr;
-            if (batch_build(count, Qs, distances, n_shifts, tol, o, cand[k], 0.0, &t) != LD_OK) continue;
+            if (batch_build(count, Qs, distances, n_shifts, tol, o, cand[k], 0.0, false, &t) != LD_OK) continue;
             std::vector<double> v(count);
             ld_info info{};
             ld_batch_logdet(t, v.data(), nullptr, &info);      // warm (usually LD_ENOTCONV)
@@ -2206,7 +2338,7 @@ ld_status ld_batch_create(int count, const ld_matrix *Qs, const int *distances, 
         std::lock_guard<std::mutex> lock(g_tune_mu);
         g_batch_tune[key] = {T, step_s};
     }
-    return batch_build(count, Qs, distances, n_shifts, tol, opt, T, step_s, out);
+    return batch_build(count, Qs, distances, n_shifts, tol, opt, T, step_s, resident, out);
 }
 
 ld_status ld_batch_logdet(ld_ctx *c, double *logdets, double *grads, ld_info *info) {
@@ -2217,9 +2349,35 @@ ld_status ld_batch_logdet(ld_ctx *c, double *logdets, double *grads, ld_info *in
     const int nsmall = (int)c->small_idx.size();
     std::vector<double> out(2 * std::max(nsmall, 1));
     std::vector<int> flags(4 * std::max(nsmall, 1));
+    const int nres = (int)c->res_idx.size();
+    std::vector<double> rout(2 * std::max(nres, 1));
+    std::vector<int> rint(3 * std::max(nres, 1));
     const auto t0 = std::chrono::steady_clock::now();
     // the persistent launch for the small instances first (asynchronous) ...
     if (nsmall > 0) CUDA_TRY(cudaGraphLaunch(c->bgraph, c->stream));
+    // the resident instances: one launch per kind and cluster size, side by side
+    if (nres > 0) {
+        const int max_iter = c->opt.max_iter > 0 ? c->opt.max_iter : 100000;
+        Solve *sd = c->d_rb_solves.as<Solve>();
+        double *od = c->d_rb_out.as<double>();
+        int *id = c->d_rb_int.as<int>();
+        ENGINE_TRY(ld::engine_resident_batch_prep(sd, nres, c->stream));
+        CUDA_TRY(cudaEventRecord(c->gfork, c->stream));
+        const int ns = std::min((int)c->res_class.size(), (int)ld_ctx::kMaxGroups);
+        for (int g = 0; g < ns; ++g) CUDA_TRY(cudaStreamWaitEvent(c->gstream[g], c->gfork, 0));
+        for (size_t k = 0; k < c->res_class.size(); ++k) {
+            const ld_ctx::ResClass &rc = c->res_class[k];
+            ENGINE_TRY(ld::engine_resident_batch(c->opt.precision == LD_MIXED ? 1 : 0, rc.kind, rc.M, rc.smem, sd,
+                                                 c->d_rb_plans.as<ld::ResPlan>(), c->d_rb_items.as<int2>() + rc.first,
+                                                 rc.count, max_iter, c->gstream[k % ld_ctx::kMaxGroups]));
+        }
+        for (int g = 0; g < ns; ++g) {
+            CUDA_TRY(cudaEventRecord(c->gjoin[g], c->gstream[g]));
+            CUDA_TRY(cudaStreamWaitEvent(c->stream, c->gjoin[g], 0));
+        }
+        ENGINE_TRY(ld::engine_batch_finish(sd, c->d_rb_ncol.as<int>(), nres, od, od + nres, id, id + nres, id + 2 * nres,
+                                           c->stream));
+    }
     // ... then the large ones, each across the GPU on its own stream; up to kLargeThreads
     // host threads drive them at once (a solve waits on its own stream between chunks of
     // passes, so one host thread per instance keeps several instances' passes in flight)
@@ -2249,7 +2407,7 @@ ld_status ld_batch_logdet(ld_ctx *c, double *logdets, double *grads, ld_info *in
         for (std::thread &th : pool) th.join();
     }
     int iters = 0;
-    int64_t tile_iters = 0, vertex_tile_iters = 0, launches = nsmall > 0 ? 3 : 0;
+    int64_t tile_iters = 0, vertex_tile_iters = 0, launches = (nsmall > 0 ? 3 : 0) + (nres > 0 ? 2 + (int)c->res_class.size() : 0);
     ld_status st = LD_OK;
     for (size_t k = 0; k < nl; ++k) {
         if (lst[k] != LD_OK) {
@@ -2265,6 +2423,10 @@ ld_status ld_batch_logdet(ld_ctx *c, double *logdets, double *grads, ld_info *in
         CUDA_TRY(cudaMemcpyAsync(out.data(), c->d_bout.p, sizeof(double) * 2 * nsmall, cudaMemcpyDeviceToHost, c->stream));
         CUDA_TRY(cudaMemcpyAsync(flags.data(), c->d_bint.p, sizeof(int) * 4 * nsmall, cudaMemcpyDeviceToHost, c->stream));
     }
+    if (nres > 0) {
+        CUDA_TRY(cudaMemcpyAsync(rout.data(), c->d_rb_out.p, sizeof(double) * 2 * nres, cudaMemcpyDeviceToHost, c->stream));
+        CUDA_TRY(cudaMemcpyAsync(rint.data(), c->d_rb_int.p, sizeof(int) * 3 * nres, cudaMemcpyDeviceToHost, c->stream));
+    }
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     const double ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     for (int k = 0; k < nsmall && st == LD_OK; ++k) {
@@ -2278,13 +2440,24 @@ ld_status ld_batch_logdet(ld_ctx *c, double *logdets, double *grads, ld_info *in
         else if (f == -1) st = fail(LD_ENOTCONV, "instance %d: max_iter reached", i);
         else st = fail(LD_ENUMERIC, "instance %d: non-finite CG scalar", i);
     }
+    for (int k = 0; k < nres && st == LD_OK; ++k) {
+        const int i = c->res_idx[k], f = rint[k];
+        iters = std::max(iters, rint[nres + k]);
+        tile_iters += rint[2 * nres + k];
+        vertex_tile_iters += c->subs[i]->n * rint[2 * nres + k];
+        if (f == 0) continue;
+        if (f == ld::DEV_NOTSPD) st = fail(LD_ENOTSPD, "instance %d: Q is not SPD", i);
+        else if (f == ld::DEV_TIMEOUT) st = fail(LD_ETIMEOUT, "instance %d: device wait timed out", i);
+        else if (f == -1) st = fail(LD_ENOTCONV, "instance %d: max_iter reached", i);
+        else st = fail(LD_ENUMERIC, "instance %d: non-finite CG scalar", i);
+    }
     if (info) {
         std::memset(info, 0, sizeof *info);
         info->status = st;
         info->n_shifts = c->nshift;
         info->iters = iters;
         info->tile_width = c->T;
-        info->engine = 2;
+        info->engine = nres == count ? 4 : 2;
         info->ms = ms;          // host wall time of the whole batch (both engines)
         info->iter_ms = ms;
         info->gpu_launches = launches;
@@ -2306,6 +2479,7 @@ ld_status ld_batch_logdet(ld_ctx *c, double *logdets, double *grads, ld_info *in
     };
     for (int k = 0; k < nsmall; ++k) put(c->small_idx[k], out[k], out[nsmall + k]);
     for (size_t k = 0; k < c->large_idx.size(); ++k) put(c->large_idx[k], lval[k], lseed[k]);
+    for (int k = 0; k < nres; ++k) put(c->res_idx[k], rout[k], rout[nres + k]);
     (void)count;
     return LD_OK;
 }

@@ -889,8 +889,14 @@ int engine_batch(const Solve *solves_dev, const int *ncolours_dev, int count, co
     e = dispatch<BatchLauncher>(precision, T, KIND_2D5, solves_dev, items_dev, nitems, queue_dev,
                                 max_iter, grid, st);
     if (e) return e;
-    k_batch_finish<<<(count + 127) / 128, 128, 0, st>>>(solves_dev, ncolours_dev, count, logdet_dev,
-                                                       seed_dev, flag_dev, iters_dev, tile_passes_dev);
+    return engine_batch_finish(solves_dev, ncolours_dev, count, logdet_dev, seed_dev, flag_dev, iters_dev,
+                               tile_passes_dev, stream);
+}
+
+int engine_batch_finish(const Solve *solves_dev, const int *ncolours_dev, int count, double *logdet_dev, double *seed_dev,
+                        int *flag_dev, int *iters_dev, int *tile_passes_dev, void *stream) {
+    k_batch_finish<<<(count + 127) / 128, 128, 0, static_cast<cudaStream_t>(stream)>>>(
+        solves_dev, ncolours_dev, count, logdet_dev, seed_dev, flag_dev, iters_dev, tile_passes_dev);
     return (int)cudaGetLastError();
 }
 

@@ -206,6 +206,16 @@ size_t engine_resident_halo_bytes(const ResPlan &p) {
     return p.clustered ? 0 : (size_t)p.J * p.M * 2 * p.slots * p.G * 16;
 }
 
+bool engine_resident_cluster(const Solve &s, int M, ResPlan *out, double *clocks) {
+    ResPlan p{};
+    if (!res_geometry(s, false, 0, RES_BATCH_NT, M, true, p)) return false;
+    if (p.smem > 225 * 1024) return false;          // beside the kernel's copies of Solve and plan
+    p.J = 1;
+    *out = p;
+    *clocks = res_clocks(s, p, false);
+    return true;
+}
+
 // state of the columns the engine does not solve, and the counters
 __global__ void k_resident_init(Solve s, int cb, int ce) {
     __shared__ int cnt;

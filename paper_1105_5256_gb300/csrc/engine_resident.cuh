@@ -492,6 +492,11 @@ static __device__ __noinline__ void res_shift_role(const Solve &s, int stride, i
         }
         for (int l = lane; l < s.nshift; l += 32) s.pi[(size_t)c * s.nshift + l] = sh.pi[l];
         if (lane == 0) {
+            if (ar.terms) {
+                double t = 0.0;
+                for (int l = 0; l < s.nshift; ++l) t += s.weight[l].x * sh.pi[l].x - s.weight[l].y * sh.pi[l].y;
+                s.terms[c] = t;
+            }
             s.pi0[c] = pi0;
             s.col_iters[c] = iters;
         }
@@ -1275,12 +1280,10 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
 // ------------------------------------------------------------------ kernel
 // NT vector threads, then the scalar warp and the shift warp
 template <typename V, int KIND, int NT, bool KX, bool RP>
-__global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__ Solve s, const __grid_constant__ ResPlan pl,
-                                                         const __grid_constant__ ResArgs ar) {
+__device__ __forceinline__ void resident_body(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team, int m,
+                                              unsigned char *smem) {
     constexpr int NW = NT / 32;
-    extern __shared__ __align__(16) unsigned char smem[];
     const int wid = threadIdx.x >> 5;
-    const int team = blockIdx.x / pl.M, m = blockIdx.x - team * pl.M;
     const ResSmem lay = res_smem(pl, (int)sizeof(V), KIND, s.nshift, s.keep_x0, KIND != KIND_2D13_SQ && s.op.field_d != nullptr);
     ResCtl *const ctl = reinterpret_cast<ResCtl *>(smem + lay.bc);
     constexpr uint32_t TM_COLS = NT == 256 ? 256 : 512;
@@ -1325,6 +1328,35 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__
     if (pl.clustered) cluster_sync_all();          // no CTA leaves while another may still store to it
     if (wid == NW)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(ctl->tm), "n"(TM_COLS));
+}
+
+template <typename V, int KIND, int NT, bool KX, bool RP>
+__global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__ Solve s, const __grid_constant__ ResPlan pl,
+                                                         const __grid_constant__ ResArgs ar) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int team = blockIdx.x / pl.M;
+    resident_body<V, KIND, NT, KX, RP>(s, pl, ar, team, blockIdx.x - team * pl.M, smem);
+}
+
+// A batch's items (instance, column) of one kind and cluster size: a cluster solves one item.
+template <typename V, int KIND, int NT>
+__global__ void __launch_bounds__(NT + 64, 1) k_resident_batch(const Solve *solves, const ResPlan *plans, const int2 *items,
+                                                               int M, int cap) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ Solve s;
+    __shared__ ResPlan pl;
+    const int2 it = items[blockIdx.x / M];
+    for (int q = threadIdx.x; q < (int)(sizeof(Solve) / 4); q += blockDim.x)
+        reinterpret_cast<uint32_t *>(&s)[q] = reinterpret_cast<const uint32_t *>(solves + it.x)[q];
+    for (int q = threadIdx.x; q < (int)(sizeof(ResPlan) / 4); q += blockDim.x)
+        reinterpret_cast<uint32_t *>(&pl)[q] = reinterpret_cast<const uint32_t *>(plans + it.x)[q];
+    __syncthreads();
+    ResArgs ar{};
+    ar.cb = it.y;
+    ar.ce = it.y + 1;
+    ar.cap = cap;
+    ar.terms = 1;
+    resident_body<V, KIND, NT, false, false>(s, pl, ar, 0, blockIdx.x % M, smem);
 }
 
 }  // namespace ld

@@ -129,6 +129,7 @@ struct ResPlan {
 struct ResArgs {
     int cb, ce;           // colour range
     int cap;              // iterations at most
+    int terms;            // 1: the shift warp also writes s.terms (batches)
     ulonglong2 *rec;      // cooperative teams: partial-sum records [J][2][M][8]
     void *halo;           // cooperative teams: boundary rows [J][M][2][slots][G]
     // vector form (engine_resident_funmv): right-hand sides and results row-major, n x ld
@@ -147,6 +148,15 @@ int engine_resident_funmv(const Solve &s, const ResPlan &p, const ResArgs &a, in
 // 0 and a plan when the engine takes the solve; nonzero otherwise.  streams: the context
 // would otherwise run the grid engine, so the plan must beat its passes
 int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, ResPlan *out);
+// batches: geometry of a cluster of M CTAs for one column (false: does not fit), estimated
+// clocks of an iteration, and the launches of one kind and cluster size
+constexpr int RES_BATCH_NT = 512;
+bool engine_resident_cluster(const Solve &s, int M, ResPlan *out, double *clocks);
+int engine_resident_batch_prep(const Solve *solves_dev, int count, void *stream);
+int engine_resident_batch(int precision, int kind, int M, size_t smem, const Solve *solves_dev, const ResPlan *plans_dev,
+                          const int2 *items_dev, int nitems, int cap, void *stream);
+int engine_batch_finish(const Solve *solves_dev, const int *ncolours_dev, int count, double *logdet_dev, double *seed_dev,
+                        int *flag_dev, int *iters_dev, int *tile_passes_dev, void *stream);
 size_t engine_resident_rec_bytes(const ResPlan &p);
 size_t engine_resident_halo_bytes(const ResPlan &p);
 int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *stream);

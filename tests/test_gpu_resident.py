@@ -216,3 +216,39 @@ def test_vector_form_errors_leave_the_context_usable():
     Y, info = L.ld_logmv(ctx, V)
     W, _ = L.ld_logmv(build((5, (40, 30), False, 50.0, 1, "", (), 20), L.LD_FP64, 1, None, 1e-10), V)
     assert info["engine"] == 4 and np.linalg.norm(Y - W) <= 50e-10 * np.linalg.norm(W)
+
+
+# ------------------------------------------------------------------ batches
+@pytest.mark.parametrize("prec", [L.LD_FP64, L.LD_MIXED])
+def test_resident_batch_matches_single_solves(prec):
+    """A batch over kinds, boundaries and sizes from one CTA a column to sixteen, and a lattice
+    too wide for any cluster beside them, against streaming contexts one by one (both stop at
+    tol: 50 tol of the terms' sum, FP32 vectors 2e-5)."""
+    tol = 1e-9 if prec == L.LD_FP64 else 1e-6
+    insts = [(5, (9, 7), False, 0.5, 2, ""), (13, (30, 34), True, 0.3, 1, ""), (5, (61, 50), True, 0.3, 2, "mask"),
+             (7, (13, 11, 10), False, 1.0, 2, "field"), (13, (130, 90), False, 0.2, 2, ""), (5, (300, 220), False, 0.5, 1, ""),
+             (5, (2100, 6), False, 0.5, 1, ""), (13, (200, 210), False, 0.6, 1, "")]
+    mats, ref, bars = [], [], []
+    for points, dims, per, k2, d, form in insts:
+        n = int(np.prod(dims))
+        m = lambda: L.grid_matrix(K[points], dims, k2, periodic=per, tau=3.0 if form == "mask" else 0.0,
+                                  kappa2_field=synth.kappa2_field(7, dims) if form == "field" else None,
+                                  obs_mask=synth.obs_mask(8, n, 0.2) if form == "mask" else None)
+        mats.append(m())
+        ctx = L.ld_create(m(), d, 20, tol, L.options(precision=prec, engine=1, tile_width=2))
+        ref.append(L.ld_logdet(ctx)[0])
+        bars.append((50 * tol if prec == L.LD_FP64 else 2e-5) * np.abs(L.ld_column_terms(ctx)[0]).sum())
+    b = L.ld_batch_create(mats, [i[4] for i in insts], 20, tol, L.options(precision=prec))
+    vals, grads, info = L.ld_batch_logdet(b, with_grad=True)
+    assert np.all(np.abs(vals - ref) <= bars), (vals, ref)
+    assert np.isnan(grads[1]) and np.isnan(grads[3]) and np.all(np.isfinite(np.delete(grads, [1, 3, 4, 7])))
+    again, _, _ = L.ld_batch_logdet(b)
+    assert np.array_equal(again, vals)
+
+
+def test_resident_batch_names_the_instance_that_fails():
+    mats = [L.grid_matrix(K[5], (40, 30), k2) for k2 in (0.5, 1e-5, 0.5)]
+    b = L.ld_batch_create(mats, [1, 1, 1], 20, 1e-10, L.options(max_iter=60))
+    with pytest.raises(L.LogDetError) as e:
+        L.ld_batch_logdet(b)
+    assert e.value.status == L.LD_ENOTCONV and "instance 1" in str(e.value)
