@@ -534,6 +534,141 @@ __global__ void __launch_bounds__(256) k_true_residual(Solve s, int set, int cb,
     if (threadIdx.x < T) atomicAdd(&norm2[tile * T + threadIdx.x], tot[threadIdx.x]);
 }
 
+// The same for the 5- and 7-point lattices, as a sweep: a warp owns 32 lattice columns and
+// marches along the slowest axis with a register window, so that every x is loaded (and
+// widened) once and horizontal neighbours cross the lanes; in 3D eight warps own eight lines
+// in y and exchange them through shared memory.  Bound by the FP64 units (19 clocks a warp
+// instruction): with the seed solution in x_hi the difference form, its horizontal and
+// marching differences shared between neighbours, else the direct form, whose 1e-15 |x| is
+// far below what x in its own precision leaves.  Against the gather kernel above: 2048^2
+// with x_hi, 18 columns, 2.62 -> 1.75 ms; 128^3, x in FP32, 112 columns, 10.1 -> 5.6 ms.
+template <typename V, int T, int KIND, bool DIFF>
+__global__ void __launch_bounds__(256) k_residual_sweep(Solve s, int set, int cb, int ce, int replace, int seg,
+                                                        double *norm2) {
+    constexpr bool D3 = KIND == KIND_3D7;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int nx = s.op.nx, ny = s.op.ny, nm = D3 ? s.op.nz : ny;       // nm: extent of the marching axis
+    const bool per = s.op.periodic;
+    const int tile = blockIdx.z;
+    // y blocks (3D) and segments of the marching axis share blockIdx.y
+    const int yb = D3 ? (ny + 7) / 8 : 1;
+    const int m0 = ((int)blockIdx.y / yb) * seg, m1 = min(m0 + seg, nm);
+    // difference form: lane 0 only supplies its neighbour's left difference
+    constexpr int W = DIFF ? 31 : 32;
+    const int gx = (D3 ? (int)blockIdx.x : (int)blockIdx.x * 8 + wid) * W + lane - (DIFF ? 1 : 0);
+    const int gy = D3 ? ((int)blockIdx.y % yb) * 8 + wid : 0;
+    const bool own = gx < nx && (!D3 || gy < ny) && (!DIFF || lane > 0);
+    const bool in = own || (DIFF && lane == 0 && (!D3 || gy < ny));       // lanes that load
+    const int64_t n = s.op.n, off = (int64_t)tile * n * T;
+    const int64_t step = D3 ? (int64_t)nx * ny : nx;                    // vertices between marching positions
+    const V *const x = static_cast<const V *>(s.x) + off;
+    const double *const xh = s.xhi ? s.xhi + off : nullptr;
+    V *const r = static_cast<V *>(set ? s.rbuf[1] : s.rbuf[0]) + off;
+    const bool write = replace && !s.tile_done[tile];
+    struct D { double v[T]; };
+    auto load = [&](int64_t j) {
+        D o;
+        if (xh) {
+            const Pack<double, T> q = ldpack<double, T, true>(xh, j);
+#pragma unroll
+            for (int t = 0; t < T; ++t) o.v[t] = q.v[t];
+        } else {
+            const Pack<V, T> q = ldpack<V, T, true>(x, j);
+#pragma unroll
+            for (int t = 0; t < T; ++t) o.v[t] = (double)q.v[t];
+        }
+        return o;
+    };
+    const D zero = {};
+    // x at (xx, yy) of marching position m, wrapped on a torus, zero outside a Dirichlet grid
+    auto at = [&](int xx, int yy, int m) {
+        if (per) {
+            xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
+            if constexpr (D3) yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
+            m = m < 0 ? m + nm : (m >= nm ? m - nm : m);
+        } else if (xx < 0 || xx >= nx || m < 0 || m >= nm || (D3 && (yy < 0 || yy >= ny))) {
+            return zero;
+        }
+        return load((int64_t)m * step + (D3 ? (int64_t)yy * nx : 0) + xx);
+    };
+    __shared__ double sh[D3 ? 2 * 8 * 32 * T : 1];
+    __shared__ double red[8 * T];
+    __shared__ double tot[T];
+    const bool rfix = lane == 31 || gx == nx - 1, lfix = !DIFF && (lane == 0 || gx == 0);
+    const double sc = s.op.scale, k2 = s.op.kappa2;
+    double acc[T];
+#pragma unroll
+    for (int t = 0; t < T; ++t) acc[t] = 0.0;
+    D dn = in ? at(gx, gy, m0 - 1) : zero, c = in ? at(gx, gy, m0) : zero;
+    double dp[DIFF ? T : 1];                           // c - up of the position before
+    if constexpr (DIFF) {
+#pragma unroll
+        for (int t = 0; t < T; ++t) dp[t] = dn.v[t] - c.v[t];
+    }
+    for (int m = m0; m < m1; ++m) {
+        const D up = in ? at(gx, gy, m + 1) : zero;
+        const int64_t i = own ? (int64_t)m * step + (D3 ? (int64_t)gy * nx : 0) + gx : 0;
+        const int col = s.colour[i];
+        const double dg = s.op.diag_d ? s.op.diag_d[i] : k2;
+        D ya = zero, yc = zero;
+        if constexpr (D3) {
+            double *row = sh + (size_t)((m & 1) * 8 + wid) * 32 * T + lane * T;
+#pragma unroll
+            for (int t = 0; t < T; ++t) row[t] = c.v[t];
+            __syncthreads();
+            if (wid > 0) {
+#pragma unroll
+                for (int t = 0; t < T; ++t) ya.v[t] = row[t - 32 * T];
+            } else if (in) {
+                ya = at(gx, gy - 1, m);
+            }
+            if (wid < 7 && gy + 1 < ny) {
+#pragma unroll
+                for (int t = 0; t < T; ++t) yc.v[t] = row[t + 32 * T];
+            } else if (in) {
+                yc = at(gx, gy + 1, m);
+            }
+        }
+        D rt, lf;
+#pragma unroll
+        for (int t = 0; t < T; ++t) rt.v[t] = __shfl_down_sync(0xffffffffu, c.v[t], 1);
+        if (rfix && in) rt = at(gx + 1, gy, m);
+        if constexpr (!DIFF) {
+#pragma unroll
+            for (int t = 0; t < T; ++t) lf.v[t] = __shfl_up_sync(0xffffffffu, c.v[t], 1);
+            if (lfix && in) lf = at(gx - 1, gy, m);
+        }
+        V out[T];
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+            double w;
+            if constexpr (DIFF) {
+                // E = c - right, the left lane's E is left - c; D = c - up, the last one dn - c
+                const double e = c.v[t] - rt.v[t], d = c.v[t] - up.v[t];
+                const double el = __shfl_up_sync(0xffffffffu, e, 1);
+                double h = (e - el) + (d - dp[t]);
+                dp[t] = d;
+                if constexpr (D3) h += (c.v[t] - ya.v[t]) + (c.v[t] - yc.v[t]);
+                w = fma(dg, c.v[t], h);
+            } else {
+                double h = (lf.v[t] + rt.v[t]) + (dn.v[t] + up.v[t]);
+                if constexpr (D3) h += ya.v[t] + yc.v[t];
+                w = fma(dg + (D3 ? 6.0 : 4.0), c.v[t], -h);
+            }
+            const int k = tile * T + t;
+            const bool live = k >= cb && k < ce;
+            const double res = live ? fma(-sc, w, col == k ? 1.0 : 0.0) : 0.0;
+            if (own) acc[t] = fma(res, res, acc[t]);
+            out[t] = (V)res;
+        }
+        if (write && own) stpack<V, T>(r, i, out);
+        dn = c;
+        c = up;
+    }
+    block_sum_to<double, T>(acc, red, tot);
+    if (threadIdx.x < T) atomicAdd(&norm2[tile * T + threadIdx.x], tot[threadIdx.x]);
+}
+
 // ------------------------------------------------------------------ gradient (backward)
 // g_eta = sum_c (E_eta v_c)^T x0_c = sum_i sum_j E_ij x0[i, colour(j)], E = dQ/d eta.
 // E per parameter id: kappa2 -> scale*diag(field or 1) (grid 5/7-pt), 2*scale*Q1 (13-pt);
@@ -689,6 +824,24 @@ struct ResidualLauncher {
             k_fold_x<V, T><<<blocks, 256, 0, st>>>(s);
             e = (int)cudaGetLastError();
             if (e) return e;
+        }
+        if constexpr (KIND == KIND_2D5 || KIND == KIND_3D7) {
+            // segments of the marching axis: about eight blocks an SM, at least 16 positions each
+            constexpr bool D3 = KIND == KIND_3D7;
+            const int nm = D3 ? s.op.nz : s.op.ny, yb = D3 ? (s.op.ny + 7) / 8 : 1;
+            const int W = (D3 ? 1 : 8) * (s.xhi ? 31 : 32), xb = (s.op.nx + W - 1) / W;
+            int64_t segs = (int64_t)152 * 8 / std::max<int64_t>(1, (int64_t)xb * yb * s.ntiles);
+            segs = std::max<int64_t>(1, std::min<int64_t>(segs, (nm + 15) / 16));
+            while (segs * yb > 65535) segs = (segs + 1) / 2;
+            const int seg = (int)((nm + segs - 1) / segs);
+            if (yb <= 65535 && s.ntiles <= 65535) {
+                const dim3 grid(xb, (unsigned)(yb * ((nm + seg - 1) / seg)), s.ntiles);
+                if (s.xhi)
+                    k_residual_sweep<V, T, KIND, true><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, seg, norm2);
+                else
+                    k_residual_sweep<V, T, KIND, false><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, seg, norm2);
+                return (int)cudaGetLastError();
+            }
         }
         int bx = (int)((s.op.n + 255) / 256);
         if (bx > 152 * 8) bx = 152 * 8;
