@@ -97,6 +97,9 @@ struct ld_ctx {
     int64_t n = 0;
     double kappa2 = 0, tau = 0, scale = 1;
     bool has_field = false, has_mask = false, mask_any = false;
+    // the field's range: kappa2 >= 0, so its products' range is kappa2 times this, rounding
+    // included, and ld_set_params need not read the field back and scan it (128^3: about 3 of 140 ms a step)
+    double field_min = NAN, field_max = NAN, field_some = NAN;   // field_some: any finite value
     int distance = 0, nshift = 0;
     bool auto_shift = false;   // n_shifts = 0: N chosen from the quadrature certificate
     int nshift_cap = 0;        // shift-state capacity of d_shift / d_nodes (columns x nodes)
@@ -365,7 +368,7 @@ ld_status set_nodes(ld_ctx *c) {
     return LD_OK;
 }
 
-ld_status compute_bounds(ld_ctx *c, const double *field) {
+ld_status compute_bounds(ld_ctx *c) {
     if (c->user_bounds) {
         c->lmin = c->opt.lambda_min;
         c->lmax = std::max(c->opt.lambda_max, 1.01 * c->opt.lambda_min);
@@ -378,11 +381,11 @@ ld_status compute_bounds(ld_ctx *c, const double *field) {
     }
     double k2min = c->kappa2, k2max = c->kappa2;
     if (c->has_field) {
-        k2min = INFINITY;
+        k2min = INFINITY;                // what a field without a number in it leaves
         k2max = -INFINITY;
-        for (int64_t i = 0; i < c->n; ++i) {
-            k2min = std::min(k2min, c->kappa2 * field[i]);
-            k2max = std::max(k2max, c->kappa2 * field[i]);
+        for (double f : {c->field_min, c->field_max, c->field_some}) {
+            k2min = std::min(k2min, c->kappa2 * f);       // 0 * inf drops out, as any NaN does
+            k2max = std::max(k2max, c->kappa2 * f);
         }
     }
     grid_bounds(c->kind, c->dims, c->periodic, k2min, k2max, c->mask_any ? c->tau : 0.0, c->scale,
@@ -1181,7 +1184,12 @@ static ld_status create_context(const ld_matrix *Q, int colouring_distance, int 
     CUDA_TRY(cudaMemcpy(c->d_colour.p, c->colour.data(), c->n * sizeof(int32_t), cudaMemcpyHostToDevice));
     if (c->has_field) {
         std::vector<float> ff(c->n);
-        for (int64_t i = 0; i < c->n; ++i) ff[i] = (float)Q->kappa2_field[i];
+        for (int64_t i = 0; i < c->n; ++i) {
+            ff[i] = (float)Q->kappa2_field[i];
+            c->field_min = std::fmin(c->field_min, Q->kappa2_field[i]);
+            c->field_max = std::fmax(c->field_max, Q->kappa2_field[i]);
+            if (std::isfinite(Q->kappa2_field[i])) c->field_some = Q->kappa2_field[i];
+        }
         CUDA_TRY(c->d_field_d.alloc(c->n * sizeof(double)));
         CUDA_TRY(cudaMemcpy(c->d_field_d.p, Q->kappa2_field, c->n * sizeof(double), cudaMemcpyHostToDevice));
         CUDA_TRY(c->d_field_f.alloc(c->n * sizeof(float)));
@@ -1301,7 +1309,7 @@ static ld_status create_context(const ld_matrix *Q, int colouring_distance, int 
     s.partial = c->d_partial.as<double>();
     CUDA_TRY(cudaMemset(c->d_tile.p, 0, c->d_tile.bytes));
 
-    if (ld_status b = compute_bounds(c, Q->kappa2_field)) return b;
+    if (ld_status b = compute_bounds(c)) return b;
     if (ld_status nd = set_nodes(c)) return nd;
     *out = guard.release();
     return LD_OK;
@@ -1407,12 +1415,7 @@ ld_status ld_set_params(ld_ctx *c, double kappa2, double tau, double scale) {
     c->solved = false;
     c->have_x0 = false;
     if (!c->user_bounds) {
-        std::vector<double> field;
-        if (c->has_field) {
-            field.resize(c->n);
-            CUDA_TRY(cudaMemcpy(field.data(), c->d_field_d.p, c->n * sizeof(double), cudaMemcpyDeviceToHost));
-        }
-        if (ld_status b = compute_bounds(c, field.empty() ? nullptr : field.data())) return b;
+        if (ld_status b = compute_bounds(c)) return b;
     }
     return set_nodes(c);
 }
