@@ -109,6 +109,21 @@ __device__ __forceinline__ ResItem<V> res_level(const ResItem<V> &c, const ResIt
     }
 }
 
+// The FP32 level of a 2D lattice with each difference formed once: e between neighbours of
+// the line (scalar adds, which need no re-paired operands and leave the paired pipe free),
+// d = m - (next line) kept for the next line's level as its dp.  Bits as in res_level.
+__device__ __forceinline__ ResItem<float> res_level_sh(const ResItem<float> &c, const ResItem<float> &m, float l,
+                                                       float r, const ResItem<float> &d, const ResItem<float> &dp) {
+    using M = PackMath<float, 4>;
+    const float el = l - m.v[0], e0 = m.v[0] - m.v[1], e1 = m.v[1] - m.v[2], e2 = m.v[2] - m.v[3], er = m.v[3] - r;
+    ResItem<float> h;
+    h.v[0] = e0 - el;
+    h.v[1] = e1 - e0;
+    h.v[2] = e2 - e1;
+    h.v[3] = er - e2;
+    return M::fma(c, m, M::add(h, M::sub(d, dp)));
+}
+
 // Sum eight values over the warp: on return lane l holds the total of value l >> 2.
 // Halving exchange: 4 + 2 + 1 + 1 + 1 additions instead of 8 x 5 (FP64 adds are narrow).
 template <typename A>
@@ -721,6 +736,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
     constexpr int E = res_epi<V>(), NW = NT / 32;
     constexpr bool MAT = KIND == KIND_2D13_SQ, D3 = KIND == KIND_3D7;
     constexpr int H = MAT ? 2 : 1, NB = D3 ? 6 : 4;
+    constexpr bool SH = sizeof(V) == 4 && !D3;   // differences shared between lines
     constexpr bool PRIV = !MAT || KX;          // second private vector: r, or p (Matern with x)
     using It = ResItem<V>;
     using PM = PackMath<V, E>;
@@ -998,39 +1014,46 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
             if constexpr (MAT) {
                 // ---- u = Q1 r + beta u on own lines and one line beyond on each side
                 const It cc = PM::splat(k2);
-                // a row ahead: the line below and the old u of the next row load, and its
-                // neighbours cross the lanes, while this row is formed
-                const V *row = A + (size_t)(H + l0) * pitch + go;
+                // a row ahead: the line below, the old u and the side neighbours of the next row
+                // load while this row is formed.  Loads past the run's end are clamped to the
+                // block's lines and not used.
+                int om = (H + l0) * pitch + go, od = om + pitch, ou = (1 + l0) * pitch + go;
+                const int odmax = (L + 2 * H - 1) * pitch + go, oumax = (L + 1) * pitch + go;
                 V *ul = B + (size_t)(1 + l0) * pitch;
-                It up = ri_ld(row - pitch), mid = ri_ld(row), dn = ri_ld(row + pitch), uo = ri_ld(ul + go);
-                V l = __shfl_up_sync(0xffffffffu, mid.v[E - 1], 1), r = __shfl_down_sync(0xffffffffu, mid.v[0], 1);
-                if (lfix) l = row[-1];
-                if (rfix) r = row[E];
+                It up = ri_ld(A + om - pitch), mid = ri_ld(A + om), dn = ri_ld(A + od), uo = ri_ld(B + ou);
+                if constexpr (SH) up = PM::sub(up, mid);
+                V l = A[om - 1], r = A[om + E];
 #pragma unroll 2
                 for (int i = 0; i < items; ++i) {
-                    const bool more = i + 1 < cnt;
-                    It dn2 = dn, uo2 = uo;
-                    if (more) {
-                        dn2 = ri_ld(row + 2 * pitch);
-                        uo2 = ri_ld(ul + pitch + go);
+                    om = od;
+                    od = min(od + pitch, odmax);
+                    ou = min(ou + pitch, oumax);
+                    const It dn2 = ri_ld(A + od), uo2 = ri_ld(B + ou);
+                    // side neighbours: across the lanes, and from the line at the warp's ends
+                    const V ls = __shfl_up_sync(0xffffffffu, dn.v[E - 1], 1), rs = __shfl_down_sync(0xffffffffu, dn.v[0], 1);
+                    V le = (V)0, re = (V)0;
+                    if (lfix) le = A[om - 1];
+                    if (rfix) re = A[om + E];
+                    It u;
+                    if constexpr (SH) {
+                        const It d = PM::sub(mid, dn);
+                        u = res_level_sh(cc, mid, l, r, d, up);
+                        up = d;
+                    } else {
+                        u = res_level<V, 4>(cc, mid, l, r, dn, up, zz, zz);
+                        up = mid;
                     }
-                    V l2 = __shfl_up_sync(0xffffffffu, dn.v[E - 1], 1), r2 = __shfl_down_sync(0xffffffffu, dn.v[0], 1);
-                    if (lfix && more) l2 = row[pitch - 1];
-                    if (rfix && more) r2 = row[pitch + E];
-                    It u = res_level<V, 4>(cc, mid, l, r, dn, up, zz, zz);
                     u = PM::fma(bb, uo, u);
                     clip(u);
                     if (i < cnt) {
                         if constexpr (!RP) d_pw = PM::fma(u, u, d_pw);
                         put(ul, g, u);
                     }
-                    up = mid;
                     mid = dn;
                     dn = dn2;
                     uo = uo2;
-                    l = l2;
-                    r = r2;
-                    row += pitch;
+                    l = lfix ? le : ls;
+                    r = rfix ? re : rs;
                     ul += pitch;
                 }
                 for (int q = tid; q < 2 * G; q += NT) {
@@ -1065,17 +1088,28 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                 auto row_of = [&](int i) -> const V * {       // 3D: lines of the block, clamped to it
                     return A + (size_t)(i < cnt ? sline(jy, jz) : PY + 1) * pitch + go;
                 };
-                const V *row = D3 ? row_of(0) : (MAT ? B : A) + (size_t)(SO + l0) * pitch + go;
+                V *const S = MAT ? B : A;
+                int om = (SO + l0) * pitch + go, od = om + pitch;        // 2D: this line, the next
+                const int odmax = (L + 2 * SO - 1) * pitch + go;
+                const V *row = D3 ? row_of(0) : S + om;
                 const V *rrow = A + (size_t)(H + l0) * pitch + go;       // r (Matern)
                 It up = ri_ld(row - pitch), mid = ri_ld(row), dn = ri_ld(row + pitch), fr = zz, bck = zz, rv = zz;
+                if constexpr (SH) up = PM::sub(up, mid);
                 if constexpr (D3) {
                     fr = ri_ld(row - PY * pitch);
                     bck = ri_ld(row + PY * pitch);
                 }
                 if constexpr (MAT) rv = ri_ld(rrow);
-                V l = __shfl_up_sync(0xffffffffu, mid.v[E - 1], 1), r = __shfl_down_sync(0xffffffffu, mid.v[0], 1);
-                if (lfix) l = row[-1];
-                if (rfix) r = row[E];
+                V l, r;
+                if constexpr (D3) {
+                    l = __shfl_up_sync(0xffffffffu, mid.v[E - 1], 1);
+                    r = __shfl_down_sync(0xffffffffu, mid.v[0], 1);
+                    if (lfix) l = row[-1];
+                    if (rfix) r = row[E];
+                } else {
+                    l = row[-1];
+                    r = row[E];
+                }
                 TmItem ta, td;
                 if constexpr (!MAT) tm_ld(ta, tma);
                 if (!MAT && d_tm) tm_ld(td, tmd);
@@ -1108,10 +1142,9 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         cc = PM::splat(k2);
                     }
                     const int jyc = jy, jzc = jz;
-                    const bool more = i + 1 < cnt;
                     It up2, mid2, dn2, fr2 = zz, bck2 = zz, rv2 = rv;
-                    V l2, r2;
-                    const V *nrow = row + pitch;
+                    V l2, r2, le = (V)0, re = (V)0;
+                    const V *nrow = nullptr;
                     if constexpr (D3) {
                         next_line(jy, jz);
                         nrow = row_of(i + 1);
@@ -1120,19 +1153,34 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         up2 = ri_ld(nrow - pitch);
                         fr2 = ri_ld(nrow - PY * pitch);
                         bck2 = ri_ld(nrow + PY * pitch);
+                        const bool more = i + 1 < cnt;
+                        l2 = __shfl_up_sync(0xffffffffu, mid2.v[E - 1], 1);
+                        r2 = __shfl_down_sync(0xffffffffu, mid2.v[0], 1);
+                        if (lfix && more) l2 = nrow[-1];
+                        if (rfix && more) r2 = nrow[E];
                     } else {
                         ++jy;
-                        up2 = mid;
+                        om = od;
+                        od = min(od + pitch, odmax);      // past the run's end: not used
                         mid2 = dn;
-                        dn2 = dn;
-                        if (more) dn2 = ri_ld(row + 2 * pitch);
+                        dn2 = ri_ld(S + od);
+                        l2 = __shfl_up_sync(0xffffffffu, mid2.v[E - 1], 1);
+                        r2 = __shfl_down_sync(0xffffffffu, mid2.v[0], 1);
+                        if (lfix) le = S[om - 1];
+                        if (rfix) re = S[om + E];
+                        if constexpr (MAT) {
+                            rrow += pitch;
+                            rv2 = ri_ld(rrow);
+                        }
                     }
-                    if (MAT && more) rv2 = ri_ld(rrow + pitch);
-                    l2 = __shfl_up_sync(0xffffffffu, mid2.v[E - 1], 1);
-                    r2 = __shfl_down_sync(0xffffffffu, mid2.v[0], 1);
-                    if (lfix && more) l2 = nrow[-1];
-                    if (rfix && more) r2 = nrow[E];
-                    It wv = res_level<V, NB>(cc, mid, l, r, dn, up, fr, bck);
+                    It wv;
+                    if constexpr (SH) {
+                        up2 = PM::sub(mid, dn);
+                        wv = res_level_sh(cc, mid, l, r, up2, up);
+                    } else {
+                        if constexpr (!D3) up2 = mid;
+                        wv = res_level<V, NB>(cc, mid, l, r, dn, up, fr, bck);
+                    }
                     clip(wv);
                     if constexpr (MAT) clip(rv);   // a torus ghost inside a partial item is not r
                     tm_st<V>(tmw + 4u * i, wv);
@@ -1160,8 +1208,10 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                                 send(3, 2 * (bk.z_begin(zn + 1) - bk.z_begin(zn)) + jyc, wv);
                             }
                         } else {
-                            if (jyc < H && bk.has[0]) send(0, H + jyc, wv);
-                            if (jyc >= L - H && bk.has[1]) send(1, jyc - (L - H), wv);
+                            if (jyc < H || jyc >= L - H) {
+                                if (jyc < H && bk.has[0]) send(0, H + jyc, wv);
+                                if (jyc >= L - H && bk.has[1]) send(1, jyc - (L - H), wv);
+                            }
                         }
                     }
                     vb >>= E;
@@ -1171,10 +1221,9 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     fr = fr2;
                     bck = bck2;
                     rv = rv2;
-                    l = l2;
-                    r = r2;
+                    l = !D3 && lfix ? le : l2;
+                    r = !D3 && rfix ? re : r2;
                     row = nrow;
-                    rrow += pitch;
                 }
                 if constexpr (!MAT) {
                     if (d_tm) tm_wait(ta, td);     // the load past the last item
