@@ -75,30 +75,34 @@ bool res_geometry(const Solve &s, bool keep_x0, int yw, int nt, int M, bool clus
 // 48 x 40 to 1024 x 1024 and 40^3 to 128^3 lattices within about 20 %.
 double res_clocks(const Solve &s, const ResPlan &p, bool keep_x0) {
     const bool f64 = s.precision == 0;
-    double item = s.op.kind == KIND_2D13_SQ ? (f64 ? 560 : 80) : s.op.kind == KIND_3D7 ? (f64 ? 470 : 110) : (f64 ? 390 : 62);
-    if (keep_x0) item += f64 ? (s.op.kind == KIND_2D13_SQ ? 120 : 60) : 18;
-    if (s.op.kind != KIND_2D13_SQ && s.op.field_d) item += f64 ? 10 : 15;
-    if (!f64 && p.nt == 256) item *= 1.3;      // half the warps to cover the latencies
+    double item = s.op.kind == KIND_2D13_SQ ? (f64 ? 525 : 60) : s.op.kind == KIND_3D7 ? (f64 ? 470 : 96) : (f64 ? 390 : 42);
+    if (keep_x0) item += f64 ? (s.op.kind == KIND_2D13_SQ ? 120 : 60) : (s.op.kind == KIND_3D7 ? 16 : 8);
+    if (s.op.kind != KIND_2D13_SQ && s.op.field_d) item += f64 ? 10 : (s.op.kind == KIND_3D7 ? 13 : 2);
+    if (!f64 && p.nt == 256) item *= 1.25;      // half the warps to cover the latencies
     const double warps = p.nt / 32.0, halo = (double)p.slots * p.G / p.nt;
     const double active = (p.G * p.nseg + 31) / 32;            // warps that own lines
     const double work = item * (active * p.cmax + 0.35 * warps * halo);
-    const double fixed = p.clustered ? 5000 + (f64 ? 330 : 170) * warps : (f64 ? 8000 + 330 * warps : 8500 + 60 * warps) + 50.0 * p.M;
+    const double fixed = p.clustered ? (f64 ? 4800 + 210 * warps + 50.0 * p.M : 1600 + 255 * warps + 300.0 * p.M)
+                                     : (f64 ? 7400 + 500 * warps + 50.0 * p.M : 10800 + 150 * warps);
     return work + fixed;
 }
 
-// Clocks of one streamed pass over the same vectors (grid engine): its launches and end of
-// pass, and its state words at the rate measured for the kind (FP32: bytes; FP64: 13 or 18
-// FP64 instructions a vertex and column).
+// Clocks of one streamed pass over the same vectors (grid engine).  FP64: its launches and end
+// of pass, or 13 or 18 FP64 instructions a vertex and column.  FP32: fitted to passes of 400^2
+// to 1200^2 and 48^3 to 80^3 (18 to 45 columns) within 10 %, an intercept by kind and the state
+// words at a rate.  Measured at the line, stream against resident, us: Matern 520^2 30.0 / 25.9,
+// 640^2 36.6 / 39.3; 5-point 600^2 32.8 / 24.4, 900^2 48.7 / 51.7; 3D field 64^3 94 / 72, 80^3
+// 135 / 200.
 double stream_clocks(const Solve &s, int ncolours, bool keep_x0) {
     const double vc = (double)s.op.n * ncolours;
-    const double launch = 15.0 * 1950;
+    const bool mat = s.op.kind == KIND_2D13_SQ, d3 = s.op.kind == KIND_3D7;
     if (s.precision == 0) {
-        const double instr = s.op.kind == KIND_2D13_SQ ? 18 : s.op.kind == KIND_3D7 ? 15 : 13;
-        return std::max(launch, vc * (instr + (keep_x0 ? 3 : 0)) / (152 * 1.5));
+        const double instr = mat ? 18 : d3 ? 15 : 13;
+        return std::max(15.0 * 1950, vc * (instr + (keep_x0 ? 3 : 0)) / (152 * 1.5));
     }
-    const int words = (s.op.kind == KIND_2D13_SQ && keep_x0 ? 8 : 4) + (keep_x0 && s.op.kind != KIND_2D13_SQ ? 2 : 0);
-    const double rate = s.op.kind == KIND_3D7 ? 2350 : 3000;    // bytes a clock
-    return 0.5 * launch + vc * words * 4 / rate;
+    const int words = (mat && keep_x0 ? 8 : 4) + (keep_x0 && !mat ? 2 : 0);
+    const double rate = d3 ? 2600 : mat ? (keep_x0 ? 2640 : 3000) : 4200;    // bytes a clock
+    return (d3 ? 60000 : mat && keep_x0 ? 24000 : 32000) + vc * words * 4 / rate;
 }
 
 template <class F>
@@ -187,7 +191,7 @@ static int resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
     }
     cudaGetLastError();
     // contexts the grid engine would run: only where the passes would take longer
-    if (streams && best >= stream_clocks(s, ncolours, keep_x0)) return 1;
+    if (streams && best >= (s.precision == 0 ? 1.0 : 0.9) * stream_clocks(s, ncolours, keep_x0)) return 1;
     return best < 1e300 ? 0 : 1;
 }
 

@@ -124,50 +124,82 @@ __device__ __forceinline__ ResItem<float> res_level_sh(const ResItem<float> &c, 
     return M::fma(c, m, M::add(h, M::sub(d, dp)));
 }
 
-// Sum eight values over the warp: on return lane l holds the total of value l >> 2.
-// Halving exchange: 4 + 2 + 1 + 1 + 1 additions instead of 8 x 5 (FP64 adds are narrow).
-template <typename A>
-__device__ __forceinline__ A warp_sum8(const A (&v)[8]) {
-    const int lane = threadIdx.x & 31;
-    A a[4], b[2], c;
-    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+// Sums of K values over the lanes with equal lane % NG by halving exchange: each step a lane
+// sends one half of its values and adds to the other, (K + 1) / 2 left.  A lane ends with the
+// totals of values [at, at + N) (those below K) in v[0 .. N), N = group_sum_left(K, NG).
+__host__ __device__ constexpr int group_sum_left(int K, int NG) {
+    for (int o = 16; o >= NG; o /= 2) K = (K + 1) / 2;
+    return K;
+}
+template <int NG, int O = 16, typename A, int K, int R>
+__device__ __forceinline__ void group_sum(const A (&v)[K], A (&out)[R], int &at, int &end) {
+    constexpr int N = (K + 1) / 2;
+    const bool up = threadIdx.x & O;
+    A w[N];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const A keep = h4 ? v[4 + k] : v[k], send = h4 ? v[k] : v[4 + k];
-        a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    for (int k = 0; k < N; ++k) {
+        const A hi = N + k < K ? v[N + k < K ? N + k : 0] : (A)0;
+        w[k] = (up ? hi : v[k]) + __shfl_xor_sync(0xffffffffu, up ? v[k] : hi, O);
     }
+    if (up) at += N;
+    else end = min(end, at + N);
+    if constexpr (O == NG) {
+        static_assert(N == R, "values left");
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const A keep = h3 ? a[2 + k] : a[k], send = h3 ? a[k] : a[2 + k];
-        b[k] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+        for (int k = 0; k < N; ++k) out[k] = w[k];
+    } else {
+        group_sum<NG, O / 2>(w, out, at, end);
     }
-    {
-        const A keep = h2 ? b[1] : b[0], send = h2 ? b[0] : b[1];
-        c = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    c += __shfl_xor_sync(0xffffffffu, c, 2);
-    c += __shfl_xor_sync(0xffffffffu, c, 1);
-    return c;
 }
 
-// Sum four values over the warp: lane l gets the total of value l >> 3.
-__device__ __forceinline__ double warp_sum4(const double (&v)[4]) {
-    const int lane = threadIdx.x & 31;
-    double a[2], b;
-    const bool h4 = lane & 16, h3 = lane & 8;
+// sum over the warp's lanes below W, the same in all of them
+template <int W = 32>
+__device__ __forceinline__ double lane_sum(double v) {
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        const double keep = h4 ? v[2 + k] : v[k], send = h4 ? v[k] : v[2 + k];
-        a[k] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// ---- the scalar chain of an iteration, every step of which the vector warps wait for.
+// FP64 compares and quotients cost as much as several adds here, so signs are read from the
+// bits and the reciprocals are formed from the hardware's 20-bit estimate by one third-order
+// Householder step, y += y (e + e^2) with e = 1 - a y: 2^-60 before its last rounding.
+__device__ __forceinline__ bool res_positive(double v) {           // v > 0
+    const long long b = __double_as_longlong(v);
+    return b > 0 && b <= 0x7ff0000000000000ll;
+}
+__device__ __forceinline__ bool res_plain(double v) {              // 2^-900 < v < 2^900
+    return (unsigned)((__double2hiint(v) >> 20) - 123) < 1800u;
+}
+__device__ __forceinline__ double res_recip(double a) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+    const double e = fma(-a, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// alpha, beta and the predicted |r_{k+1}|^2 of one iteration from its dots; all lanes alike.
+// Returns a DEV_ code or 0.
+__device__ __forceinline__ int res_scalars(double rr, double pw, double rw, double ww, double &na, double &nb, double &rho) {
+    const int lane = threadIdx.x & 31;
+    na = nb = 0.0;
+    rho = rr;
+    if (!res_positive(pw)) return isfinite(pw) ? DEV_NOTSPD : DEV_NUMERIC;
+    const double m2 = -2.0 * rw;
+    double irr;
+    if (res_plain(rr) && res_plain(pw)) {
+        // lane 1 takes 1 / rr while lane 0 takes 1 / pw
+        const double y = res_recip(lane & 1 ? rr : pw);
+        na = rr * __shfl_sync(0xffffffffu, y, 0);
+        irr = __shfl_sync(0xffffffffu, y, 1);
+    } else {
+        const double quo = (lane & 1 ? 1.0 : rr) / (lane & 1 ? rr : pw);
+        na = __shfl_sync(0xffffffffu, quo, 0);
+        irr = __shfl_sync(0xffffffffu, quo, 1);
     }
-    {
-        const double keep = h3 ? a[1] : a[0], send = h3 ? a[0] : a[1];
-        b = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    b += __shfl_xor_sync(0xffffffffu, b, 4);
-    b += __shfl_xor_sync(0xffffffffu, b, 2);
-    b += __shfl_xor_sync(0xffffffffu, b, 1);
-    return b;
+    const double x = fma(na, fma(na, ww, m2), rr);
+    rho = res_positive(x) ? x : 0.0;
+    nb = res_positive(rr) ? rho * irr : 0.0;
+    return 0;
 }
 
 // 16-byte record {value, tag}: one 128-bit access each way, so that a reader that sees the
@@ -366,9 +398,10 @@ struct ResCtl {
     uint32_t tm;                 // tensor memory base
     volatile int done;           // queue entries processed when the last column's shifts converged
     volatile int head, tail;     // queue entries posted, processed
-    int pad0;
+    int bad;                     // a vector warp's wait ran out
     uint64_t bar[2];             // exchange barriers by iteration parity
     double dflag[2];             // done flag of the team's first CTA, by parity
+    double tot[4];               // the team's rr, pw, rw, ww
     struct Entry {
         double alpha, beta, rho, vr;
         int code, pad;
@@ -527,6 +560,8 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
     const int lane = threadIdx.x & 31, M = pl.M;
     const bool clustered = pl.clustered;
     const double ds = s.precision == 0 ? s.op.scale : (double)s.op.scale_f;
+    const double ds2 = ds * ds;
+    const bool scaled = ds != 1.0;
     ulonglong2 *const rec = clustered ? nullptr : ar.rec + (size_t)team * 2 * M * 8;
     unsigned long long tick = 0;
     int head = 0;
@@ -547,90 +582,38 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
         for (int it = 0;; ++it, ++tick) {
             const int par = (int)(tick & 1);
             const double *pp = part + (size_t)par * RES_NDOT * NP;
-            double v4[4] = {0.0, 0.0, 0.0, 0.0}, vr_sum = 0.0;
-            int stop = 0;
+            const unsigned long long tag = tick + 1;
+            ulonglong2 *const rp = rec + (size_t)par * M * 8;
+            double fl = 0.0;
             bool ok = true;
+            if (m == 0) fl = finished(base) ? 1.0 : 0.0;
             if (clustered) {
-                if (m == 0) {
-                    const int fl = finished(base);
-                    if (lane < M)
-                        st_async(mapa(smem_u32(&ctl->dflag[par]), lane), mapa(smem_u32(&ctl->bar[par]), lane), (double)fl);
-                }
-                ok = res_bar_wait(smem_u32(&ctl->bar[par]), (unsigned)(tick >> 1) & 1u);
-                __syncwarp();
-                if (lane == 0) mbar_arrive_tx(&ctl->bar[par], in_bytes);      // armed for tick + 2
-                for (int q = lane; q < NP; q += 32)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) v4[k] += pp[(size_t)k * NP + q];
-                stop = ctl->dflag[par] != 0.0;
+                if (m == 0 && lane < M)
+                    st_async(mapa(smem_u32(&ctl->dflag[par]), lane), mapa(smem_u32(&ctl->bar[par]), lane), fl);
             } else {
-                bar_sync(3, NT + 32);
-                double loc[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) loc[k] = k < RES_NDOT && lane < NW ? pp[(size_t)k * NP + lane] : 0.0;
-                __threadfence();
-                const double mysum = warp_sum8<double>(loc);
-                const int fin = m == 0 ? finished(base) : 0;
-                const unsigned long long tag = tick + 1;
-                ulonglong2 *rp = rec + (size_t)par * M * 8;
-                const int k = lane >> 2;
-                if ((lane & 3) == 0 && k < RES_NDOT + 1)
-                    rec_st(rp + (size_t)m * 8 + k, k == RES_NDOT ? (double)fin : mysum, tag);
-                // four CTAs' records a lane, all loads in flight together until every tag is there
-                const int nk = m == 0 ? 5 : 4;
-                uint64_t t0 = 0;
-                for (int q0 = lane; q0 < M; q0 += 64) {
-                    double v[2][RES_NDOT];
-                    for (unsigned spin = 0;; ++spin) {
-                        bool got = true;
-#pragma unroll
-                        for (int b = 0; b < 2; ++b) {
-                            const int q = q0 + 32 * b;
-#pragma unroll
-                            for (int kk = 0; kk < RES_NDOT; ++kk) {
-                                v[b][kk] = 0.0;
-                                if (q < M && kk < nk) got &= rec_ld(rp + (size_t)q * 8 + kk, tag, v[b][kk]);
-                            }
-                        }
-                        if (got) break;
-                        if ((spin & 255) == 255) {
-                            const uint64_t t = global_ns();
-                            if (t0 == 0) t0 = t;
-                            else if (t - t0 > 2000000000ull) { ok = false; break; }
-                        }
-                    }
-#pragma unroll
-                    for (int b = 0; b < 2; ++b) {
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk) v4[kk] += v[b][kk];
-                        vr_sum += v[b][4];
-                    }
-                }
-                double fl = 0.0;
-                ok = ok && rec_wait(rp + 5, tag, fl);
-                stop = fl != 0.0;
-                __threadfence();
+                if (m == 0 && lane == 0) rec_st(rp + 5, fl, tag);
+                ok = rec_wait(rp + 5, tag, fl);
             }
-            if (!__all_sync(0xffffffffu, ok)) {
+            bar_sync(3, 160);                 // the sums of vector warps 0 to 3
+            if (clustered) {
+                if (lane == 0) mbar_arrive_tx(&ctl->bar[par], in_bytes);      // armed for tick + 2
+                fl = ctl->dflag[par];
+            }
+            int stop = __double2hiint(fl) != 0;
+            if (!__all_sync(0xffffffffu, ok) || ctl->bad) {
                 set_status(s.status, DEV_TIMEOUT);
                 stop = 2;
             }
-            const double tot = warp_sum4(v4);
             // the levels ran unscaled: p.w and r.w carry one factor s, w.w two
-            const double rr = __shfl_sync(0xffffffffu, tot, 0), pw = ds * __shfl_sync(0xffffffffu, tot, 8);
-            const double rw = ds * __shfl_sync(0xffffffffu, tot, 16), ww = ds * ds * __shfl_sync(0xffffffffu, tot, 24);
-            double na = 0.0, nb = 0.0, rho = rr;
-            int ncode = 0;
-            if (!(pw > 0.0)) {
-                ncode = isfinite(pw) ? DEV_NOTSPD : DEV_NUMERIC;
-            } else {
-                // lane 1 takes 1 / rr while lane 0 takes rr / pw
-                const double quo = (lane & 1 ? 1.0 : rr) / (lane & 1 ? rr : pw);
-                na = __shfl_sync(0xffffffffu, quo, 0);
-                const double irr = __shfl_sync(0xffffffffu, quo, 1);
-                rho = fmax(fma(na, fma(na, ww, -2.0 * rw), rr), 0.0);
-                nb = rr > 0.0 ? rho * irr : 0.0;
+            const double rr = ctl->tot[0];
+            double pw = ctl->tot[1], rw = ctl->tot[2], ww = ctl->tot[3];
+            if (scaled) {
+                pw *= ds;
+                rw *= ds;
+                ww *= ds2;
             }
+            double na, nb, rho;
+            const int ncode = res_scalars(rr, pw, rw, ww, na, nb, rho);
             if (lane == 0) {
                 ctl->alpha = na;
                 ctl->beta = nb;
@@ -641,10 +624,16 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
             if (m == 0) {
                 // iteration it - 1 to the shift warp: its v^T r_{it} is this iteration's v.r
                 if (it > 0) {
-                    if (clustered)
-                        for (int q = lane; q < NP; q += 32) vr_sum += pp[(size_t)4 * NP + q];
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) vr_sum += __shfl_xor_sync(0xffffffffu, vr_sum, o);
+                    double vr_sum = 0.0;
+                    for (int q = lane; q < (clustered ? NP : M); q += 32) {
+                        double v = 0.0;
+                        if (clustered) v = pp[(size_t)4 * NP + q];
+                        else ok = rec_wait(rp + (size_t)q * 8 + 4, tag, v) && ok;
+                        vr_sum += v;
+                    }
+                    __syncwarp();
+                    vr_sum = lane_sum(vr_sum);
+                    if (!__all_sync(0xffffffffu, ok)) set_status(s.status, DEV_TIMEOUT);
                     while (head - ctl->tail >= 4) {}
                     if (lane == 0) {
                         ResCtl::Entry &e = ctl->q[head & 3];
@@ -1236,25 +1225,86 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         bar_arrive(3, NT + 32);
                     }
                 } else {
-                V flat[8] = {(V)0, (V)0, (V)0, (V)0, d_vr, (V)0, (V)0, (V)0};
+                V flat[RES_NDOT] = {d_rr.v[0], d_pw.v[0], d_rw.v[0], d_ww.v[0], d_vr}, sum[1];
 #pragma unroll
-                for (int e = 0; e < E; ++e) {
+                for (int e = 1; e < E; ++e) {
                     flat[0] += d_rr.v[e];
                     flat[1] += d_pw.v[e];
                     flat[2] += d_rw.v[e];
                     flat[3] += d_ww.v[e];
                 }
-                const double tot = (double)warp_sum8<V>(flat);
-                const int k = lane >> 2;
+                int k = 0, end = RES_NDOT;                // four lanes hold dot k, where k < end
+                group_sum<4>(flat, sum, k, end);
+#pragma unroll
+                for (int o = 2; o > 0; o >>= 1) sum[0] += __shfl_xor_sync(0xffffffffu, sum[0], o);
+                const double tot = (double)sum[0];
+                // One warp adds FP64 numbers at a quarter of the SM's rate (64 clocks an
+                // instruction whatever its lanes), so the team's sums are formed by four or five
+                // vector warps, one a dot, and the scalar warp starts from the totals.
                 if (clustered) {
-                    if (k < RES_NDOT) {
+                    if (k < end) {
                         const uint32_t slot = smem_u32(part + (size_t)(par * RES_NDOT + k) * NP + m * NW + wid);
                         for (int q = lane & 3; q < M; q += 4) st_async(mapa(slot, q), mapa(bar_addr, q), tot);
                     }
+                    if (wid < 4) {
+                        if (!res_bar_wait(bar_addr, (unsigned)(tick >> 1) & 1u)) ctl->bad = 1;
+                        const double *pp = part + (size_t)(par * RES_NDOT + wid) * NP;
+                        double a = lane < NP ? pp[lane] : 0.0;
+                        for (int q = lane + 32; q < NP; q += 32) a += pp[q];
+                        __syncwarp();
+                        a = lane_sum(a);
+                        if (lane == 0) ctl->tot[wid] = a;
+                        bar_arrive(3, 160);
+                    }
                 } else {
-                    if (k < RES_NDOT && (lane & 3) == 0) part[(size_t)(par * RES_NDOT + k) * NP + wid] = tot;
-                    __threadfence();       // boundary rows before the record of the scalar warp
-                    bar_arrive(3, NT + 32);
+                    if (k < end && (lane & 3) == 0) part[(size_t)(par * RES_NDOT + k) * NP + wid] = tot;
+                    // every thread's boundary rows on their way: a fence by the publishers alone
+                    // orders them too, but waits for all of them at the end (FP64 Matern 200 x
+                    // 150, four vectors: 19.9 against 18.8 ms)
+                    __threadfence();
+                    bar_sync(1, NT);
+                    const unsigned long long tag = tick + 1;
+                    ulonglong2 *const rp = ar.rec + ((size_t)team * 2 + par) * M * 8;
+                    if (wid < RES_NDOT) {
+                        const double a = lane_sum<NW>(lane < NW ? part[(size_t)(par * RES_NDOT + wid) * NP + lane] : 0.0);
+                        __threadfence();
+                        if (lane == 0) rec_st(rp + (size_t)m * 8 + wid, a, tag);
+                    }
+                    if (wid < 4) {
+                        bool ok = true;
+                        double a = 0.0;
+                        for (int q0 = lane; q0 < M; q0 += 128) {      // four records a lane in flight
+                            double v[4];
+                            uint64_t t0 = 0;
+                            for (unsigned spin = 0;; ++spin) {
+                                bool got = true;
+#pragma unroll
+                                for (int b = 0; b < 4; ++b) {
+                                    v[b] = 0.0;
+                                    if (q0 + 32 * b < M) got &= rec_ld(rp + (size_t)(q0 + 32 * b) * 8 + wid, tag, v[b]);
+                                }
+                                if (got) break;
+                                if ((spin & 255) == 255) {
+                                    const uint64_t t = global_ns();
+                                    if (t0 == 0) t0 = t;
+                                    else if (t - t0 > 2000000000ull) {
+                                        ok = false;
+                                        break;
+                                    }
+                                }
+                            }
+                            a = q0 == lane ? v[0] : a + v[0];
+#pragma unroll
+                            for (int b = 1; b < 4; ++b)
+                                if (q0 - lane + 32 * b < M) a += v[b];
+                        }
+                        __syncwarp();
+                        if (!ok) ctl->bad = 1;
+                        a = lane_sum(a);
+                        if (lane == 0) ctl->tot[wid] = a;
+                        __threadfence();     // the neighbours' boundary rows after their records
+                        bar_arrive(3, 160);
+                    }
                 }
                 }
             }
@@ -1351,6 +1401,7 @@ __device__ __forceinline__ void resident_body(const Solve &s, const ResPlan &pl,
         if ((threadIdx.x & 31) == 0) {
             ctl->done = 0;
             ctl->head = ctl->tail = 0;
+            ctl->bad = 0;
             if (pl.clustered) {
                 mbar_init(&ctl->bar[0], 1);
                 mbar_init(&ctl->bar[1], 1);

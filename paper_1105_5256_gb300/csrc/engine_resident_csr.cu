@@ -2,6 +2,7 @@
 #include "engine_resident_csr.cuh"
 
 #include <algorithm>
+#include <cmath>
 #include <atomic>
 #include <thread>
 
@@ -59,9 +60,12 @@ int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int
         return 1;
     }
     const double avg = (double)rowptr[n] / (double)n;
-    // Cost of a plan in clocks.  FP64: 19 a warp instruction (entries, r, p, dots); FP32: the
-    // shared-memory wavefronts of the product (about nine an entry and warp) and the updates.
-    // The exchange has two hops (partials to the vector's owner, alpha and beta back).
+    // Cost of a plan in clocks, by the warps' rows and external columns.  FP64: 19 a warp
+    // instruction (entries, r, p, dots); FP32: the shared-memory wavefronts of the product
+    // (about nine an entry and warp) and the updates.  The exchange has two hops (partials to
+    // the vector's owner, alpha and beta back); fewer teams of more vectors make it shorter
+    // (13K-vertex second-order mesh, FP32, 31 vectors: T 4, 8 teams 11.5, T 8, 4 teams 10.2 us;
+    // 3000-vertex graph, FP64, 15: T 2, 8 teams 10.3, T 4, 4 teams 9.2).
     double best = 1e300;
     CsrPlan bp{};
     std::vector<int32_t> seen(n, -1), tmp;
@@ -97,10 +101,10 @@ int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int
             if (3 * p.items_own + p.items_ext > room || p.own_max + p.ext_max > 65000) continue;
             if (csr_smem(p, word, nshift).bytes > 227 * 1024) continue;
             auto clocks = [&](const CsrPlan &q) {
-                const double warps = nt / 32.0;
-                if (precision == 0)
-                    return 17000 + 20.0 * M + warps * (q.items_own * (42 * avg + 310) + q.items_ext * 80.0 + 330);
-                return 17000 + 20.0 * M + warps * (q.items_own * (10.5 * avg + 60) + q.items_ext * 40.0);
+                const double lanes = q.T / E / 32.0, own = std::ceil(q.own_max * lanes), ex = std::ceil(q.ext_max * lanes);
+                const double fixed = (precision == 0 ? 14500 : 13000) + 20.0 * M + 400.0 * J;
+                if (precision == 0) return fixed + own * (42 * avg + 310) + ex * 80.0 + nt / 32.0 * 250;
+                return fixed + own * (9 * avg + 60) + ex * 22.0;
             };
             // whole rounds of J T vectors, then the remainder on the fewest vectors a team that hold it
             const int rest = ncolours % (J * T);

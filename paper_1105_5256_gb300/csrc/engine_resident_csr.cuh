@@ -32,43 +32,17 @@ struct CsrCtl {
     int stop;                    // 1: every vector of the group is finished, 2: a wait ran out
     uint32_t tm;
     volatile int done, head, tail;
-    int pad;
+    int bad;                     // a vector warp's wait ran out
     ResCtl::Entry q[4];
     double alpha[RES_CSR_T], beta[RES_CSR_T];
+    double tot[4];               // rr, pw, rw, ww of the vector this CTA owns
 };
 static_assert(sizeof(CsrCtl) <= RES_CSR_CTL_BYTES, "control block");
-
-// sums of the K values over the warp's lanes with equal lane % NG; on return lane g < NG has
-// the totals of group g in v
-template <typename A, int K, int NG>
-__device__ __forceinline__ void group_sum(A (&v)[K]) {
-#pragma unroll
-    for (int o = 16; o >= NG; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < K; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-}
-
-// FP64, one group: K <= 16 values over the 32 lanes by halving exchange; lane l ends with
-// the total of value l >> 1
-__device__ __forceinline__ double warp_sum16(const double (&v)[16]) {
-    const int lane = threadIdx.x & 31;
-    double a[8], b[4], c[2], d;
-    const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) a[k] = (h4 ? v[8 + k] : v[k]) + __shfl_xor_sync(0xffffffffu, h4 ? v[k] : v[8 + k], 16);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) b[k] = (h3 ? a[4 + k] : a[k]) + __shfl_xor_sync(0xffffffffu, h3 ? a[k] : a[4 + k], 8);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) c[k] = (h2 ? b[2 + k] : b[k]) + __shfl_xor_sync(0xffffffffu, h2 ? b[k] : b[2 + k], 4);
-    d = (h1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h1 ? c[0] : c[1], 2);
-    return d + __shfl_xor_sync(0xffffffffu, d, 1);
-}
 
 // ------------------------------------------------------------------ scalar warp
 template <int NT>
 __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, const ResArgs &ar, int team, int m,
-                                             CsrCtl *ctl, const double *part) {
-    constexpr int NW = NT / 32;
+                                             CsrCtl *ctl) {
     const int lane = threadIdx.x & 31, M = pl.M, T = pl.T;
     // records: partials [2][T][M][6], then scalars [2][T][4]
     ulonglong2 *const rec = ar.rec + (size_t)team * pl.rec_team;
@@ -92,52 +66,12 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
             const int par = (int)(tick & 1);
             const unsigned long long tag = tick + 1;
             bool ok = true;
-            bar_sync(3, NT + 32);
-            __threadfence();
-            // this CTA's partials of every vector, to the vector's owner
-            for (int v = lane; v < 5 * T; v += 32) {
-                const double *pp = part + ((size_t)par * 5 * T + v) * NW;
-                double a[4] = {0.0, 0.0, 0.0, 0.0};
-                for (int w = 0; w < NW; w += 4)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) a[k] += pp[w + k];
-                const int t = v / 5, k = v - 5 * t;
-                rec_st(rec + (((size_t)par * T + t) * M + m) * 6 + k, (a[0] + a[1]) + (a[2] + a[3]), tag);
-            }
-            double vr_sum = 0.0;
             double na = 0.0, nb = 0.0, rho = 0.0;
             int ncode = 0, fin = 1;
+            const ulonglong2 *const rp = rec + ((size_t)par * T + m) * M * 6;      // (owner)
             if (owner) {
-                double v4[4] = {0.0, 0.0, 0.0, 0.0};
-                const ulonglong2 *rp = rec + ((size_t)par * T + m) * M * 6;
-                uint64_t t0 = 0;
-                for (int q0 = lane; q0 < M; q0 += 64) {
-                    double v[2][RES_NDOT];
-                    for (unsigned spin = 0;; ++spin) {
-                        bool got = true;
-#pragma unroll
-                        for (int b = 0; b < 2; ++b) {
-                            const int q = q0 + 32 * b;
-#pragma unroll
-                            for (int k = 0; k < RES_NDOT; ++k) {
-                                v[b][k] = 0.0;
-                                if (q < M) got &= rec_ld(rp + (size_t)q * 6 + k, tag, v[b][k]);
-                            }
-                        }
-                        if (got) break;
-                        if ((spin & 255) == 255 && timed(t0)) {
-                            ok = false;
-                            break;
-                        }
-                    }
-#pragma unroll
-                    for (int b = 0; b < 2; ++b) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) v4[k] += v[b][k];
-                        vr_sum += v[b][4];
-                    }
-                }
-                __syncwarp();
+                bar_sync(3, 160);             // the sums of vector warps 0 to 3
+                ok = !ctl->bad;
                 if (live) {
                     // stop a fixed two iterations after the shift warp's verdict
                     while (ctl->tail < head - 1) {}
@@ -146,22 +80,9 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
                     if (d > base && d <= head - 1) live = false;
                 }
                 fin = !live;
-                const double tot = warp_sum4(v4);
-                const double rr = __shfl_sync(0xffffffffu, tot, 0), pw = __shfl_sync(0xffffffffu, tot, 8);
-                const double rw = __shfl_sync(0xffffffffu, tot, 16), ww = __shfl_sync(0xffffffffu, tot, 24);
+                const double rr = ctl->tot[0], pw = ctl->tot[1], rw = ctl->tot[2], ww = ctl->tot[3];
                 rho = rr;
-                if (live) {
-                    if (!(pw > 0.0)) {
-                        ncode = isfinite(pw) ? DEV_NOTSPD : DEV_NUMERIC;
-                    } else {
-                        // lane 1 takes 1 / rr while lane 0 takes rr / pw
-                        const double quo = (lane & 1 ? 1.0 : rr) / (lane & 1 ? rr : pw);
-                        na = __shfl_sync(0xffffffffu, quo, 0);
-                        const double irr = __shfl_sync(0xffffffffu, quo, 1);
-                        rho = fmax(fma(na, fma(na, ww, -2.0 * rw), rr), 0.0);
-                        nb = rr > 0.0 ? rho * irr : 0.0;
-                    }
-                }
+                if (live) ncode = res_scalars(rr, pw, rw, ww, na, nb, rho);
                 if (lane < 3) rec_st(rec2 + ((size_t)par * T + m) * 4 + lane, lane == 0 ? na : lane == 1 ? nb : (double)fin, tag);
             }
             // every vector's alpha, beta and finished flag
@@ -194,8 +115,15 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
             if (stop) break;
             if (live) {
                 if (it > 0) {        // iteration it - 1 to the shift warp
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) vr_sum += __shfl_xor_sync(0xffffffffu, vr_sum, o);
+                    double vr_sum = 0.0;
+                    for (int q = lane; q < M; q += 32) {
+                        double v = 0.0;
+                        ok = rec_wait(rp + (size_t)q * 6 + 4, tag, v) && ok;
+                        vr_sum += v;
+                    }
+                    __syncwarp();
+                    vr_sum = lane_sum(vr_sum);
+                    if (!__all_sync(0xffffffffu, ok)) set_status(s.status, DEV_TIMEOUT);
                     while (head - ctl->tail >= 4) {}
                     if (lane == 0) {
                         ResCtl::Entry &e = ctl->q[head & 3];
@@ -239,7 +167,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
     using It = ResItem<V>;
     using PM = PackMath<V, E>;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int T = pl.T;
+    const int T = pl.T, M = pl.M;
     const int r0 = pl.row0[m], own = pl.row0[m + 1] - r0, e0 = pl.ext0[m], ext = pl.ext0[m + 1] - e0;
     const int n = (int)s.op.n;
     double *const part = reinterpret_cast<double *>(smem + lay.part);
@@ -307,21 +235,29 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
             const It na = ri_ld(coef + g * E), be = ri_ld(coef + T + g * E), aa = ri_ld(coef + 2 * T + g * E);
             // ---- r, p (x) of own rows, r and p of external columns
             const V *wprev = wbuf + (size_t)(par ^ 1) * n * T;
-#pragma unroll 2
-            for (int i = 0; i < ie; ++i) {
-                const int q = i * RS + rs;
-                TmItem tr;
-                tm_ld(tr, tme + 4u * i);
-                It wv = zz, old = zz;
-                V *pp = P + ((size_t)(own + min(q, ext - 1)) * NG + g) * E;
-                if (q < ext) {
-                    if (it > 0) wv = ri_ldcg(wprev + ((size_t)pl.ext[e0 + q] * NG + g) * E);
-                    old = ri_ld(pp);
+            // four items at a time: their gathers from L2 are in flight together
+            constexpr int U = 4;
+            for (int i0 = 0; i0 < ie; i0 += U) {
+                It wv[U];
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                    const int q = (i0 + k) * RS + rs;
+                    wv[k] = zz;
+                    if (q < ext && it > 0) wv[k] = ri_ldcg(wprev + ((size_t)pl.ext[e0 + q] * NG + g) * E);
                 }
-                tm_wait(tr);
-                const It r = PM::fma(na, wv, tm_get<V>(tr));
-                tm_st<V>(tme + 4u * i, r);
-                if (q < ext) ri_st(pp, PM::fma(be, old, r));
+#pragma unroll
+                for (int k = 0; k < U; ++k) {
+                    const int i = i0 + k, q = i * RS + rs;
+                    if (i >= ie) break;
+                    TmItem tr;
+                    tm_ld(tr, tme + 4u * i);
+                    V *pp = P + ((size_t)(own + min(q, ext - 1)) * NG + g) * E;
+                    const It old = ri_ld(pp);
+                    tm_wait(tr);
+                    const It r = PM::fma(na, wv[k], tm_get<V>(tr));
+                    tm_st<V>(tme + 4u * i, r);
+                    if (q < ext) ri_st(pp, PM::fma(be, old, r));
+                }
             }
 #pragma unroll 2
             for (int i = 0; i < io; ++i) {
@@ -391,28 +327,68 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
                 __syncwarp();
             }
             tm_wait_st();
-            // partials [par][vector][dot][warp]
-            double *pp = part + (size_t)par * 5 * T * NW;
-            if constexpr (sizeof(V) == 8 && NG == 1) {
-                double v[16];
+            // partials [par][warp][vector][dot]
+            double *pp = part + ((size_t)par * NW + wid) * 5 * T;
+            constexpr int NS = group_sum_left(5 * E, NG);
+            V v[5 * E], sum[NS];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) v[k] = k < 10 ? d[k >> 1].v[k & 1] : 0.0;
-                const double t = warp_sum16(v);
-                const int k = lane >> 1;
-                if (k < 10 && !(lane & 1)) pp[(size_t)((k & 1) * 5 + (k >> 1)) * NW + wid] = t;
-            } else {
-                V v[5 * E];
+            for (int k = 0; k < 5 * E; ++k) v[k] = d[k % 5].v[k / 5];
+            int at = 0, end = 5 * E;
+            group_sum<NG>(v, sum, at, end);
 #pragma unroll
-                for (int k = 0; k < 5 * E; ++k) v[k] = d[k / E].v[k % E];
-                group_sum<V, 5 * E, NG>(v);
-                if (lane < NG) {
+            for (int k = 0; k < NS; ++k)
+                if (at + k < end) pp[g * 5 * E + at + k] = (double)sum[k];
+            bar_sync(1, NT);           // every warp's w and partials, before the fence of who publishes
+            const unsigned long long tag = tick + 1;
+            ulonglong2 *const rec = ar.rec + (size_t)team * pl.rec_team;
+            // one thread a sum, to the vector's owner; then the owner's vector's dots over the
+            // team, one a warp (see engine_resident.cuh: FP64 sums want warps of all SM quarters)
+            if (tid < 5 * T) {
+                const double *q = part + (size_t)par * NW * 5 * T + tid;
+                double a = q[0];
 #pragma unroll
-                    for (int k = 0; k < 5 * E; ++k)
-                        pp[(size_t)((lane * E + k % E) * 5 + k / E) * NW + wid] = (double)v[k];
-                }
+                for (int w = 1; w < NW; ++w) a += q[(size_t)w * 5 * T];
+                __threadfence();
+                const int t = tid / 5, k = tid - 5 * t;
+                rec_st(rec + (((size_t)par * T + t) * M + m) * 6 + k, a, tag);
             }
-            __threadfence();           // w before the records of the scalar warp
-            bar_arrive(3, NT + 32);
+            if (m < T && wid < 4) {
+                __syncwarp();
+                const ulonglong2 *rp = rec + ((size_t)par * T + m) * M * 6 + wid;
+                bool ok = true;
+                double a = 0.0;
+                for (int q0 = lane; q0 < M; q0 += 160) {         // five records a lane in flight
+                    double v[5];
+                    uint64_t t0 = 0;
+                    for (unsigned spin = 0;; ++spin) {
+                        bool got = true;
+#pragma unroll
+                        for (int b = 0; b < 5; ++b) {
+                            v[b] = 0.0;
+                            if (q0 + 32 * b < M) got &= rec_ld(rp + (size_t)(q0 + 32 * b) * 6, tag, v[b]);
+                        }
+                        if (got) break;
+                        if ((spin & 255) == 255) {
+                            const uint64_t t = global_ns();
+                            if (t0 == 0) t0 = t;
+                            else if (t - t0 > 2000000000ull) {
+                                ok = false;
+                                break;
+                            }
+                        }
+                    }
+                    a = q0 == lane ? v[0] : a + v[0];
+#pragma unroll
+                    for (int b = 1; b < 5; ++b)
+                        if (q0 - lane + 32 * b < M) a += v[b];
+                }
+                __syncwarp();
+                if (!ok) ctl->bad = 1;
+                a = lane_sum(a);
+                if (lane == 0) ctl->tot[wid] = a;
+                __threadfence();         // every CTA's w before the owner's alpha and beta
+                bar_arrive(3, 160);
+            }
             bar_sync(2, NT + 32);
             stop = ctl->stop;
             if (stop) break;
@@ -462,6 +438,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident_csr(const __grid_consta
         if ((threadIdx.x & 31) == 0) {
             ctl->done = 0;
             ctl->head = ctl->tail = 0;
+            ctl->bad = 0;
         }
         __syncwarp();
     }
@@ -469,7 +446,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident_csr(const __grid_consta
     if (wid < NW) {
         csr_vector_role<V, NG, NT>(s, pl, ar, team, m, smem, lay, ctl);
     } else if (wid == NW) {
-        csr_scalar_role<NT>(s, pl, ar, team, m, ctl, reinterpret_cast<const double *>(smem + lay.part));
+        csr_scalar_role<NT>(s, pl, ar, team, m, ctl);
     } else if (m < pl.T) {
         res_shift_role(s, pl.J * pl.T, ar.cb + team * pl.T + m, ar, ctl->q, &ctl->head, &ctl->tail, &ctl->done,
                        reinterpret_cast<double2 *>(smem + lay.shift));

@@ -56,7 +56,7 @@ __host__ __device__ inline ResSmem res_smem(const ResPlan &p, int word, int kind
 
 // ---- CSR (engine_resident_csr.cuh)
 constexpr int RES_CSR_T = 16;            // vectors of a team at most
-constexpr int RES_CSR_CTL_BYTES = 24 + 4 * 40 + 16 * RES_CSR_T + 8;
+constexpr int RES_CSR_CTL_BYTES = 24 + 4 * 40 + 16 * RES_CSR_T + 32 + 8;
 
 struct CsrSmem {
     size_t part, ctl, shift, val, col, row, colour, coef, p, bytes;
