@@ -12,17 +12,20 @@ namespace {
 // tensor memory, and a 64-bit mask of its own-colour vertices
 constexpr int RES_ITEMS = 16;
 
-template <typename V, int KIND, int NT, bool KX>
-const void *res_fn() {
-    return reinterpret_cast<const void *>(&k_resident<V, KIND, NT, KX, false>);
+template <typename V, int KIND>
+const void *res_fn(int nt, bool kx) {
+    if (kx)
+        return nt == 256 ? reinterpret_cast<const void *>(&k_resident<V, KIND, 256, true, false>)
+                         : reinterpret_cast<const void *>(&k_resident<V, KIND, 512, true, false>);
+    return nt == 256 ? reinterpret_cast<const void *>(&k_resident<V, KIND, 256, false, false>)
+                     : reinterpret_cast<const void *>(&k_resident<V, KIND, 512, false, false>);
 }
 
 template <typename V>
 const void *res_fn_for(int kind, int nt, bool kx) {
-    if (kind == KIND_2D5) return nt == 256 ? res_fn<V, KIND_2D5, 256, false>() : res_fn<V, KIND_2D5, 512, false>();
-    if (kind == KIND_3D7) return nt == 256 ? res_fn<V, KIND_3D7, 256, false>() : res_fn<V, KIND_3D7, 512, false>();
-    if (kx) return nt == 256 ? res_fn<V, KIND_2D13_SQ, 256, true>() : res_fn<V, KIND_2D13_SQ, 512, true>();
-    return nt == 256 ? res_fn<V, KIND_2D13_SQ, 256, false>() : res_fn<V, KIND_2D13_SQ, 512, false>();
+    if (kind == KIND_2D5) return res_fn<V, KIND_2D5>(nt, kx);
+    if (kind == KIND_3D7) return res_fn<V, KIND_3D7>(nt, kx);
+    return res_fn<V, KIND_2D13_SQ>(nt, kx);
 }
 
 const void *res_kernel(const Solve &s, int nt, bool keep_x0) {

@@ -9,7 +9,9 @@
 //                          w = Q p, x (when kept) and a kappa^2 field's diagonal private
 //   Matern kind s Q1^2     r (two halo lines) and u = Q1 p (one) in shared memory:
 //                          u_k = Q1 r_k + beta u_{k-1}, w = s Q1 u, p.w = s |u|^2;
-//                          w private, and with x kept p and x
+//                          w private.  With x kept, p (two halo lines) and u = Q1 p formed
+//                          from it, r, w and x private: with u by its own recurrence w
+//                          drifts from Q p, and FP32 x was two to nine times less exact
 //
 // Private vectors (read and written only by the thread that owns the vertex) live in tensor
 // memory: 128 words a thread, addressed by a loop index (registers would need the loop
@@ -35,14 +37,15 @@
 // iteration's measured v.r; a converged vector is found an iteration or two late, and the
 // iterations past its last are discarded (counts and projections are unaffected).
 //
-// Bound by what the SMs issue (FP32: about 80 instructions a 16-byte item and level, 16
-// warps an SM) or by their FP64 units (19 clocks a warp instruction), plus one exchange of
-// 2.5 to 5 us an iteration; the state costs no DRAM or L2 traffic at all.  Measured a CG
-// iteration over all vectors (before: the streaming or the one-CTA engine): 48 x 40
-// Matern FP64, 52 vectors, with x 63 -> 9.5 us; 128^2 5-point FP64, 18, with x 143 -> 13.5;
-// 300 x 200 Matern FP32, 19, with x 22.6 -> 7.5; 500 x 333 torus field FP32, 26, with x
-// 29.6 -> 18.5; 512 x 384 Matern FP64, 18 (FP64 units busy in both) 137 -> 114.  Large FP32
-// problems stay with the lean passes: 1024^2 Matern, 18 vectors: 68 us here, 58 streamed.
+// Bound by what the SMs issue (FP32: about 45 to 65 instructions a 16-byte item and level, 16
+// warps an SM) or by their FP64 units (19 clocks a warp instruction), plus one exchange of 2
+// to 4.5 us an iteration, most of it dependent FP64 instructions; the state costs no DRAM or
+// L2 traffic at all.  Measured a CG iteration over all vectors (before: the streaming or the
+// one-CTA engine): 48 x 40 Matern FP64, 52 vectors, with x 63 -> 9.2 us; 128^2 5-point FP64,
+// 18, with x 143 -> 13.5; 300 x 200 Matern FP32, 19, with x 22.6 -> 8.0; 500 x 333 torus
+// field FP32, 26, with x 29.6 -> 16; 512 x 384 Matern FP64, 18 (FP64 units busy in both) 137
+// -> 114.  Large FP32 problems stay with the lean passes: 1024^2 Matern, 18 vectors: 77 us
+// here, 60 streamed.
 //
 // Where x, r or w live was tried three ways: registers with unrolled loops (12 items a
 // thread spilled, half the capacity), shared memory only (two thirds of the capacity), and
@@ -556,7 +559,6 @@ static __device__ __noinline__ void res_shift_role(const Solve &s, int stride, i
 template <int NT>
 __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team, int m,
                                              ResCtl *ctl, const double *part, int NP, unsigned in_bytes) {
-    constexpr int NW = NT / 32;
     const int lane = threadIdx.x & 31, M = pl.M;
     const bool clustered = pl.clustered;
     const double ds = s.precision == 0 ? s.op.scale : (double)s.op.scale_f;
@@ -726,7 +728,8 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
     constexpr bool MAT = KIND == KIND_2D13_SQ, D3 = KIND == KIND_3D7;
     constexpr int H = MAT ? 2 : 1, NB = D3 ? 6 : 4;
     constexpr bool SH = sizeof(V) == 4 && !D3;   // differences shared between lines
-    constexpr bool PRIV = !MAT || KX;          // second private vector: r, or p (Matern with x)
+    constexpr bool RS = MAT && !KX;            // r in shared memory and u by its recurrence (else p shared, r private)
+    constexpr bool PRIV = !RS;
     using It = ResItem<V>;
     using PM = PackMath<V, E>;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -738,20 +741,23 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
     const int PY = Ly + 2 * H;                 // shared lines per z-plane
     double *const part = reinterpret_cast<double *>(smem + lay.part);     // [2][5][NP]
     const int NP = clustered ? NW * M : NW;
-    V *const A = reinterpret_cast<V *>(smem + lay.a);       // p (5/7-point) or r (Matern), with halo lines
+    V *const A = reinterpret_cast<V *>(smem + lay.a);       // p, or r (Matern without x), with halo lines
     V *const B = reinterpret_cast<V *>(smem + lay.b);       // u (Matern), one halo line a side
-    V *const RH = reinterpret_cast<V *>(smem + lay.rh);     // r on the halo lines (5/7-point)
+    V *const RH = reinterpret_cast<V *>(smem + lay.rh);     // r on the halo lines (where A is p)
     const V *const HB = reinterpret_cast<const V *>(smem + lay.hb);   // incoming boundary w (clustered), [2][slots][GE]
     V *const XS = reinterpret_cast<V *>(smem + lay.x) + (size_t)tid * E;   // + i * NT * E
+    V *const XLS = reinterpret_cast<V *>(smem + lay.xl) + (size_t)tid * E;
     V *const DS = reinterpret_cast<V *>(smem + lay.d) + (size_t)tid * E;
-    // tensor memory: [w | r or p | x | diagonal], cmax items of 4 words each, in the 128
+    // tensor memory: [w | r | x | its low words | diagonal], cmax items of 4 words each, in the 128
     // columns of this warp (two warps of a CTA of 256 share a lane quarter, four of 512)
     const uint32_t tmw = ctl->tm + ((uint32_t)(wid & 3) << 21) + (uint32_t)(wid >> 2) * 128u;    // w
-    const uint32_t tma = tmw + 4u * cmax;                                                        // r or p
+    const uint32_t tma = tmw + 4u * cmax;                                                        // r
     constexpr uint32_t YW = sizeof(V) == 8 ? 4 : 8;            // words of an item's y (FP64)
     const uint32_t tmy = tma + (PRIV ? 4u * cmax : 0u);
-    const uint32_t tmx = tmy + (uint32_t)pl.yw * cmax, tmd = tmx + (lay.x_tm ? 4u * cmax : 0u);
-    const bool x_tm = lay.x_tm, d_tm = lay.d_tm, keepx = s.keep_x0;
+    const uint32_t tmx = tmy + (uint32_t)pl.yw * cmax, tmxl = tmx + (lay.x_tm ? 4u * cmax : 0u);
+    const uint32_t tmd = tmxl + (lay.xl_tm ? 4u * cmax : 0u);
+    const bool x_tm = lay.x_tm, xl_tm = lay.xl_tm, d_tm = lay.d_tm;
+    constexpr bool keepx = KX;
     const size_t hstride = (size_t)pl.slots * GE;   // one parity of one CTA's halo buffer
     V *const hglob = clustered ? nullptr : static_cast<V *>(ar.halo) + (size_t)team * M * 2 * hstride;
     // ---- this thread's run: group g of lines [l0, l0 + cnt)
@@ -810,15 +816,30 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
         }
     };
     auto sline = [&](int jy, int jz) { return D3 ? (jz + 1) * PY + jy + 1 : jy + H; };
-    auto x_add = [&](int i, const It &aa, const It &p) {       // x += alpha p
-        if (x_tm) {
-            TmItem t;
-            tm_ld(t, tmx + 4u * i);
-            tm_wait(t);
-            tm_st<V>(tmx + 4u * i, PM::fma(aa, p, tm_get<V>(t)));
+    // x += alpha p.  FP32 Matern solves run hundreds of iterations, and the roundings of these
+    // additions are most of the gradient's error: there x carries a low word (compensated
+    // summation: t = x + y, low = y - (t - x)), dropped when x is written.  300 x 200, eight
+    // kappa^2: median relative error of the gradient 4.8e-7 -> 7e-8, 4.9 -> 5.5 ms; sums of 32
+    // terms added to x at a time: 4.1e-7
+    constexpr bool XL = MAT && KX && sizeof(V) == 4;
+    auto x_get = [&](bool tmem, uint32_t col, const V *sh, int i) -> It {
+        if (!tmem) return ri_ld(sh + (size_t)i * NT * E);
+        TmItem t;
+        tm_ld(t, col + 4u * i);
+        tm_wait(t);
+        return tm_get<V>(t);
+    };
+    auto x_put = [&](bool tmem, uint32_t col, V *sh, int i, const It &v) {
+        if (tmem) tm_st<V>(col + 4u * i, v);
+        else ri_st(sh + (size_t)i * NT * E, v);
+    };
+    auto x_add = [&](int i, const It &aa, const It &p) {
+        if constexpr (XL) {
+            const It x = x_get(x_tm, tmx, XS, i), y = PM::fma(aa, p, x_get(xl_tm, tmxl, XLS, i)), t = PM::add(x, y);
+            x_put(x_tm, tmx, XS, i, t);
+            x_put(xl_tm, tmxl, XLS, i, PM::sub(y, PM::sub(t, x)));
         } else {
-            V *xp = XS + (size_t)i * NT * E;
-            ri_st(xp, PM::fma(aa, p, ri_ld(xp)));
+            x_put(x_tm, tmx, XS, i, PM::fma(aa, p, x_get(x_tm, tmx, XS, i)));
         }
     };
     unsigned long long tick = 0;                    // iterations of this launch: parity and record tags
@@ -861,13 +882,14 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         r.v[e] = start(v0 + e);
                         if (!ar.rhs && r.v[e] != (V)0) vbits |= 1ull << (i * E + e);
                     }
-                if constexpr (MAT) put(A + (size_t)sline(jy, jz) * pitch, g, r);
+                if constexpr (RS) put(A + (size_t)sline(jy, jz) * pitch, g, r);
             }
             __syncwarp();
             const It zz = zero_pack<V, E>();
             tm_st<V>(tmw + 4u * i, zz);
-            if constexpr (PRIV) tm_st<V>(tma + 4u * i, MAT ? zz : r);
+            if constexpr (PRIV) tm_st<V>(tma + 4u * i, r);
             if (keepx && x_tm) tm_st<V>(tmx + 4u * i, zz);
+            if (XL && xl_tm) tm_st<V>(tmxl + 4u * i, zz);
             if constexpr (RP) {
 #pragma unroll
                 for (uint32_t k = 0; k < YW; k += 4) tm_st<V>(tmy + YW * i + k, zz);
@@ -888,7 +910,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
 #pragma unroll
             for (int e = 0; e < E; ++e)
                 if (gg * E + e < nx) r.v[e] = start(v0 + e);
-            if constexpr (MAT) put(A + (size_t)line * pitch, gg, r);
+            if constexpr (RS) put(A + (size_t)line * pitch, gg, r);
             else ri_st(RH + (size_t)sl * GE + gg * E, r);
         }
         V al = (V)0, be = (V)0;
@@ -933,7 +955,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                 const It nas = PM::splat(-al * sc), aa = PM::splat(al);
                 // four items at a time, their loads in flight together
                 int jy = jy0, jz = jz0;
-                constexpr int U = KX ? 2 : 4;
+                constexpr int U = MAT && KX ? 2 : 4;
                 for (int i0 = 0; i0 < items; i0 += U) {
                     TmItem tw[U], ta[PRIV ? U : 1];
                     V *line[U];
@@ -955,17 +977,12 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         if (i >= items) break;
                         const bool act = i < cnt;
                         const It wv = tm_get<V>(tw[k]);
-                        if constexpr (RP) y_add(i, MAT ? old[k] : tm_get<V>(ta[PRIV ? k : 0]), wv);
-                        if constexpr (MAT) {
+                        if constexpr (RP) y_add(i, RS ? old[k] : tm_get<V>(ta[PRIV ? k : 0]), wv);
+                        if constexpr (RS) {
                             const It r = PM::fma(nas, wv, old[k]);
-                            if constexpr (KX) {
-                                const It pv = tm_get<V>(ta[k]);
-                                x_add(i, aa, pv);
-                                tm_st<V>(tma + 4u * i, PM::fma(bb, pv, r));
-                            }
                             if (act) put(line[k], g, r);
                         } else {
-                            if (keepx) x_add(i, aa, old[k]);
+                            if constexpr (keepx) x_add(i, aa, old[k]);
                             const It r = PM::fma(nas, wv, tm_get<V>(ta[k]));
                             tm_st<V>(tma + 4u * i, r);
                             if (act) put(line[k], g, PM::fma(bb, old[k], r));
@@ -986,7 +1003,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         wn = clustered ? ri_ld(src) : ri_ldcg(src);
                     }
                     V *line = A + (size_t)li * pitch;
-                    if constexpr (MAT) {
+                    if constexpr (RS) {
                         put(line, gg, PM::fma(nas, wn, ri_ld(line + E + gg * E)));
                     } else {
                         V *rp = RH + (size_t)sl * GE + gg * E;
@@ -1001,7 +1018,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
             It d_rr = zz, d_pw = zz, d_rw = zz, d_ww = zz;
             V d_vr = (V)0;
             if constexpr (MAT) {
-                // ---- u = Q1 r + beta u on own lines and one line beyond on each side
+                // ---- u = Q1 r + beta u, or Q1 p, on own lines and one line beyond on each side
                 const It cc = PM::splat(k2);
                 // a row ahead: the line below, the old u and the side neighbours of the next row
                 // load while this row is formed.  Loads past the run's end are clamped to the
@@ -1017,7 +1034,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     om = od;
                     od = min(od + pitch, odmax);
                     ou = min(ou + pitch, oumax);
-                    const It dn2 = ri_ld(A + od), uo2 = ri_ld(B + ou);
+                    const It dn2 = ri_ld(A + od), uo2 = RS ? ri_ld(B + ou) : zz;
                     // side neighbours: across the lanes, and from the line at the warp's ends
                     const V ls = __shfl_up_sync(0xffffffffu, dn.v[E - 1], 1), rs = __shfl_down_sync(0xffffffffu, dn.v[0], 1);
                     V le = (V)0, re = (V)0;
@@ -1032,7 +1049,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         u = res_level<V, 4>(cc, mid, l, r, dn, up, zz, zz);
                         up = mid;
                     }
-                    u = PM::fma(bb, uo, u);
+                    if constexpr (RS) u = PM::fma(bb, uo, u);
                     clip(u);
                     if (i < cnt) {
                         if constexpr (!RP) d_pw = PM::fma(u, u, d_pw);
@@ -1051,7 +1068,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     const V *rw = A + (size_t)(side ? H + L : H - 1) * pitch + E + gg * E;
                     V *uo = B + (size_t)(side ? L + 1 : 0) * pitch;
                     It u = res_level<V, 4>(cc, ri_ld(rw), rw[-1], rw[E], ri_ld(rw + pitch), ri_ld(rw - pitch), zz, zz);
-                    u = PM::fma(bb, ri_ld(uo + E + gg * E), u);
+                    if constexpr (RS) u = PM::fma(bb, ri_ld(uo + E + gg * E), u);
                     const int nv = min(E, nx - gg * E);
 #pragma unroll
                     for (int e = 0; e < E; ++e)
@@ -1088,7 +1105,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     fr = ri_ld(row - PY * pitch);
                     bck = ri_ld(row + PY * pitch);
                 }
-                if constexpr (MAT) rv = ri_ld(rrow);
+                if constexpr (RS) rv = ri_ld(rrow);
                 V l, r;
                 if constexpr (D3) {
                     l = __shfl_up_sync(0xffffffffu, mid.v[E - 1], 1);
@@ -1100,19 +1117,21 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     r = row[E];
                 }
                 TmItem ta, td;
-                if constexpr (!MAT) tm_ld(ta, tma);
+                if constexpr (PRIV) tm_ld(ta, tma);
                 if (!MAT && d_tm) tm_ld(td, tmd);
                 uint64_t vb = vbits, mb = mbits;
 #pragma unroll 2
                 for (int i = 0; i < items; ++i) {
                     const bool act = i < cnt;
                     It cc;
-                    if constexpr (!MAT) {
-                        if (d_tm) tm_wait(ta, td);
+                    const int in = min(i + 1, cmax - 1);
+                    if constexpr (PRIV) {
+                        if (!MAT && d_tm) tm_wait(ta, td);
                         else tm_wait(ta);
                         rv = tm_get<V>(ta);
-                        const int in = min(i + 1, cmax - 1);
                         tm_ld(ta, tma + 4u * in);
+                    }
+                    if constexpr (!MAT) {
                         if (use_d) {
                             if (d_tm) {
                                 cc = tm_get<V>(td);
@@ -1157,7 +1176,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         r2 = __shfl_down_sync(0xffffffffu, mid2.v[0], 1);
                         if (lfix) le = S[om - 1];
                         if (rfix) re = S[om + E];
-                        if constexpr (MAT) {
+                        if constexpr (RS) {
                             rrow += pitch;
                             rv2 = ri_ld(rrow);
                         }
@@ -1171,7 +1190,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         wv = res_level<V, NB>(cc, mid, l, r, dn, up, fr, bck);
                     }
                     clip(wv);
-                    if constexpr (MAT) clip(rv);   // a torus ghost inside a partial item is not r
+                    if constexpr (RS) clip(rv);    // a torus ghost inside a partial item is not r
                     tm_st<V>(tmw + 4u * i, wv);
                     if (act) {
                         if constexpr (!RP) {
@@ -1214,8 +1233,8 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     r = !D3 && rfix ? re : r2;
                     row = nrow;
                 }
-                if constexpr (!MAT) {
-                    if (d_tm) tm_wait(ta, td);     // the load past the last item
+                if constexpr (PRIV) {
+                    if (!MAT && d_tm) tm_wait(ta, td);     // the load past the last item
                     else tm_wait(ta);
                 }
                 tm_wait_st();
@@ -1349,19 +1368,11 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                 __syncwarp();
             }
         }
-        if (keepx) {
+        if constexpr (keepx) {
             const int tile = c / s.T, t = c - tile * s.T;
             V *x = static_cast<V *>(s.x) + (int64_t)tile * s.op.n * s.T + t;
             for (int i = 0, jy = jy0, jz = jz0; i < items; ++i, next_line(jy, jz)) {
-                It xv;
-                if (x_tm) {
-                    TmItem tx;
-                    tm_ld(tx, tmx + 4u * i);
-                    tm_wait(tx);
-                    xv = tm_get<V>(tx);
-                } else {
-                    xv = ri_ld(XS + (size_t)i * NT * E);
-                }
+                const It xv = x_get(x_tm, tmx, XS, i);
                 if (i < cnt) {
                     const int64_t v0 = own_vertex(jy, jz);
 #pragma unroll
@@ -1383,7 +1394,7 @@ __device__ __forceinline__ void resident_body(const Solve &s, const ResPlan &pl,
                                               unsigned char *smem) {
     constexpr int NW = NT / 32;
     const int wid = threadIdx.x >> 5;
-    const ResSmem lay = res_smem(pl, (int)sizeof(V), KIND, s.nshift, s.keep_x0, KIND != KIND_2D13_SQ && s.op.field_d != nullptr);
+    const ResSmem lay = res_smem(pl, (int)sizeof(V), KIND, s.nshift, KX, KIND != KIND_2D13_SQ && s.op.field_d != nullptr);
     ResCtl *const ctl = reinterpret_cast<ResCtl *>(smem + lay.bc);
     constexpr uint32_t TM_COLS = NT == 256 ? 256 : 512;
     const int NP = pl.clustered ? NW * pl.M : NW;

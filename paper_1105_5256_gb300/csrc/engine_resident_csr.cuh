@@ -16,13 +16,13 @@
 //
 // r, w, x of own rows and r of external columns are private to a thread: tensor memory.
 //
-// Bound by the two hops of the exchange (about 8 us of an iteration) on small matrices, by
+// Bound by the two hops of the exchange (about 7 us of an iteration) on small matrices, by
 // shared-memory wavefronts of the gathers (FP32) or the FP64 units on larger ones.  Measured
 // a CG iteration over all vectors (before: one CTA a tile, or the streaming step and product):
-// 64^2 torus FP64, 25 vectors 38.7 -> 10.6 us; second-order FEM mesh of 13K vertices, 31
-// vectors, FP32 220 -> 12.3, FP64 80 -> 40; of 90K vertices, 33 vectors, FP32 85 -> 60 (the
+// 64^2 torus FP64, 25 vectors 38.7 -> 11 us; second-order FEM mesh of 13K vertices, 31
+// vectors, FP32 220 -> 10.2, FP64 80 -> 38; of 90K vertices, 33 vectors, FP32 85 -> 44 (the
 // last vector of 33 runs in a round of its own, on four vectors a team); FP64 of that size
-// stays with the streaming passes (295 against 206).
+// stays with the streaming passes (270 against 206).
 #pragma once
 #include "engine_resident.cuh"
 

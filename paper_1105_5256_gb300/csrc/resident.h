@@ -12,9 +12,10 @@ constexpr int RES_CTL_BYTES = 288;
 
 // bytes of one CTA's shared memory by purpose (offsets from the dynamic base)
 struct ResSmem {
-    size_t part, bc, shift, a, b, rh, hb, x, d, bytes;
+    size_t part, bc, shift, a, b, rh, hb, x, xl, d, bytes;
     size_t zero_bytes;      // from `a`: what a new column starts from zero
-    bool x_tm, d_tm;        // x, diagonal in tensor memory (else in shared memory)
+    bool xl_on;             // x carries its low words (FP32 Matern, see x_add)
+    bool x_tm, xl_tm, d_tm; // x, its low words, diagonal in tensor memory (else in shared memory)
 };
 
 __host__ __device__ inline ResSmem res_smem(const ResPlan &p, int word, int kind, int nshift, int keepx, bool field) {
@@ -24,11 +25,14 @@ __host__ __device__ inline ResSmem res_smem(const ResPlan &p, int word, int kind
     const size_t np = p.clustered ? (size_t)NW * p.M : NW;
     const size_t priv = (size_t)p.cmax * p.nt * 16;
     ResSmem s;
-    // private vectors in tensor memory, 128 words a thread: w; r or (Matern with x) p; then
+    // private vectors in tensor memory, 128 words a thread: w; r (but Matern without x); then
     // x and the diagonal while they fit
     int room = 32 - p.cmax * ((mat && !keepx ? 1 : 2) + p.yw / 4);
     s.x_tm = keepx && room >= p.cmax;
     if (s.x_tm) room -= p.cmax;
+    s.xl_on = mat && keepx && word == 4;
+    s.xl_tm = s.xl_on && room >= p.cmax;
+    if (s.xl_tm) room -= p.cmax;
     s.d_tm = field && room >= p.cmax;
     size_t o = 0;
     s.part = o;
@@ -42,9 +46,11 @@ __host__ __device__ inline ResSmem res_smem(const ResPlan &p, int word, int kind
     s.b = o;
     if (mat) o += (size_t)(p.Ly + 2) * pitch;
     s.rh = o;
-    if (!mat) o += (size_t)p.slots * ge;
+    if (!mat || keepx) o += (size_t)p.slots * ge;
     s.x = o;
     if (keepx && !s.x_tm) o += priv;
+    s.xl = o;
+    if (s.xl_on && !s.xl_tm) o += priv;
     s.zero_bytes = o - s.a;
     s.hb = o;
     if (p.clustered) o += 2 * (size_t)p.slots * ge;
