@@ -4,6 +4,7 @@
 #include "engine_device.cuh"
 #include "engine_lean.cuh"
 #include "engine_lean3d.cuh"
+#include "sweep.h"
 
 namespace ld {
 
@@ -553,12 +554,9 @@ __global__ void __launch_bounds__(256) k_residual_sweep(Solve s, int set, int cb
     // y blocks (3D) and segments of the marching axis share blockIdx.y
     const int yb = D3 ? (ny + 7) / 8 : 1;
     const int m0 = ((int)blockIdx.y / yb) * seg, m1 = min(m0 + seg, nm);
-    // difference form: lane 0 only supplies its neighbour's left difference
-    constexpr int W = DIFF ? 31 : 32;
-    const int gx = (D3 ? (int)blockIdx.x : (int)blockIdx.x * 8 + wid) * W + lane - (DIFF ? 1 : 0);
-    const int gy = D3 ? ((int)blockIdx.y % yb) * 8 + wid : 0;
-    const bool own = gx < nx && (!D3 || gy < ny) && (!DIFF || lane > 0);
-    const bool in = own || (DIFF && lane == 0 && (!D3 || gy < ny));       // lanes that load
+    const SweepLane<D3, DIFF> me(nx, ny, blockIdx.x, (int)blockIdx.y % yb, wid, lane);
+    const int gx = me.gx, gy = me.gy;
+    const bool own = me.own, in = me.in;
     const int64_t n = s.op.n, off = (int64_t)tile * n * T;
     const int64_t step = D3 ? (int64_t)nx * ny : nx;                    // vertices between marching positions
     const V *const x = static_cast<const V *>(s.x) + off;
@@ -582,14 +580,8 @@ __global__ void __launch_bounds__(256) k_residual_sweep(Solve s, int set, int cb
     const D zero = {};
     // x at (xx, yy) of marching position m, wrapped on a torus, zero outside a Dirichlet grid
     auto at = [&](int xx, int yy, int m) {
-        if (per) {
-            xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-            if constexpr (D3) yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
-            m = m < 0 ? m + nm : (m >= nm ? m - nm : m);
-        } else if (xx < 0 || xx >= nx || m < 0 || m >= nm || (D3 && (yy < 0 || yy >= ny))) {
-            return zero;
-        }
-        return load((int64_t)m * step + (D3 ? (int64_t)yy * nx : 0) + xx);
+        const int64_t j = sweep_vertex<D3>(nx, ny, nm, per, xx, yy, m);
+        return j < 0 ? zero : load(j);
     };
     __shared__ double sh[D3 ? 2 * 8 * 32 * T : 1];
     __shared__ double red[8 * T];
