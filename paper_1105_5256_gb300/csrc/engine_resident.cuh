@@ -689,12 +689,14 @@ __device__ __noinline__ void res_replay_role(const Solve &s, const ResPlan &pl, 
             const int par = (int)(tick & 1);
             const double2 ab = ar.ab[(size_t)c * ar.hcap + it];
             bool ok = true;
+            // every vector warp has read the last alpha and beta (and, cooperative, sent its rows):
+            // a neighbour's rows may be here before this CTA's own warps have come that far
+            bar_sync(3, NT + 32);
             if (clustered) {
                 ok = res_bar_wait(smem_u32(&ctl->bar[par]), (unsigned)(tick >> 1) & 1u);
                 __syncwarp();
                 if (lane == 0) mbar_arrive_tx(&ctl->bar[par], in_bytes);      // armed for tick + 2
             } else {
-                bar_sync(3, NT + 32);
                 __threadfence();
                 ulonglong2 *rp = rec + (size_t)par * M * 8;
                 if (lane == 0) rec_st(rp + (size_t)m * 8, 0.0, tick + 1);
@@ -1239,10 +1241,8 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                 }
                 tm_wait_st();
                 if constexpr (RP) {
-                    if (!clustered) {
-                        __threadfence();
-                        bar_arrive(3, NT + 32);
-                    }
+                    if (!clustered) __threadfence();
+                    bar_arrive(3, NT + 32);
                 } else {
                 V flat[RES_NDOT] = {d_rr.v[0], d_pw.v[0], d_rw.v[0], d_ww.v[0], d_vr}, sum[1];
 #pragma unroll
