@@ -318,9 +318,16 @@ ld_status ld_hutchinson(ld_ctx *ctx, int s, const double *Z, double *estimate, d
 /* Failure-path self-test of the library's bounded device waits (the paper has no
  * counterpart): one CTA on the current device waits on a barrier that nothing
  * completes, gives up after limit_ns nanoseconds (1e3 .. 1e10) and the call returns
- * LD_ETIMEOUT, as a pass whose bulk copies never arrived would; LD_OK would mean the
- * wait was not bounded as documented.  Allocates 4 bytes of device memory. */
+ * LD_ETIMEOUT, as a pass whose bulk copies never arrived would; so do the resident
+ * engines' waits, on a record that nobody writes and on a cluster barrier.  LD_OK would
+ * mean that a wait was not bounded as documented.  Allocates under 1 KB of device memory. */
 ld_status ld_wait_selftest(int64_t limit_ns);
+
+/* The same for whole teams: the solve of ld_logdet on the resident engine's cooperative
+ * teams, with the launch's last CTA left out and waits of limit_ns (1e6 .. 1e10).  The
+ * CTAs that wait for it give up, the kernel ends, and the call returns LD_ETIMEOUT; the
+ * context stays usable.  LD_EUNSUPPORTED: the context's solves use no cooperative teams. */
+ld_status ld_team_wait_selftest(ld_ctx *ctx, int64_t limit_ns);
 
 /* Host utilities (no device work; usable without a GPU). */
 

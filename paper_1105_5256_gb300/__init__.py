@@ -116,6 +116,7 @@ def library(build_if_missing: bool = False):
         "ld_select_distance": ([vp, i64, dbl, C.c_int, P(i32), vp, P(Info)], st),
         "ld_hutchinson": ([vp, C.c_int, vp, P(dbl), P(dbl), vp, P(Info)], st),
         "ld_wait_selftest": ([i64], st),
+        "ld_team_wait_selftest": ([vp, i64], st),
         "ld_invsqrt_mv": ([vp, C.c_int, vp, vp, P(Info)], st),
         "ld_colour_csr": ([i64, vp, vp, C.c_int, vp, P(i32)], st),
         "ld_colour_grid": ([C.c_int, vp, C.c_int, C.c_int, vp, P(i32)], st),
@@ -387,6 +388,12 @@ def ld_wait_selftest(limit_ns: int):
     """Bounded-wait self-test: raises LogDetError(LD_ETIMEOUT) when the device wait gave
     up after limit_ns as documented."""
     _check(library().ld_wait_selftest(int(limit_ns)))
+
+
+def ld_team_wait_selftest(ctx: Context, limit_ns: int):
+    """The same on a context's cooperative teams, one CTA of which is left out: raises
+    LogDetError(LD_ETIMEOUT) when its team gave up."""
+    _check(library().ld_team_wait_selftest(ctx.handle, int(limit_ns)))
 
 
 def ld_hutchinson(ctx: Context, Z: np.ndarray):

@@ -649,7 +649,8 @@ std::mutex g_coop_mu;   // cooperative resident solves of this process
 
 // One probed solve over colours [cb, ce).  On LD_OK, result[0..1] hold
 // sum of terms and sum of seed projections on the device and in *out.
-ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_info *info) {
+// test_wait_ns > 0: self-test, see ld_team_wait_selftest.
+ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_info *info, uint64_t test_wait_ns = 0) {
     Range range("ld solve");
     int64_t launches = 0;
     int iters = 0;
@@ -706,6 +707,10 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
             resident = true;
         }
     }
+    if (test_wait_ns > 0) {
+        const bool teams = resident && (c->kind == LD_CSR ? c->csr_plan.M : c->res_plan[want_x0].clustered ? 1 : c->res_plan[want_x0].M) > 1;
+        if (!teams) return fail(LD_EUNSUPPORTED, "the context does not run on cooperative teams");
+    }
     // the lean lattice pass (four state words per vertex and column) wherever it applies;
     // the stored-w pass otherwise (FP64, other kinds, the Matern kind with a kept x0)
     const int want_lean = c->engine == 1 && c->opt.lattice_pass == 0 && !resident ? ld::engine_lean_x(c->s, keep_x0) : 0;
@@ -734,6 +739,8 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
     }
     if (resident) {
         ld::ResArgs ra{};
+        ra.wait_ns = test_wait_ns > 0 ? test_wait_ns : ld::RES_WAIT_NS;
+        ra.missing = test_wait_ns > 0 ? 1 : 0;
         ra.cb = cb;
         ra.ce = ce;
         // the iteration cap of the engine this context would otherwise run (whole chunks)
@@ -1628,6 +1635,7 @@ static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y
     for (int64_t i = 0; i < n; ++i)
         for (size_t k = 0; k < C; ++k) norm2[k] += V[i * C + k] * V[i * C + k];
     ld::ResArgs ra{};
+    ra.wait_ns = ld::RES_WAIT_NS;
     ra.cb = 0;
     ra.ce = ncols;
     ra.cap = max_iter;
@@ -1832,15 +1840,27 @@ ld_status ld_invsqrt_mv(ld_ctx *c, int ncols, const double *V, double *Y, ld_inf
 
 ld_status ld_wait_selftest(int64_t limit_ns) {
     if (limit_ns < 1000 || limit_ns > 10000000000LL) return fail(LD_EINVAL, "limit_ns out of range");
-    DevBuf st;
-    CUDA_TRY(st.alloc(sizeof(int32_t)));
-    CUDA_TRY(cudaMemset(st.p, 0xff, sizeof(int32_t)));
+    DevBuf st, rec;
+    CUDA_TRY(st.alloc(2 * sizeof(int32_t)));
+    CUDA_TRY(rec.alloc(16));
+    CUDA_TRY(cudaMemset(st.p, 0xff, st.bytes));
+    CUDA_TRY(cudaMemset(rec.p, 0, rec.bytes));
     ENGINE_TRY(ld::engine_wait_selftest((uint64_t)limit_ns, st.as<int32_t>(), nullptr));
-    int32_t h = -1;
-    CUDA_TRY(cudaMemcpy(&h, st.p, sizeof h, cudaMemcpyDeviceToHost));
-    if (h == ld::DEV_TIMEOUT) return fail(LD_ETIMEOUT, "device wait gave up after %lld ns", (long long)limit_ns);
-    if (h == ld::DEV_OK) return LD_OK;
-    return fail(LD_ECUDA, "self-test kernel did not report (status %d)", h);
+    ENGINE_TRY(ld::engine_resident_wait_selftest((uint64_t)limit_ns, rec.p, st.as<int32_t>() + 1, nullptr));
+    int32_t h[2] = {-1, -1};
+    CUDA_TRY(cudaMemcpy(h, st.p, sizeof h, cudaMemcpyDeviceToHost));
+    if (h[0] == ld::DEV_TIMEOUT && h[1] == 3)
+        return fail(LD_ETIMEOUT, "device waits gave up after %lld ns: bulk copy, record, cluster barrier", (long long)limit_ns);
+    if (h[0] == ld::DEV_OK || (h[1] >= 0 && h[1] < 3)) return LD_OK;
+    return fail(LD_ECUDA, "self-test kernels did not report (status %d, %d)", h[0], h[1]);
+}
+
+ld_status ld_team_wait_selftest(ld_ctx *c, int64_t limit_ns) {
+    if (!c || limit_ns < 1000000 || limit_ns > 10000000000LL) return fail(LD_EINVAL, "limit_ns out of range");
+    if (c->is_batch) return fail(LD_EINVAL, "batched context");
+    REJECT_MATFREE(c);
+    double out[2];
+    return run_solve(c, 0, c->ncolours, c->opt.keep_x0 != 0, out, nullptr, (uint64_t)limit_ns);
 }
 
 ld_status ld_hutchinson(ld_ctx *c, int s, const double *Z, double *estimate, double *std_error,

@@ -109,9 +109,9 @@ double stream_clocks(const Solve &s, int ncolours, bool keep_x0) {
 }
 
 template <class F>
-cudaError_t res_launch(const ResPlan &p, cudaStream_t st, F &&fn) {
+cudaError_t res_launch(const ResPlan &p, int missing, cudaStream_t st, F &&fn) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(p.J * p.M));
+    cfg.gridDim = dim3((unsigned)(p.J * p.M - missing));
     cfg.blockDim = dim3((unsigned)(p.nt + 64));
     cfg.dynamicSmemBytes = p.smem;
     cfg.stream = st;
@@ -150,7 +150,7 @@ static int resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
             if (!res_geometry(s, keep_x0, yw, nt, M, true, p)) continue;
             p.J = ncolours;
             int act = 0;
-            cudaError_t e = res_launch(p, nullptr, [&](cudaLaunchConfig_t &cfg) {
+            cudaError_t e = res_launch(p, 0, nullptr, [&](cudaLaunchConfig_t &cfg) {
                 return cudaOccupancyMaxActiveClusters(&act, fn, &cfg);
             });
             if (e != cudaSuccess || act < 1) {
@@ -265,9 +265,31 @@ int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *st
     ResArgs av = a;
     pv.smem = res_smem(p, s.precision == 0 ? 8 : 4, s.op.kind, s.nshift, kx, s.op.kind != KIND_2D13_SQ && s.op.field_d).bytes;
     void *args[] = {&sv, &pv, &av};
-    e = res_launch(pv, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
+    e = res_launch(pv, a.missing, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
+}
+
+// One CTA waits on a record that nobody writes (status bit 0: it gave up) and on a phase of its
+// own barrier that nobody completes (bit 1).
+__global__ void k_resident_wait_selftest(uint64_t limit_ns, const ulonglong2 *rec, int32_t *status) {
+    __shared__ uint64_t bar;
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    double v;
+    const bool got = rec_wait(rec, 1, v, limit_ns);
+    const bool done = res_bar_wait(smem_u32(&bar), 0u, limit_ns);
+    __syncthreads();
+    if (threadIdx.x == 0) *status = (got ? 0 : 1) | (done ? 0 : 2);
+}
+
+int engine_resident_wait_selftest(uint64_t limit_ns, void *rec_dev, int32_t *status_dev, void *stream) {
+    k_resident_wait_selftest<<<1, 32, 0, static_cast<cudaStream_t>(stream)>>>(
+        limit_ns, static_cast<const ulonglong2 *>(rec_dev), status_dev);
+    return (int)cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ vector form
@@ -340,7 +362,7 @@ int engine_resident_funmv(const Solve &s, const ResPlan &p, const ResArgs &a, in
     ResPlan pv = p;
     ResArgs av = a;
     void *args[] = {&sv, &pv, &av};
-    e = res_launch(pv, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
+    e = res_launch(pv, 0, st, [&](cudaLaunchConfig_t &cfg) { return cudaLaunchKernelExC(&cfg, fn, args); });
     if (e != cudaSuccess) cudaGetLastError();
     return (int)e;
 }

@@ -224,8 +224,8 @@ __device__ __forceinline__ bool rec_ld(const ulonglong2 *p, unsigned long long t
     v = __longlong_as_double(a);
     return b == tag;
 }
-// wait for a record's tag; false after two seconds
-__device__ __forceinline__ bool rec_wait(const ulonglong2 *p, unsigned long long tag, double &v) {
+// wait for a record's tag; false after limit_ns
+__device__ __forceinline__ bool rec_wait(const ulonglong2 *p, unsigned long long tag, double &v, uint64_t limit_ns) {
     if (rec_ld(p, tag, v)) return true;
     uint64_t t0 = 0;
     for (unsigned it = 0;; ++it) {
@@ -233,7 +233,7 @@ __device__ __forceinline__ bool rec_wait(const ulonglong2 *p, unsigned long long
         if ((it & 255) == 0) {
             const uint64_t t = global_ns();
             if (it == 0) t0 = t;
-            else if (t - t0 > 2000000000ull) return false;
+            else if (t - t0 > limit_ns) return false;
         }
     }
 }
@@ -365,8 +365,8 @@ __device__ __forceinline__ void st_async(uint32_t addr, uint32_t bar, const ResI
                  "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(bar)
                  : "memory");
 }
-// wait for a phase of this CTA's mbarrier, with the remote stores it counted; false after two seconds
-__device__ __forceinline__ bool res_bar_wait(uint32_t bar, unsigned parity) {
+// wait for a phase of this CTA's mbarrier, with the remote stores it counted; false after limit_ns
+__device__ __forceinline__ bool res_bar_wait(uint32_t bar, unsigned parity, uint64_t limit_ns) {
     uint64_t t0 = 0;
     for (unsigned it = 0;; ++it) {
         unsigned ok;
@@ -380,7 +380,7 @@ __device__ __forceinline__ bool res_bar_wait(uint32_t bar, unsigned parity) {
         if ((it & 63) == 0) {
             const uint64_t t = global_ns();
             if (it == 0) t0 = t;
-            else if (t - t0 > 2000000000ull) return false;
+            else if (t - t0 > limit_ns) return false;
         }
     }
 }
@@ -594,7 +594,7 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
                     st_async(mapa(smem_u32(&ctl->dflag[par]), lane), mapa(smem_u32(&ctl->bar[par]), lane), fl);
             } else {
                 if (m == 0 && lane == 0) rec_st(rp + 5, fl, tag);
-                ok = rec_wait(rp + 5, tag, fl);
+                ok = rec_wait(rp + 5, tag, fl, ar.wait_ns);
             }
             bar_sync(3, 160);                 // the sums of vector warps 0 to 3
             if (clustered) {
@@ -630,7 +630,7 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
                     for (int q = lane; q < (clustered ? NP : M); q += 32) {
                         double v = 0.0;
                         if (clustered) v = pp[(size_t)4 * NP + q];
-                        else ok = rec_wait(rp + (size_t)q * 8 + 4, tag, v) && ok;
+                        else ok = rec_wait(rp + (size_t)q * 8 + 4, tag, v, ar.wait_ns) && ok;
                         vr_sum += v;
                     }
                     __syncwarp();
@@ -693,7 +693,7 @@ __device__ __noinline__ void res_replay_role(const Solve &s, const ResPlan &pl, 
             // a neighbour's rows may be here before this CTA's own warps have come that far
             bar_sync(3, NT + 32);
             if (clustered) {
-                ok = res_bar_wait(smem_u32(&ctl->bar[par]), (unsigned)(tick >> 1) & 1u);
+                ok = res_bar_wait(smem_u32(&ctl->bar[par]), (unsigned)(tick >> 1) & 1u, ar.wait_ns);
                 __syncwarp();
                 if (lane == 0) mbar_arrive_tx(&ctl->bar[par], in_bytes);      // armed for tick + 2
             } else {
@@ -701,7 +701,7 @@ __device__ __noinline__ void res_replay_role(const Solve &s, const ResPlan &pl, 
                 ulonglong2 *rp = rec + (size_t)par * M * 8;
                 if (lane == 0) rec_st(rp + (size_t)m * 8, 0.0, tick + 1);
                 double v;
-                if (lane < 4 && bk.has[lane]) ok = rec_wait(rp + (size_t)bk.nb(lane) * 8, tick + 1, v);
+                if (lane < 4 && bk.has[lane]) ok = rec_wait(rp + (size_t)bk.nb(lane) * 8, tick + 1, v, ar.wait_ns);
                 __threadfence();
             }
             if (!__all_sync(0xffffffffu, ok)) {
@@ -1266,7 +1266,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         for (int q = lane & 3; q < M; q += 4) st_async(mapa(slot, q), mapa(bar_addr, q), tot);
                     }
                     if (wid < 4) {
-                        if (!res_bar_wait(bar_addr, (unsigned)(tick >> 1) & 1u)) ctl->bad = 1;
+                        if (!res_bar_wait(bar_addr, (unsigned)(tick >> 1) & 1u, ar.wait_ns)) ctl->bad = 1;
                         const double *pp = part + (size_t)(par * RES_NDOT + wid) * NP;
                         double a = lane < NP ? pp[lane] : 0.0;
                         for (int q = lane + 32; q < NP; q += 32) a += pp[q];
@@ -1306,7 +1306,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                                 if ((spin & 255) == 255) {
                                     const uint64_t t = global_ns();
                                     if (t0 == 0) t0 = t;
-                                    else if (t - t0 > 2000000000ull) {
+                                    else if (t - t0 > ar.wait_ns) {
                                         ok = false;
                                         break;
                                     }
@@ -1463,6 +1463,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident_batch(const Solve *solv
         reinterpret_cast<uint32_t *>(&pl)[q] = reinterpret_cast<const uint32_t *>(plans + it.x)[q];
     __syncthreads();
     ResArgs ar{};
+    ar.wait_ns = RES_WAIT_NS;
     ar.cb = it.y;
     ar.ce = it.y + 1;
     ar.cap = cap;

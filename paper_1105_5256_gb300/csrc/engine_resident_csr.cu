@@ -215,7 +215,7 @@ int engine_resident_csr(const Solve &s, const CsrPlan &p, const ResArgs &a, void
         const void *fn = csr_kernel(s.precision, pv.T / E);
         Solve sv = s;
         void *args[] = {&sv, &pv, &av};
-        e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)(p.J * p.M)), dim3((unsigned)(p.nt + 64)), args, pv.smem, st);
+        e = cudaLaunchCooperativeKernel(fn, dim3((unsigned)(p.J * p.M - a.missing)), dim3((unsigned)(p.nt + 64)), args, pv.smem, st);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return (int)e;

@@ -50,10 +50,10 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
     const bool owner = m < T;                    // of vector c0 + m
     unsigned long long tick = 0;
     int head = 0;
-    auto timed = [&](uint64_t &t0) -> bool {     // two seconds from the first call
+    auto timed = [&](uint64_t &t0) -> bool {     // the limit, from the first call
         const uint64_t t = global_ns();
         if (t0 == 0) t0 = t;
-        return t - t0 > 2000000000ull;
+        return t - t0 > ar.wait_ns;
     };
     for (int c0 = ar.cb + team * T; c0 < ar.ce; c0 += pl.J * T) {
         const int c = c0 + m;
@@ -118,7 +118,7 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
                     double vr_sum = 0.0;
                     for (int q = lane; q < M; q += 32) {
                         double v = 0.0;
-                        ok = rec_wait(rp + (size_t)q * 6 + 4, tag, v) && ok;
+                        ok = rec_wait(rp + (size_t)q * 6 + 4, tag, v, ar.wait_ns) && ok;
                         vr_sum += v;
                     }
                     __syncwarp();
@@ -371,7 +371,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
                         if ((spin & 255) == 255) {
                             const uint64_t t = global_ns();
                             if (t0 == 0) t0 = t;
-                            else if (t - t0 > 2000000000ull) {
+                            else if (t - t0 > ar.wait_ns) {
                                 ok = false;
                                 break;
                             }

@@ -126,7 +126,10 @@ struct ResPlan {
     int yw;               // vector form: words of y per item in tensor memory (4 FP64, 8 FP32), else 0
     size_t smem;
 };
+constexpr uint64_t RES_WAIT_NS = 2000000000;   // limit of every device wait of the resident engines
 struct ResArgs {
+    uint64_t wait_ns;     // limit of a device wait: RES_WAIT_NS but in the self-test
+    int missing;          // self-test: CTAs of a cooperative launch left out at its end
     int cb, ce;           // colour range
     int cap;              // iterations at most
     int terms;            // 1: the shift warp also writes s.terms (batches)
@@ -207,6 +210,9 @@ int engine_grad_params(const Solve &s, int nparam, const int *ids, double *out_d
 // one CTA waits on an mbarrier nothing arrives at, giving up after limit_ns: writes
 // DEV_TIMEOUT (or DEV_OK) to *status_dev
 int engine_wait_selftest(uint64_t limit_ns, int32_t *status_dev, void *stream);
+// the same for the resident engines' waits, on a record nobody writes (rec_dev: 16 zeroed
+// bytes) and on a barrier phase nobody completes
+int engine_resident_wait_selftest(uint64_t limit_ns, void *rec_dev, int32_t *status_dev, void *stream);
 // diag_d[i] = kappa2 * (field ? field[i] : 1) + tau * (mask ? mask[i] : 0), diag_f its FP32 copy
 int engine_fill_diag(const Operator &op, double *diag_d, float *diag_f, void *stream);
 // reliable updates: x_hi += x_lo, x_lo = 0 (all tiles); then with replace != 0 the active
