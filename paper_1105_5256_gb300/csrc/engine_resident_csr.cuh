@@ -144,7 +144,10 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
                 code = ncode;
             }
         }
-        if (live0) {
+        // After a wait that ran out every owner posts the end, whether or not its vector of this group
+        // is live: the shift warp passes over an empty colour class and may be waiting for a later
+        // group's entries (or be gone, and the entry stays unread).
+        if (live0 || (owner && ctl->stop == 2)) {
             while (head - ctl->tail >= 4) {}
             if (lane == 0) {
                 ctl->q[head & 3].code = ctl->stop == 2 ? -2 : -1;

@@ -47,6 +47,21 @@ def test_a_csr_team_without_its_last_cta_gives_up(prec):
     assert L.ld_logdet(ctx)[0] == v
 
 
+@pytest.mark.parametrize("prec", [L.LD_FP64, L.LD_MIXED])
+def test_a_csr_team_gives_up_with_empty_colour_classes(prec):
+    """A caller's colouring with gaps: of the first 200 colours the odd ones are empty, the others
+    have a vertex each.  A team solves at most 152 colours at a time over a launch, in tiles of an
+    even number, so odd owners start with an empty class and have vectors in later rounds."""
+    n = 640
+    rp, ci, vv = synth.csr_from_edges(n, *synth.random_sparse_spd_pattern(9, n), 0.3)
+    col = np.concatenate([np.arange(0, 200, 2), np.arange(200, 740)]).astype(np.int32)
+    ctx = L.ld_create(L.csr_matrix(rp, ci, vv), 1, 16, 1e-6, L.options(precision=prec, colouring=col))
+    v, info = L.ld_logdet(ctx)
+    assert info["engine"] == 4 and info["n_colours"] == 740
+    gives_up(ctx)
+    assert L.ld_logdet(ctx)[0] == v
+
+
 def test_the_self_test_needs_teams():
     ctx = L.ld_create(L.grid_matrix(L.LD_STENCIL_2D5, (32, 16), 0.5), 1, 16, 1e-8, L.options(engine=1))
     with pytest.raises(L.LogDetError) as e:
