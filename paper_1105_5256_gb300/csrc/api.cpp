@@ -78,9 +78,12 @@ struct DevBuf {
     cudaError_t alloc(size_t b) {
         if (p) cudaFree(p);
         p = nullptr;
-        bytes = b;
+        bytes = 0;          // and after a failure: callers compare it with what they need
         if (b == 0) return cudaSuccess;
-        return cudaMalloc(&p, b);
+        const cudaError_t e = cudaMalloc(&p, b);
+        if (e == cudaSuccess) bytes = b;
+        else p = nullptr;
+        return e;
     }
     template <class X>
     X *as() const { return static_cast<X *>(p); }
