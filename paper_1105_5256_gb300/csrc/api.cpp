@@ -689,14 +689,18 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         invalidate_graph(c);
     }
     std::unique_lock<std::mutex> coop;
-    // the resident engine takes what it has a plan for unless the caller chose an engine or a pass
+    // the resident engine takes what it has a plan for unless the caller chose an engine or a pass,
+    // or there is no memory for its exchange buffers (the other engines' vectors are there)
     bool resident = false;
+    auto room = [](DevBuf &d, size_t bytes) {
+        if (bytes <= d.bytes || d.alloc(bytes) == cudaSuccess) return true;
+        cudaGetLastError();
+        return false;
+    };
     if (c->kind == LD_CSR) {
         if (c->res_state[0] == 1 && c->nshift <= (c->auto_shift ? 64 : c->nshift)) {
             const size_t hb = (size_t)c->csr_plan.J * 2 * c->n * c->csr_plan.T * (c->opt.precision == LD_FP64 ? 8 : 4);
-            if (!c->d_res_rec.p) CUDA_TRY(c->d_res_rec.alloc(ld::engine_csr_rec_bytes(c->csr_plan)));
-            if (!c->d_res_halo.p) CUDA_TRY(c->d_res_halo.alloc(hb));
-            resident = true;
+            resident = room(c->d_res_rec, ld::engine_csr_rec_bytes(c->csr_plan)) && room(c->d_res_halo, hb);
         }
     } else if (c->opt.engine == 0 && c->opt.lattice_pass == 0 && !ru) {
         int &state = c->res_state[want_x0];
@@ -705,9 +709,7 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         if (state == 1) {
             const size_t rb = ld::engine_resident_rec_bytes(c->res_plan[want_x0]);
             const size_t hb = ld::engine_resident_halo_bytes(c->res_plan[want_x0]);
-            if (rb > c->d_res_rec.bytes) CUDA_TRY(c->d_res_rec.alloc(rb));
-            if (hb > c->d_res_halo.bytes) CUDA_TRY(c->d_res_halo.alloc(hb));
-            resident = true;
+            resident = room(c->d_res_rec, rb) && room(c->d_res_halo, hb);
         }
     }
     if (test_wait_ns > 0) {
@@ -1228,28 +1230,6 @@ static ld_status create_context(const ld_matrix *Q, int colouring_distance, int 
             CUDA_TRY(cudaMemcpy(c->d_val_f.p, vf.data(), nnz * sizeof(float), cudaMemcpyHostToDevice));
         }
     }
-    if (c->kind == LD_CSR && opt.engine == 0 && opt.reliable_delta == 0.0) {
-        // the resident engine's row split and local column numbers
-        std::vector<int32_t> row0, ext0, ext;
-        std::vector<uint16_t> lcol;
-        const bool fits = ld::engine_csr_plan(c->n, Q->rowptr, Q->colidx, f32 ? 1 : 0, c->ncolours,
-                                              c->auto_shift ? 64 : c->nshift, &c->csr_plan, row0, ext0, ext, lcol) == 0;
-        c->res_state[0] = c->res_state[1] = fits ? 1 : 2;
-        if (fits) {
-            auto put = [](DevBuf &d, const void *src, size_t bytes) {
-                cudaError_t e = d.alloc(std::max<size_t>(bytes, 16));
-                return e != cudaSuccess || bytes == 0 ? e : cudaMemcpy(d.p, src, bytes, cudaMemcpyHostToDevice);
-            };
-            CUDA_TRY(put(c->d_csr_row0, row0.data(), row0.size() * 4));
-            CUDA_TRY(put(c->d_csr_ext0, ext0.data(), ext0.size() * 4));
-            CUDA_TRY(put(c->d_csr_ext, ext.data(), ext.size() * 4));
-            CUDA_TRY(put(c->d_csr_lcol, lcol.data(), lcol.size() * 2));
-            c->csr_plan.row0 = c->d_csr_row0.as<int32_t>();
-            c->csr_plan.ext0 = c->d_csr_ext0.as<int32_t>();
-            c->csr_plan.ext = c->d_csr_ext.as<int32_t>();
-            c->csr_plan.lcol = c->d_csr_lcol.as<uint16_t>();
-        }
-    }
     // work buffers
     const size_t w = f32 ? 4 : 8;
     const size_t vb = (size_t)c->ntiles * c->n * c->T * w;
@@ -1318,6 +1298,37 @@ static ld_status create_context(const ld_matrix *Q, int colouring_distance, int 
     CUDA_TRY(c->d_partial.alloc(part * sizeof(double)));
     s.partial = c->d_partial.as<double>();
     CUDA_TRY(cudaMemset(c->d_tile.p, 0, c->d_tile.bytes));
+
+    if (c->kind == LD_CSR && opt.engine == 0 && opt.reliable_delta == 0.0) {
+        // the resident engine's row split and local column numbers, if there is room beside the
+        // vectors of the other engines
+        std::vector<int32_t> row0, ext0, ext;
+        std::vector<uint16_t> lcol;
+        bool fits = ld::engine_csr_plan(c->n, Q->rowptr, Q->colidx, f32 ? 1 : 0, c->ncolours,
+                                        c->auto_shift ? 64 : c->nshift, &c->csr_plan, row0, ext0, ext, lcol) == 0;
+        if (fits) {
+            struct Table { DevBuf &d; const void *src; size_t bytes; };
+            const Table tables[] = {{c->d_csr_row0, row0.data(), row0.size() * 4}, {c->d_csr_ext0, ext0.data(), ext0.size() * 4},
+                                    {c->d_csr_ext, ext.data(), ext.size() * 4}, {c->d_csr_lcol, lcol.data(), lcol.size() * 2}};
+            for (const Table &t : tables) {
+                const cudaError_t e = t.d.alloc(std::max<size_t>(t.bytes, 16));
+                if (e == cudaErrorMemoryAllocation) {
+                    cudaGetLastError();
+                    fits = false;
+                    break;
+                }
+                CUDA_TRY(e);
+                CUDA_TRY(cudaMemcpy(t.d.p, t.src, t.bytes, cudaMemcpyHostToDevice));
+            }
+            if (!fits)
+                for (const Table &t : tables) t.d.alloc(0);
+            c->csr_plan.row0 = c->d_csr_row0.as<int32_t>();
+            c->csr_plan.ext0 = c->d_csr_ext0.as<int32_t>();
+            c->csr_plan.ext = c->d_csr_ext.as<int32_t>();
+            c->csr_plan.lcol = c->d_csr_lcol.as<uint16_t>();
+        }
+        c->res_state[0] = c->res_state[1] = fits ? 1 : 2;
+    }
 
     if (ld_status b = compute_bounds(c)) return b;
     if (ld_status nd = set_nodes(c)) return nd;

@@ -14,10 +14,10 @@ torch = pytest.importorskip("torch")
 def hold_all_but(free_bytes):
     """Device memory held until at most free_bytes are left (never touched)."""
     held = []
-    for chunk in (1 << 30, 1 << 24, 1 << 21):
-        while torch.cuda.mem_get_info()[0] - chunk >= free_bytes:
-            k = (torch.cuda.mem_get_info()[0] - free_bytes) // chunk if chunk == 1 << 30 else 1
-            held.append(torch.empty(int(k) * chunk, dtype=torch.uint8, device="cuda"))
+    for left in (free_bytes + (256 << 20), free_bytes):      # the second piece is large enough not to be rounded up
+        size = (torch.cuda.mem_get_info()[0] - left) >> 21 << 21
+        held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+    assert torch.cuda.mem_get_info()[0] <= free_bytes + (4 << 20)
     return held
 
 
@@ -40,3 +40,26 @@ def test_vector_form_without_room_for_its_records_streams_every_time():
         torch.cuda.empty_cache()
     Y, info = L.ld_logmv(ctx, V)
     assert info["engine"] == 4 and np.linalg.norm(Y - ref) <= 50e-9 * np.linalg.norm(ref)
+
+
+def test_a_solve_without_room_for_its_exchange_buffers_takes_the_other_engine():
+    p, t = synth.perturbed_triangulation(6, 141, 97)
+    from paper_1105_5256_gb300 import mesh
+    rp, ci, vv = mesh.spde_csr(p, t, 0.3 * 140 * 96, 2, 1.0)
+    lo, hi = L.ld_csr_bounds(rp, ci, vv)
+    make = lambda engine: L.ld_create(L.csr_matrix(rp, ci, vv), 2, 16, 1e-6,
+                                      L.options(engine=engine, lambda_min=lo, lambda_max=hi))
+    ref, info = L.ld_logdet(make(2))
+    assert info["engine"] == 2
+    ctx = make(0)                                # w of every team's vectors: 7 MB, allocated by the first solve
+    torch.cuda.empty_cache()
+    held = hold_all_but(4 << 20)
+    try:
+        for _ in range(2):
+            v, info = L.ld_logdet(ctx)
+            assert info["engine"] == 2 and abs(v - ref) <= 50e-6 * abs(ref)
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    v, info = L.ld_logdet(ctx)
+    assert info["engine"] == 4 and abs(v - ref) <= 50e-6 * abs(ref)
