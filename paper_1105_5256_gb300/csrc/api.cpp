@@ -155,7 +155,7 @@ struct ld_ctx {
     DevBuf d_vec;                 // vector form on chip: one workspace, kept while it is small
     ld::ResPlan vec_plan{};       // its plan for vec_ncols columns and vec_nshift nodes (0: none yet)
     int vec_ncols = 0, vec_nshift = 0;
-    bool vec_fits = false;
+    bool vec_fits = false, vec_over = false;   // vec_over: a call on these parameters overran its records
     int32_t *h_pinned = nullptr;  // remaining, status
     bool have_x0 = false;
     int last_cb = 0, last_ce = 0;
@@ -1435,6 +1435,7 @@ ld_status ld_set_params(ld_ctx *c, double kappa2, double tau, double scale) {
     invalidate_graph(c);
     c->solved = false;
     c->have_x0 = false;
+    c->vec_over = false;
     if (!c->user_bounds) {
         if (ld_status b = compute_bounds(c)) return b;
     }
@@ -1590,8 +1591,9 @@ ld_status ld_apply(ld_ctx *c, int ncols, const double *x, double *y) {
 // Vector form on chip (see engine_resident_funmv): false in *taken leaves the call to the
 // streaming form (no plan, or more iterations than the records hold).
 static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y, ld_info *info,
-                                const double2 *weight_dev, bool *taken) {
+                                const double2 *weight_dev, bool *taken, int64_t *launched) {
     *taken = false;
+    *launched = 0;
     if (c->opt.engine != 0 || c->opt.lattice_pass != 0 || c->kind == LD_CSR) return LD_OK;
     const int N = c->nshift;
     const int64_t n = c->n;
@@ -1606,8 +1608,9 @@ static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y
         c->vec_fits = ld::engine_resident_plan_vec(s, ncols, &c->vec_plan) == 0;
         c->vec_ncols = ncols;
         c->vec_nshift = N;
+        c->vec_over = false;
     }
-    if (!c->vec_fits) return LD_OK;
+    if (!c->vec_fits || c->vec_over) return LD_OK;
     const ld::ResPlan &plan = c->vec_plan;
     const int max_iter = c->opt.max_iter > 0 ? c->opt.max_iter : 100000;
     // records of every iteration's shift scalars: within the streaming form's shifted directions
@@ -1674,7 +1677,14 @@ static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y
     CUDA_TRY(cudaMemcpyAsync(it.data(), s.col_iters, C * sizeof(int32_t), cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     int remaining = c->h_pinned[0], status = c->h_pinned[1];
-    if (status == ld::DEV_OVERFLOW && hcap < max_iter) return LD_OK;      // nothing written: the streaming form
+    if (status == ld::DEV_OVERFLOW && hcap < max_iter) {
+        // Nothing written: the streaming form, with the records' memory (its shifted directions
+        // take as much), and without another attempt while the parameters stay.
+        c->vec_over = true;
+        *launched = 2;
+        CUDA_TRY(c->d_vec.alloc(0));
+        return LD_OK;
+    }
     if (status == ld::DEV_OVERFLOW) status = 0;                            // max_iter itself
     *taken = true;
     int64_t launches = 2;
@@ -1718,7 +1728,8 @@ static ld_status funmv(ld_ctx *c, int ncols, const double *V, double *Y, ld_info
     if (c->is_batch) return fail(LD_EINVAL, "batched context");
     REJECT_MATFREE(c);
     bool taken = false;
-    if (ld_status st = funmv_resident(c, ncols, V, Y, info, weight_dev, &taken)) return st;
+    int64_t launched = 0;         // by an attempt on chip that ran out of records
+    if (ld_status st = funmv_resident(c, ncols, V, Y, info, weight_dev, &taken, &launched)) return st;
     if (taken) return LD_OK;
     const int T = c->T, N = c->nshift;
     const int nt = (ncols + T - 1) / T, C = nt * T;
@@ -1792,7 +1803,7 @@ static ld_status funmv(ld_ctx *c, int ncols, const double *V, double *Y, ld_info
     ENGINE_TRY(ld::engine_modev(s, 0, 0, psig.as<double2>(), y.as<double>(), c->stream));
     const int max_iter = c->opt.max_iter > 0 ? c->opt.max_iter : 100000;
     int it = 0, remaining = 1, status = 0;
-    int64_t launches = 5;
+    int64_t launches = 5 + launched;
     while (it < max_iter && remaining > 0 && status == 0) {
         for (int k = 0; k < 16 && it < max_iter; ++k, ++it) {
             ENGINE_TRY(ld::engine_iteration(s, it & 1, c->stream));

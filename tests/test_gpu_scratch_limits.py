@@ -63,3 +63,26 @@ def test_a_solve_without_room_for_its_exchange_buffers_takes_the_other_engine():
         torch.cuda.empty_cache()
     v, info = L.ld_logdet(ctx)
     assert info["engine"] == 4 and abs(v - ref) <= 50e-6 * abs(ref)
+
+
+def test_vector_form_that_overruns_its_records_streams_at_once_from_then_on():
+    """Records for n / 3 iterations here (1500 columns of 240 vertices), fewer than the solve takes."""
+    dims, ncols = (16, 15), 1500
+    n = int(np.prod(dims))
+    V = synth.random_probe_block(3, n, ncols)
+    make = lambda engine, k2: L.ld_create(L.grid_matrix(L.LD_STENCIL_2D13_SQ, dims, k2), 1, 20, 1e-10, L.options(engine=engine))
+    Y1, info1 = L.ld_logmv(make(1, 1e-4), V)
+    assert info1["iters"] > n // 3
+    ctx = make(0, 1e-4)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    Y, first = L.ld_logmv(ctx, V)
+    assert first["engine"] != 4 and np.linalg.norm(Y - Y1) <= 50e-10 * np.linalg.norm(Y1)
+    assert free - torch.cuda.mem_get_info()[0] < 64 << 20          # the records took 115 MB
+    Y, second = L.ld_logmv(ctx, V)
+    assert second["gpu_launches"] == first["gpu_launches"] - 2     # no attempt on chip any more
+    assert np.linalg.norm(Y - Y1) <= 50e-10 * np.linalg.norm(Y1)
+    L.ld_set_params(ctx, 50.0, 0.0, 1.0)
+    Y, info = L.ld_logmv(ctx, V)
+    W, _ = L.ld_logmv(make(1, 50.0), V)
+    assert info["engine"] == 4 and np.linalg.norm(Y - W) <= 50e-10 * np.linalg.norm(W)
