@@ -329,6 +329,12 @@ ld_status ld_wait_selftest(int64_t limit_ns);
  * context stays usable.  LD_EUNSUPPORTED: the context's solves use no cooperative teams. */
 ld_status ld_team_wait_selftest(ld_ctx *ctx, int64_t limit_ns);
 
+/* The scalar step of the resident engines on count (1 .. 2^24) given sets of dots, host
+ * arrays of 4 doubles a set: {|r|^2, p.w, r.w, |w|^2} -> {alpha, beta, predicted
+ * |r_{k+1}|^2, ld_status (0, LD_ENOTSPD or LD_ENUMERIC)}, w = Q p.  Exposed so that its
+ * quotients can be compared with the host's. */
+ld_status ld_scalar_selftest(int64_t count, const double *dots, double *out);
+
 /* Host utilities (no device work; usable without a GPU). */
 
 /* Greedy distance-d colouring of the CSR pattern in natural order (Sec. 2.1).

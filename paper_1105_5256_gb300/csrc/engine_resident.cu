@@ -292,6 +292,27 @@ int engine_resident_wait_selftest(uint64_t limit_ns, void *rec_dev, int32_t *sta
     return (int)cudaGetLastError();
 }
 
+// one warp an item: {rr, pw, rw, ww} -> {alpha, beta, rho, code}
+__global__ void k_resident_scalar_selftest(int64_t count, const double *dots, double *out) {
+    for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
+        const double *d = dots + 4 * q;
+        double na, nb, rho;
+        const int code = res_scalars(d[0], d[1], d[2], d[3], na, nb, rho);
+        if (threadIdx.x == 0) {
+            out[4 * q] = na;
+            out[4 * q + 1] = nb;
+            out[4 * q + 2] = rho;
+            out[4 * q + 3] = (double)code;
+        }
+    }
+}
+
+int engine_resident_scalar_selftest(int64_t count, const double *dots_dev, double *out_dev, void *stream) {
+    k_resident_scalar_selftest<<<(unsigned)std::min<int64_t>(count, 1 << 16), 32, 0, static_cast<cudaStream_t>(stream)>>>(
+        count, dots_dev, out_dev);
+    return (int)cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ vector form
 // y = Re sum_l w_l x^{sigma_l}, every x^{sigma_l} a combination of the seed residuals r_k:
 // with p_0 = r_0, p_{k+1} = zeta_{k+1} r_{k+1} + beta_k p_k, x += alpha_k p_k per shift, the

@@ -207,6 +207,8 @@ int engine_finish(const Solve &s, int col_begin, int col_end, void *stream);
 int engine_apply(const Operator &op, int precision, int T, int ntiles, const void *x, void *y,
                  void *stream);
 int engine_grad_params(const Solve &s, int nparam, const int *ids, double *out_dev, void *stream);
+// the resident engines' scalar step on given dots: {rr, pw, rw, ww} -> {alpha, beta, rho, DEV_ code}
+int engine_resident_scalar_selftest(int64_t count, const double *dots_dev, double *out_dev, void *stream);
 // one CTA waits on an mbarrier nothing arrives at, giving up after limit_ns: writes
 // DEV_TIMEOUT (or DEV_OK) to *status_dev
 int engine_wait_selftest(uint64_t limit_ns, int32_t *status_dev, void *stream);
