@@ -333,7 +333,10 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
             // partials [par][warp][vector][dot]
             double *pp = part + ((size_t)par * NW + wid) * 5 * T;
             constexpr int NS = group_sum_left(5 * E, NG);
-            V v[5 * E], sum[NS];
+            // beyond a thread's rows the sums of FP32 vectors keep their rounding errors, as the
+            // streaming product's do in FP64
+            V v[5 * E];
+            std::conditional_t<sizeof(V) == 8, double, Sum2> sum[NS];
 #pragma unroll
             for (int k = 0; k < 5 * E; ++k) v[k] = d[k % 5].v[k / 5];
             int at = 0, end = 5 * E;
