@@ -818,20 +818,13 @@ struct ResidualLauncher {
             if (e) return e;
         }
         if constexpr (KIND == KIND_2D5 || KIND == KIND_3D7) {
-            // segments of the marching axis: about eight blocks an SM, at least 16 positions each
-            constexpr bool D3 = KIND == KIND_3D7;
-            const int nm = D3 ? s.op.nz : s.op.ny, yb = D3 ? (s.op.ny + 7) / 8 : 1;
-            const int W = (D3 ? 1 : 8) * (s.xhi ? 31 : 32), xb = (s.op.nx + W - 1) / W;
-            int64_t segs = (int64_t)152 * 8 / std::max<int64_t>(1, (int64_t)xb * yb * s.ntiles);
-            segs = std::max<int64_t>(1, std::min<int64_t>(segs, (nm + 15) / 16));
-            while (segs * yb > 65535) segs = (segs + 1) / 2;
-            const int seg = (int)((nm + segs - 1) / segs);
-            if (yb <= 65535 && s.ntiles <= 65535) {
-                const dim3 grid(xb, (unsigned)(yb * ((nm + seg - 1) / seg)), s.ntiles);
+            const SweepGrid g = sweep_grid(KIND == KIND_3D7, s.xhi != nullptr, s.op.nx, s.op.ny, s.op.nz, s.ntiles);
+            if (g.ok) {
+                const dim3 grid(g.xb, g.by, s.ntiles);
                 if (s.xhi)
-                    k_residual_sweep<V, T, KIND, true><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, seg, norm2);
+                    k_residual_sweep<V, T, KIND, true><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, g.seg, norm2);
                 else
-                    k_residual_sweep<V, T, KIND, false><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, seg, norm2);
+                    k_residual_sweep<V, T, KIND, false><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, g.seg, norm2);
                 return (int)cudaGetLastError();
             }
         }

@@ -1,6 +1,7 @@
 // Index map of the true-residual sweep (k_residual_sweep in engine.cu), common to the kernel
 // and to the host test that walks every lane of it.
 #pragma once
+#include <algorithm>
 #include <cstdint>
 
 #include <cuda_runtime.h>
@@ -25,6 +26,29 @@ struct SweepLane {
         in = own || (DIFF && lane == 0 && gx + 1 < nx && (!D3 || gy < ny));
     }
 };
+
+// Launch of the sweep: xb x (yb * number of segments) blocks a tile; segments of the marching
+// axis for about eight blocks an SM, at least 16 positions each.  ok: the grid's y and z
+// extents hold it.
+struct SweepGrid {
+    int xb, yb, seg;
+    unsigned by;
+    bool ok;
+};
+inline SweepGrid sweep_grid(bool d3, bool diff, int nx, int ny, int nz, int ntiles) {
+    constexpr int64_t MAX = 65535;
+    SweepGrid g;
+    const int nm = d3 ? nz : ny, W = (d3 ? 1 : SWEEP_WARPS) * (diff ? 31 : 32);
+    g.xb = (nx + W - 1) / W;
+    g.yb = d3 ? (ny + SWEEP_WARPS - 1) / SWEEP_WARPS : 1;
+    int64_t segs = (int64_t)152 * 8 / std::max<int64_t>(1, (int64_t)g.xb * g.yb * ntiles);
+    segs = std::max<int64_t>(1, std::min<int64_t>(segs, (nm + 15) / 16));
+    while (segs > 1 && segs * g.yb > MAX) segs = (segs + 1) / 2;
+    g.seg = (int)((nm + segs - 1) / segs);
+    g.by = (unsigned)(g.yb * ((nm + g.seg - 1) / g.seg));
+    g.ok = g.yb <= MAX && ntiles <= MAX;
+    return g;
+}
 
 // The vertex at (x, y) of marching position m (nm of them): wrapped on a torus by one period,
 // -1 outside a Dirichlet grid.

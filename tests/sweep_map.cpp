@@ -35,8 +35,30 @@ static int walk(int nx, int ny, int nz, bool per) {
     return bad;
 }
 
+// The launch: its extents hold, its segments cover the marching axis, and it is given up (for the
+// gather kernel) exactly where its y blocks or tiles exceed a grid's extent.
+static int launch(bool d3, bool diff, int nx, int ny, int nz, int ntiles) {
+    const ld::SweepGrid g = ld::sweep_grid(d3, diff, nx, ny, nz, ntiles);
+    const int nm = d3 ? nz : ny, want = d3 ? (ny + 7) / 8 : 1;
+    int bad = g.ok != (want <= 65535 && ntiles <= 65535);
+    if (g.ok) {
+        const int segs = (int)g.by / g.yb;
+        bad += g.by < 1 || g.by > 65535 || (int)g.by % g.yb != 0;
+        bad += g.seg < 1 || (int64_t)segs * g.seg < nm || (int64_t)(segs - 1) * g.seg >= nm;
+    }
+    if (bad) std::printf("launch of %dx%dx%d, %d tiles: %d faults\n", nx, ny, nz, ntiles, bad);
+    return bad;
+}
+
 int main() {
     int bad = 0;
+    for (int diff = 0; diff < 2; ++diff)
+        for (int ntiles : {1, 3, 9, 152, 5000, 65535, 65536})
+            for (int nx : {1, 31, 32, 33, 500, 70000}) {
+                for (int ny : {1, 15, 16, 17, 333, 100000, 2000000}) bad += launch(false, diff, nx, ny, 1, ntiles);
+                for (int ny : {1, 8, 9, 333, 30000, 262144, 524279, 524280, 524281, 600000})
+                    for (int nz : {1, 2, 17, 400, 100000}) bad += launch(true, diff, nx, ny, nz, ntiles);
+            }
     for (int per = 0; per < 2; ++per) {
         for (int nx : {1, 2, 3, 5, 30, 31, 32, 33, 48, 61, 62, 63, 92, 93, 94, 100, 108, 109, 124, 200, 217, 218, 247, 248, 249, 300, 500})
             for (int ny : {1, 2, 7}) bad += walk<false, true>(nx, ny, 1, per) + walk<false, false>(nx, ny, 1, per);
