@@ -539,10 +539,11 @@ __global__ void __launch_bounds__(256) k_true_residual(Solve s, int set, int cb,
 // marches along the slowest axis with a register window, so that every x is loaded (and
 // widened) once and horizontal neighbours cross the lanes; in 3D eight warps own eight lines
 // in y and exchange them through shared memory.  Bound by the FP64 units (19 clocks a warp
-// instruction): with the seed solution in x_hi the difference form, its horizontal and
-// marching differences shared between neighbours, else the direct form, whose 1e-15 |x| is
-// far below what x in its own precision leaves.  Against the gather kernel above: 2048^2
-// with x_hi, 18 columns, 2.62 -> 1.75 ms; 128^3, x in FP32, 112 columns, 10.1 -> 5.6 ms.
+// instruction): where x is FP64 (FP64 vectors, or x_hi) the difference form, its horizontal and
+// marching differences shared between neighbours; for FP32 x the direct form, whose 1e-15 |x| is
+// far below what x in its own precision leaves (for FP64 x it is not: 4 + kappa^2 already loses
+// that much of kappa^2).  Against the gather kernel above: 2048^2 with x_hi, 18 columns,
+// 2.62 -> 1.75 ms; 128^3, x in FP32, 112 columns, 10.1 -> 5.6 ms.
 template <typename V, int T, int KIND, bool DIFF>
 __global__ void __launch_bounds__(256) k_residual_sweep(Solve s, int set, int cb, int ce, int replace, int seg,
                                                         double *norm2) {
@@ -818,12 +819,13 @@ struct ResidualLauncher {
             if (e) return e;
         }
         if constexpr (KIND == KIND_2D5 || KIND == KIND_3D7) {
-            const SweepGrid g = sweep_grid(KIND == KIND_3D7, s.xhi != nullptr, s.op.nx, s.op.ny, s.op.nz, s.ntiles);
+            const bool diff = sizeof(V) == 8 || s.xhi;
+            const SweepGrid g = sweep_grid(KIND == KIND_3D7, diff, s.op.nx, s.op.ny, s.op.nz, s.ntiles);
             if (g.ok) {
                 const dim3 grid(g.xb, g.by, s.ntiles);
-                if (s.xhi)
+                if (diff)
                     k_residual_sweep<V, T, KIND, true><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, g.seg, norm2);
-                else
+                else if constexpr (sizeof(V) == 4)
                     k_residual_sweep<V, T, KIND, false><<<grid, 256, 0, st>>>(s, set, cb, ce, replace, g.seg, norm2);
                 return (int)cudaGetLastError();
             }
