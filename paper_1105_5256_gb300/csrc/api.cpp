@@ -706,7 +706,8 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         int &state = c->res_state[want_x0];
         if (state == 0)
             state = ld::engine_resident_plan(c->s, c->ncolours, keep_x0, c->engine == 1, &c->res_plan[want_x0]) == 0 ? 1 : 2;
-        if (state == 1) {
+        const bool part = cb > 0 || ce < c->ncolours;
+        if (state == 1 && (!part || c->engine != 1 || ld::engine_resident_range(c->s, c->res_plan[want_x0], cb, ce))) {
             const size_t rb = ld::engine_resident_rec_bytes(c->res_plan[want_x0]);
             const size_t hb = ld::engine_resident_halo_bytes(c->res_plan[want_x0]);
             resident = room(c->d_res_rec, rb) && room(c->d_res_halo, hb);

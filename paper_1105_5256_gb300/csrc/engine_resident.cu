@@ -3,6 +3,7 @@
 #include "engine_resident.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace ld {
 
@@ -108,6 +109,39 @@ double stream_clocks(const Solve &s, int ncolours, bool keep_x0) {
     return (d3 ? 60000 : mat && keep_x0 ? 24000 : 32000) + vc * words * 4 / rate;
 }
 
+// Clocks of one streamed FP64 pass over `tiles` of the context's tiles: each block steps through
+// its rows (planes in 3D) at the latency of a step or, with enough blocks an SM, at the FP64
+// units' rate; a pass over few tiles has few blocks.  Fitted within 20 % to 400 passes over ranges
+// of 1 to all of 7 to 111 colours, 190^2 to 640^2 and 33^3 to 64^3, with and without x.
+double stream_range_clocks(const Solve &s, int tiles) {
+    const bool mat = s.op.kind == KIND_2D13_SQ, d3 = s.op.kind == KIND_3D7, x = s.keep_x0 != 0;
+    const double load = (double)tiles * s.bpt / 152.0;
+    const double lat = d3 ? 1970 * (x ? 1.22 : 1) + 1740 * (s.T - 1)
+                      : mat ? 2150 * (x ? 1.2 : 1) + 500 * (s.T - 1) : 1780 * (x ? 1.22 : 1) + 800 * (s.T - 1);
+    const double rate = load * s.T * (d3 ? 1664 * (x ? 1.09 : 1) : mat ? 920 * (x ? 1.12 : 1) : 812 * (x ? 1.07 : 1));
+    return (d3 ? 40700 : mat ? 24000 : 32000) + (s.seg + (mat ? 4 : 2)) * std::pow(std::pow(lat, 4) + std::pow(rate, 4), 0.25);
+}
+
+// Whether the grid engine's passes would take no longer than `clocks` on chip.  FP32: margins for
+// what the two estimates miss at the line.  3D FP32 bodies spill, and a CTA that takes nearly all
+// of the SM's shared memory leaves its spills no L1: measured 1.25 (1.6) times the estimate
+// without x, 1.05 (1.35) with it.  Measured there, resident against streamed, us: 3D 60^3, 45
+// columns 79 / 69, 130 x 20 x 50, 45, 61 / 59; 64^3, 45, 66 / 79; 3D FP64 60^3, 109, 806 / 748;
+// Matern 450^2, 53 columns, 45 / 42, 400^2, 53, 36 / 40.
+bool stream_faster(const Solve &s, const ResPlan &p, double clocks, int ncolours, bool keep_x0) {
+    const double stream = stream_clocks(s, ncolours, keep_x0);
+    const bool mat = s.op.kind == KIND_2D13_SQ, d3 = s.op.kind == KIND_3D7;
+    if (s.precision == 0) {
+        // the fit is to 3D passes whose blocks are partly padding; without any they are faster
+        const double pad = !d3 ? 2.0 : (double)((s.op.nx + P3X - 3) / (P3X - 2) * (P3X - 2)) / s.op.nx *
+                                           ((s.op.ny + P3Y - 3) / (P3Y - 2) * (P3Y - 2)) / s.op.ny;
+        return clocks >= std::min(1.0, 0.95 * pad) * stream;
+    }
+    if (clocks >= (mat ? 0.85 : 0.9) * stream) return true;
+    const bool full = p.smem > 196 * 1024;
+    return d3 && clocks * (keep_x0 ? (full ? 1.35 : 1.05) : (full ? 1.6 : 1.25)) >= stream;
+}
+
 template <class F>
 cudaError_t res_launch(const ResPlan &p, int missing, cudaStream_t st, F &&fn) {
     cudaLaunchConfig_t cfg{};
@@ -158,7 +192,9 @@ static int resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
                 continue;
             }
             const int rounds = (ncolours + act - 1) / act;
-            const double t = rounds * res_clocks(s, p, keep_x0);
+            p.clocks = res_clocks(s, p, keep_x0);
+            p.wide = act;
+            const double t = rounds * p.clocks;
             if (t < best) {
                 best = t;
                 *out = p;
@@ -182,7 +218,9 @@ static int resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
                 ok = true;
                 if (k != KIND_3D7) break;
             }
-            const double t = ok ? rounds * res_clocks(s, p, keep_x0) : 1e300;
+            p.clocks = ok ? res_clocks(s, p, keep_x0) : 1e300;
+            p.wide = J;
+            const double t = rounds * p.clocks;
             int occ = 0;
             if (t < best &&
                 cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, p.nt + 64, p.smem) == cudaSuccess &&
@@ -194,7 +232,7 @@ static int resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
     }
     cudaGetLastError();
     // contexts the grid engine would run: only where the passes would take longer
-    if (streams && best >= (s.precision == 0 ? 1.0 : 0.9) * stream_clocks(s, ncolours, keep_x0)) return 1;
+    if (streams && best < 1e300 && stream_faster(s, *out, best, ncolours, keep_x0)) return 1;
     return best < 1e300 ? 0 : 1;
 }
 
@@ -204,6 +242,16 @@ int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool stream
 
 int engine_resident_plan_vec(const Solve &s, int ncols, ResPlan *out) {
     return resident_plan(s, ncols, false, false, s.precision == 0 ? 4 : 8, out);
+}
+
+// FP32: a pass over few colours takes most of a pass over all (Matern 520^2, 19 colours: 30 us, 3
+// of them 25, against 12 on chip for up to ten), so the plan holds for every range.  FP64: fewer
+// blocks leave the streamed pass the FP64 units to itself (Matern 300^2, 19 colours: 77 us streamed, 59
+// on chip; 3 of them 33 and still 59).
+bool engine_resident_range(const Solve &s, const ResPlan &p, int cb, int ce) {
+    if (s.precision != 0 || ce <= cb) return true;
+    const int rounds = (ce - cb + p.wide - 1) / p.wide;
+    return rounds * p.clocks < stream_range_clocks(s, (ce + s.T - 1) / s.T - cb / s.T);
 }
 
 size_t engine_resident_rec_bytes(const ResPlan &p) {

@@ -125,6 +125,8 @@ struct ResPlan {
     int slots;            // halo lines of a CTA at most
     int yw;               // vector form: words of y per item in tensor memory (4 FP64, 8 FP32), else 0
     size_t smem;
+    double clocks;        // an iteration of its teams (estimate)
+    int wide;             // teams that run at once
 };
 constexpr uint64_t RES_WAIT_NS = 2000000000;   // limit of every device wait of the resident engines
 struct ResArgs {
@@ -151,6 +153,9 @@ int engine_resident_funmv(const Solve &s, const ResPlan &p, const ResArgs &a, in
 // 0 and a plan when the engine takes the solve; nonzero otherwise.  streams: the context
 // would otherwise run the grid engine, so the plan must beat its passes
 int engine_resident_plan(const Solve &s, int ncolours, bool keep_x0, bool streams, ResPlan *out);
+// whether the colours [cb, ce), not all of them, run faster on the plan than on the grid engine
+// the context would otherwise run (s planned for it)
+bool engine_resident_range(const Solve &s, const ResPlan &p, int cb, int ce);
 // batches: geometry of a cluster of M CTAs for one column (false: does not fit), estimated
 // clocks of an iteration, and the launches of one kind and cluster size
 constexpr int RES_BATCH_NT = 512;
