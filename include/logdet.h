@@ -342,6 +342,12 @@ ld_status ld_scalar_selftest(int64_t count, const double *dots, double *out);
 ld_status ld_colour_csr(int64_t n, const int64_t *rowptr, const int32_t *colidx, int d,
                         int32_t *colour, int32_t *n_colours);
 
+/* The resident engine's layout of a CSR matrix (row split, external columns) as ld_create makes it,
+ * for a GPU of sms SMs: *fits whether it takes the matrix, *n_ctas the CTAs of a team (or NULL),
+ * *scanned the matrix entries read to weigh candidates (or NULL). */
+ld_status ld_csr_layout(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int n_colours,
+                        int n_shifts, int sms, int32_t *fits, int32_t *n_ctas, int64_t *scanned);
+
 /* Nodes of ld_invsqrt_mv's rational z^{-1/2} on [lmin, lmax]: the log nodes' poles sigma
  * and weights beta_j = -(2 i h / pi) w'(t_j), interleaved (re, im), N each (2N doubles per
  * array).  LD_EINVAL unless 0 < lmin < lmax and 1 <= N <= 256. */

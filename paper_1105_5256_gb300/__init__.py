@@ -119,6 +119,7 @@ def library(build_if_missing: bool = False):
         "ld_team_wait_selftest": ([vp, i64], st),
         "ld_scalar_selftest": ([i64, vp, vp], st),
         "ld_invsqrt_mv": ([vp, C.c_int, vp, vp, P(Info)], st),
+        "ld_csr_layout": ([i64, vp, vp, C.c_int, C.c_int, C.c_int, C.c_int, P(i32), P(i32), P(i64)], st),
         "ld_colour_csr": ([i64, vp, vp, C.c_int, vp, P(i32)], st),
         "ld_colour_grid": ([C.c_int, vp, C.c_int, C.c_int, vp, P(i32)], st),
         "ld_hht_nodes": ([dbl, dbl, C.c_int, vp, vp, P(dbl)], st),
@@ -440,6 +441,17 @@ def ld_select_distance(ctx: Context, j: int, eps: float, max_d: int = 32):
     _check(library().ld_select_distance(ctx.handle, int(j), float(eps), int(max_d), C.byref(d),
                                         _ptr(prof), C.byref(info)))
     return int(d.value), prof, info.as_dict()
+
+
+def ld_csr_layout(rowptr, colidx, precision: int, n_colours: int, n_shifts: int, sms: int):
+    """Whether the resident engine takes the CSR pattern on a GPU of sms SMs: (fits, CTAs of a team,
+    matrix entries read to weigh candidates).  Host only."""
+    rp = np.ascontiguousarray(rowptr, dtype=np.int64)
+    ci = np.ascontiguousarray(colidx, dtype=np.int32)
+    fits, ctas, scanned = C.c_int32(), C.c_int32(), C.c_int64()
+    _check(library().ld_csr_layout(rp.size - 1, _ptr(rp), _ptr(ci), int(precision), int(n_colours), int(n_shifts),
+                                   int(sms), C.byref(fits), C.byref(ctas), C.byref(scanned)))
+    return bool(fits.value), ctas.value, scanned.value
 
 
 def ld_colour_csr(rowptr, colidx, d: int):

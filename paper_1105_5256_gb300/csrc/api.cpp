@@ -1959,6 +1959,22 @@ ld_status ld_select_distance(ld_ctx *c, int64_t j, double eps, int max_d, int32_
     return LD_OK;
 }
 
+ld_status ld_csr_layout(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int ncolours, int n_shifts,
+                        int sms, int32_t *fits, int32_t *n_ctas, int64_t *scanned) {
+    if (n < 1 || !rowptr || !colidx || !fits || ncolours < 1 || sms < 1 || n_shifts < 1 || n_shifts > 256)
+        return fail(LD_EINVAL, "bad arguments");
+    if (precision != LD_FP64 && precision != LD_MIXED) return fail(LD_EINVAL, "bad precision");
+    ld::CsrPlan p{};
+    std::vector<int32_t> r0, e0, e;
+    std::vector<uint16_t> lc;
+    int64_t sc = 0;
+    *fits = ld::engine_csr_layout(n, rowptr, colidx, precision == LD_MIXED ? 1 : 0, ncolours, n_shifts, sms, &p, r0, e0, e,
+                                  lc, &sc) == 0;
+    if (scanned) *scanned = sc;
+    if (n_ctas) *n_ctas = *fits ? p.M : 0;
+    return LD_OK;
+}
+
 ld_status ld_colour_csr(int64_t n, const int64_t *rowptr, const int32_t *colidx, int d,
                         int32_t *colour, int32_t *n_colours) {
     if (n < 1 || !rowptr || !colidx || !colour || d < 0) return fail(LD_EINVAL, "bad arguments");

@@ -49,16 +49,12 @@ static void csr_items(CsrPlan &p, int E) {
     p.rec_team = (size_t)2 * p.T * p.M * 6 + (size_t)2 * p.T * 4;
 }
 
-int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int ncolours, int nshift,
-                    CsrPlan *out, std::vector<int32_t> &row0, std::vector<int32_t> &ext0, std::vector<int32_t> &ext,
-                    std::vector<uint16_t> &lcol) {
+int engine_csr_layout(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int ncolours, int nshift,
+                      int sms, CsrPlan *out, std::vector<int32_t> &row0, std::vector<int32_t> &ext0,
+                      std::vector<int32_t> &ext, std::vector<uint16_t> &lcol, int64_t *scanned) {
     const int word = precision == 0 ? 8 : 4, E = 16 / word, nt = precision == 0 ? 256 : 512;
-    int dev = 0, sms = 0;
-    if (n < 2 || n >= (1ll << 30) || ncolours < 1 || cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-        cudaGetLastError();
-        return 1;
-    }
+    if (scanned) *scanned = 0;
+    if (n < 2 || n >= (1ll << 30) || ncolours < 1) return 1;
     const double avg = (double)rowptr[n] / (double)n;
     // Cost of a plan in clocks, by the warps' rows and external columns.  FP64: 19 a warp
     // instruction (entries, r, p, dots); FP32: the shared-memory wavefronts of the product
@@ -86,20 +82,26 @@ int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int
             p.T = T;
             p.nt = nt;
             // the largest CTA: every one of them for the rows and entries, a sample for the
-            // external columns (the layout below takes the true maximum)
+            // external columns (the layout below takes the true maximum), which is only drawn
+            // where the rows and entries alone would fit
             for (int m = 0; m < M; ++m) {
                 const int64_t a = n * m / M, b = n * (m + 1) / M;
                 p.own_max = std::max(p.own_max, (int)(b - a));
-                p.nnz_max = (int)std::max<int64_t>(p.nnz_max, rowptr[b] - rowptr[a]);
+                p.nnz_max = (int)std::min<int64_t>(std::max<int64_t>(p.nnz_max, rowptr[b] - rowptr[a]), INT32_MAX);
             }
+            const int room = 512 / (nt / 128) / 4;
+            auto fits = [&]() {
+                csr_items(p, E);
+                return 3 * p.items_own + p.items_ext <= room && p.own_max + p.ext_max <= 65000 &&
+                       csr_smem(p, word, nshift).bytes <= 227 * 1024;
+            };
+            if (!fits()) continue;
             for (int m : {0, M / 3, M / 2, M - 1}) {
                 external_columns(rowptr, colidx, n * m / M, n * (m + 1) / M, seen, stamp++, tmp);
+                if (scanned) *scanned += rowptr[n * (m + 1) / M] - rowptr[n * m / M];
                 p.ext_max = std::max(p.ext_max, (int)tmp.size());
             }
-            csr_items(p, E);
-            const int room = 512 / (nt / 128) / 4;
-            if (3 * p.items_own + p.items_ext > room || p.own_max + p.ext_max > 65000) continue;
-            if (csr_smem(p, word, nshift).bytes > 227 * 1024) continue;
+            if (!fits()) continue;
             auto clocks = [&](const CsrPlan &q) {
                 const double lanes = q.T / E / 32.0, own = std::ceil(q.own_max * lanes), ex = std::ceil(q.ext_max * lanes);
                 const double fixed = (precision == 0 ? 14500 : 13000) + 20.0 * M + 400.0 * J;
@@ -173,6 +175,22 @@ int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int
     if (3 * bp.items_own + bp.items_ext > 512 / (nt / 128) / 4 || bp.own_max + bp.ext_max > 65000) return 1;
     bp.smem = csr_smem(bp, word, nshift).bytes;
     if (bp.smem > 227 * 1024) return 1;
+    *out = bp;
+    return 0;
+}
+
+int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int ncolours, int nshift,
+                    CsrPlan *out, std::vector<int32_t> &row0, std::vector<int32_t> &ext0, std::vector<int32_t> &ext,
+                    std::vector<uint16_t> &lcol) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
+    }
+    CsrPlan bp{};
+    if (engine_csr_layout(n, rowptr, colidx, precision, ncolours, nshift, sms, &bp, row0, ext0, ext, lcol, nullptr)) return 1;
+    const int E = precision == 0 ? 2 : 4, nt = bp.nt;
     for (int T : {bp.T, bp.T2}) {
         if (T == 0) continue;
         const void *fn = csr_kernel(precision, T / E);

@@ -188,6 +188,10 @@ struct CsrPlan {
 int engine_csr_plan(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int ncolours, int nshift,
                     CsrPlan *out, std::vector<int32_t> &row0, std::vector<int32_t> &ext0, std::vector<int32_t> &ext,
                     std::vector<uint16_t> &lcol);
+// its host part for a GPU of sms SMs; scanned: matrix entries read to weigh candidates (may be null)
+int engine_csr_layout(int64_t n, const int64_t *rowptr, const int32_t *colidx, int precision, int ncolours, int nshift,
+                      int sms, CsrPlan *out, std::vector<int32_t> &row0, std::vector<int32_t> &ext0,
+                      std::vector<int32_t> &ext, std::vector<uint16_t> &lcol, int64_t *scanned);
 size_t engine_csr_rec_bytes(const CsrPlan &p);
 int engine_resident_csr(const Solve &s, const CsrPlan &p, const ResArgs &a, void *stream);
 
