@@ -4,6 +4,8 @@
 #include <algorithm>
 #include <cmath>
 #include <atomic>
+#include <new>
+#include <system_error>
 #include <thread>
 
 namespace ld {
@@ -143,26 +145,33 @@ int engine_csr_layout(int64_t n, const int64_t *rowptr, const int32_t *colidx, i
     std::vector<std::vector<int32_t>> lists(M);
     lcol.resize(rowptr[n]);
     std::atomic<int> next{0};
+    std::atomic<bool> failed{false};
     auto work = [&]() {
-        std::vector<int32_t> mark(n, -1), loc(n);
-        for (int m = next++; m < M; m = next++) {
-            const int64_t a = row0[m], b = row0[m + 1];
-            external_columns(rowptr, colidx, a, b, mark, m, lists[m]);
-            for (size_t k = 0; k < lists[m].size(); ++k) loc[lists[m][k]] = (int32_t)(b - a + k);
-            for (int64_t e = rowptr[a]; e < rowptr[b]; ++e) {
-                const int32_t j = colidx[e];
-                lcol[e] = (uint16_t)(j >= a && j < b ? j - a : loc[j]);
+        try {
+            std::vector<int32_t> mark(n, -1), loc(n);
+            for (int m = next++; m < M; m = next++) {
+                const int64_t a = row0[m], b = row0[m + 1];
+                external_columns(rowptr, colidx, a, b, mark, m, lists[m]);
+                for (size_t k = 0; k < lists[m].size(); ++k) loc[lists[m][k]] = (int32_t)(b - a + k);
+                for (int64_t e = rowptr[a]; e < rowptr[b]; ++e) {
+                    const int32_t j = colidx[e];
+                    lcol[e] = (uint16_t)(j >= a && j < b ? j - a : loc[j]);
+                }
             }
+        } catch (const std::bad_alloc &) {
+            failed = true;          // no plan: nothing leaves a thread or the C boundary
         }
     };
     const int nth = rowptr[n] > 200000 ? (int)std::min(8u, std::max(1u, std::thread::hardware_concurrency())) : 1;
-    if (nth == 1) {
-        work();
-    } else {
-        std::vector<std::thread> pool;
-        for (int k = 0; k < nth; ++k) pool.emplace_back(work);
-        for (std::thread &t : pool) t.join();
+    std::vector<std::thread> pool;
+    pool.reserve(nth);
+    try {
+        for (int k = 1; k < nth; ++k) pool.emplace_back(work);
+    } catch (const std::system_error &) {       // fewer helpers then
     }
+    work();
+    for (std::thread &t : pool) t.join();
+    if (failed) return 1;
     ext0.assign(M + 1, 0);
     ext.clear();
     bp.ext_max = 1;
