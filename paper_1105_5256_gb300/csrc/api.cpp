@@ -2325,8 +2325,8 @@ ld_status batch_build(int count, const ld_matrix *Qs, const int *distances, int 
 
 
 // Tile width and step cost of a batch, tuned once per batch shape and process: for every
-// candidate tile width the persistent launch runs 16 iterations of every instance (all in
-// the persistent engine); the fastest width wins, and its time gives the cost of one CTA
+// candidate tile width the persistent launch runs 16 iterations of every instance that the
+// resident engine does not take (all in the persistent engine); the fastest width wins, and its time gives the cost of one CTA
 // step (total lattice-row steps over the resident CTAs) for the engine split.
 std::map<std::string, std::pair<int, double>> g_batch_tune;
 
@@ -2368,13 +2368,19 @@ ld_status ld_batch_create(int count, const ld_matrix *Qs, const int *distances, 
     }
     const double default_step = 1.2e-6;   // one CTA step before any measurement
     // no tile width asked for: instances that fit run on the resident engine, and only the
-    // others need a tuned width
+    // others need a tuned width, tuned on them alone
     const bool resident = opt.tile_width == 0 && opt.engine == 0;
-    bool all_resident = resident;
-    for (int i = 0; i < count && all_resident; ++i) all_resident = resident_batch_fits(Qs[i], n_shifts, opt.precision);
-    int T = all_resident ? (opt.precision == LD_MIXED ? 2 : 1) : opt.tile_width;
+    std::vector<ld_matrix> tuned;
+    std::vector<int> tuned_d;
+    for (int i = 0; i < count; ++i)
+        if (!resident || !resident_batch_fits(Qs[i], n_shifts, opt.precision)) {
+            tuned.push_back(Qs[i]);
+            tuned_d.push_back(distances[i]);
+        }
+    const int nt = (int)tuned.size();
+    int T = nt == 0 ? (opt.precision == LD_MIXED ? 2 : 1) : opt.tile_width;
     double step_s = default_step;
-    const std::string key = batch_key(count, Qs, distances, n_shifts, opt.precision);
+    const std::string key = batch_key(nt, tuned.data(), tuned_d.data(), n_shifts, opt.precision);
     {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_batch_tune.find(key);
@@ -2392,8 +2398,8 @@ ld_status ld_batch_create(int count, const ld_matrix *Qs, const int *distances, 
             ld_options o = opt;
             o.max_iter = 16;
             ld_ctx *t = nullptr;
-            if (batch_build(count, Qs, distances, n_shifts, tol, o, cand[k], 0.0, false, &t) != LD_OK) continue;
-            std::vector<double> v(count);
+            if (batch_build(nt, tuned.data(), tuned_d.data(), n_shifts, tol, o, cand[k], 0.0, false, &t) != LD_OK) continue;
+            std::vector<double> v(nt);
             ld_info info{};
             ld_batch_logdet(t, v.data(), nullptr, &info);      // warm (usually LD_ENOTCONV)
             ld_batch_logdet(t, v.data(), nullptr, &info);
