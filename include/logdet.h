@@ -331,9 +331,9 @@ ld_status ld_team_wait_selftest(ld_ctx *ctx, int64_t limit_ns);
 
 /* The scalar step of the resident engines on count (1 .. 2^24) given sets of dots, host
  * arrays of 4 doubles a set: {|r|^2, p.w, r.w, |w|^2} -> {alpha, beta, predicted
- * |r_{k+1}|^2, ld_status (0, LD_ENOTSPD or LD_ENUMERIC)}, w = Q p.  Exposed so that its
- * quotients can be compared with the host's. */
-ld_status ld_scalar_selftest(int64_t count, const double *dots, double *out);
+ * |r_{k+1}|^2, ld_status (0, LD_ENOTSPD or LD_ENUMERIC)}, w = Q p, as for LD_FP64 or
+ * LD_MIXED vectors.  Exposed so that the quotients can be compared with the host's. */
+ld_status ld_scalar_selftest(int64_t count, int precision, const double *dots, double *out);
 
 /* Host utilities (no device work; usable without a GPU). */
 

@@ -117,7 +117,7 @@ def library(build_if_missing: bool = False):
         "ld_hutchinson": ([vp, C.c_int, vp, P(dbl), P(dbl), vp, P(Info)], st),
         "ld_wait_selftest": ([i64], st),
         "ld_team_wait_selftest": ([vp, i64], st),
-        "ld_scalar_selftest": ([i64, vp, vp], st),
+        "ld_scalar_selftest": ([i64, C.c_int, vp, vp], st),
         "ld_invsqrt_mv": ([vp, C.c_int, vp, vp, P(Info)], st),
         "ld_csr_layout": ([i64, vp, vp, C.c_int, C.c_int, C.c_int, C.c_int, P(i32), P(i32), P(i64)], st),
         "ld_colour_csr": ([i64, vp, vp, C.c_int, vp, P(i32)], st),
@@ -398,12 +398,12 @@ def ld_team_wait_selftest(ctx: Context, limit_ns: int):
     _check(library().ld_team_wait_selftest(ctx.handle, int(limit_ns)))
 
 
-def ld_scalar_selftest(dots: np.ndarray) -> np.ndarray:
+def ld_scalar_selftest(dots: np.ndarray, precision: int = LD_FP64) -> np.ndarray:
     """The resident engines' scalar step: rows {|r|^2, p.w, r.w, |w|^2} -> {alpha, beta, predicted
-    |r_{k+1}|^2, status}."""
+    |r_{k+1}|^2, status}, as for vectors of the precision."""
     dots = np.ascontiguousarray(dots, dtype=np.float64).reshape(-1, 4)
     out = np.empty_like(dots)
-    _check(library().ld_scalar_selftest(dots.shape[0], _ptr(dots), _ptr(out)))
+    _check(library().ld_scalar_selftest(dots.shape[0], int(precision), _ptr(dots), _ptr(out)))
     return out
 
 

@@ -1881,14 +1881,15 @@ ld_status ld_wait_selftest(int64_t limit_ns) {
     return fail(LD_ECUDA, "self-test kernels did not report (status %d, %d)", h[0], h[1]);
 }
 
-ld_status ld_scalar_selftest(int64_t count, const double *dots, double *out) {
+ld_status ld_scalar_selftest(int64_t count, int precision, const double *dots, double *out) {
     if (count < 1 || count > ((int64_t)1 << 24) || !dots || !out) return fail(LD_EINVAL, "bad arguments");
+    if (precision != LD_FP64 && precision != LD_MIXED) return fail(LD_EINVAL, "bad precision");
     DevBuf b;
     const size_t bytes = (size_t)count * 4 * sizeof(double);
     CUDA_TRY(b.alloc(2 * bytes));
     double *in = b.as<double>(), *res = in + 4 * count;
     CUDA_TRY(cudaMemcpy(in, dots, bytes, cudaMemcpyHostToDevice));
-    ENGINE_TRY(ld::engine_resident_scalar_selftest(count, in, res, nullptr));
+    ENGINE_TRY(ld::engine_resident_scalar_selftest(count, precision == LD_FP64, in, res, nullptr));
     CUDA_TRY(cudaMemcpy(out, res, bytes, cudaMemcpyDeviceToHost));
     return LD_OK;
 }

@@ -322,14 +322,16 @@ int engine_resident(const Solve &s, const ResPlan &p, const ResArgs &a, void *st
 // own barrier that nobody completes (bit 1).
 __global__ void k_resident_wait_selftest(uint64_t limit_ns, const ulonglong2 *rec, int32_t *status) {
     __shared__ uint64_t bar;
+    __shared__ volatile uint64_t limit;
     if (threadIdx.x == 0) {
+        limit = limit_ns;
         mbar_init(&bar, 1);
         mbar_init_fence();
     }
     __syncthreads();
     double v;
-    const bool got = rec_wait(rec, 1, v, limit_ns);
-    const bool done = res_bar_wait(smem_u32(&bar), 0u, limit_ns);
+    const bool got = rec_wait(rec, 1, v, &limit);
+    const bool done = res_bar_wait(smem_u32(&bar), 0u, &limit);
     __syncthreads();
     if (threadIdx.x == 0) *status = (got ? 0 : 1) | (done ? 0 : 2);
 }
@@ -341,11 +343,12 @@ int engine_resident_wait_selftest(uint64_t limit_ns, void *rec_dev, int32_t *sta
 }
 
 // one warp an item: {rr, pw, rw, ww} -> {alpha, beta, rho, code}
-__global__ void k_resident_scalar_selftest(int64_t count, const double *dots, double *out) {
+__global__ void k_resident_scalar_selftest(int64_t count, bool exact, const double *dots, double *out) {
     for (int64_t q = blockIdx.x; q < count; q += gridDim.x) {
         const double *d = dots + 4 * q;
         double na, nb, rho;
-        const int code = res_scalars(d[0], d[1], d[2], d[3], na, nb, rho);
+        const int code = exact ? res_scalars<true>(d[0], d[1], d[2], d[3], na, nb, rho)
+                              : res_scalars<false>(d[0], d[1], d[2], d[3], na, nb, rho);
         if (threadIdx.x == 0) {
             out[4 * q] = na;
             out[4 * q + 1] = nb;
@@ -355,9 +358,9 @@ __global__ void k_resident_scalar_selftest(int64_t count, const double *dots, do
     }
 }
 
-int engine_resident_scalar_selftest(int64_t count, const double *dots_dev, double *out_dev, void *stream) {
+int engine_resident_scalar_selftest(int64_t count, bool exact, const double *dots_dev, double *out_dev, void *stream) {
     k_resident_scalar_selftest<<<(unsigned)std::min<int64_t>(count, 1 << 16), 32, 0, static_cast<cudaStream_t>(stream)>>>(
-        count, dots_dev, out_dev);
+        count, exact, dots_dev, out_dev);
     return (int)cudaGetLastError();
 }
 

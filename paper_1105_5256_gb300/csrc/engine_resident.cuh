@@ -190,15 +190,14 @@ __device__ __forceinline__ double lane_sum(double v) {
 }
 
 // ---- the scalar chain of an iteration, every step of which the vector warps wait for.
-// FP64 compares and quotients cost as much as several adds here, so signs are read from the
-// bits and the quotients are formed from the hardware's 20-bit reciprocal estimate: one
-// third-order Householder step, y += y (e + e^2) with e = 1 - a y (2^-60 before its last
-// rounding), then q = b y with one correction by its exact residual, q += y (b - a q)
-// (Markstein 1990).  Before its last rounding q is off by at most 2^-51 of a unit in the last
-// place, so it is the correctly rounded quotient but where that is a tie to within 2^-51.
-// Without the correction a quotient is off by up to 1.5 units; it costs two dependent
-// instructions a quotient, about 1 % of an iteration (48 x 40 Matern FP64 7.02 -> 7.07 ms,
-// 300 x 200 Matern FP32 5.33 -> 5.37).
+// FP64 compares and quotients cost as much as several adds here (one warp's FP64 instruction takes
+// 64 clocks whatever it waits for), so signs are read from the bits and the quotients are formed
+// from the hardware's 20-bit reciprocal estimate by one third-order Householder step,
+// y += y (e + e^2) with e = 1 - a y (2^-60 before its last rounding).  b y is then off by up to 1.5
+// units in the last place.  For FP64 vectors (EXACT) one correction by its exact residual,
+// q += y (b - a q) (Markstein 1990), leaves 2^-51 of a unit before the last rounding: the correctly
+// rounded quotient but for ties that close; 0.13 us an iteration (48 x 40 Matern 8.26 -> 8.39).  FP32
+// vectors round alpha and beta to FP32, and their dots are FP32 sums: there the 1.5 units stay.
 __device__ __forceinline__ bool res_positive(double v) {           // v > 0
     const long long b = __double_as_longlong(v);
     return b > 0 && b <= 0x7ff0000000000000ll;
@@ -213,12 +212,16 @@ __device__ __forceinline__ double res_recip(double a) {
     return fma(y, fma(e, e, e), y);
 }
 // b / a, y = res_recip(a)
+template <bool EXACT>
 __device__ __forceinline__ double res_quotient(double b, double a, double y) {
     const double q = b * y;
-    return fma(y, fma(-a, q, b), q);
+    return EXACT ? fma(y, fma(-a, q, b), q) : q;
 }
+// outside the plain range; a function of its own to keep its code out of the loop's
+static __device__ __noinline__ double res_divide(double b, double a) { return b / a; }
 // alpha, beta and the predicted |r_{k+1}|^2 of one iteration from its dots; all lanes alike.
 // Returns a DEV_ code or 0.
+template <bool EXACT>
 __device__ __forceinline__ int res_scalars(double rr, double pw, double rw, double ww, double &na, double &nb, double &rho) {
     const int lane = threadIdx.x & 31;
     na = nb = 0.0;
@@ -230,14 +233,14 @@ __device__ __forceinline__ int res_scalars(double rr, double pw, double rw, doub
     if (plain) {
         // lane 1 takes 1 / rr while lane 0 takes 1 / pw
         const double y = res_recip(lane & 1 ? rr : pw);
-        na = res_quotient(rr, pw, __shfl_sync(0xffffffffu, y, 0));
+        na = res_quotient<EXACT>(rr, pw, __shfl_sync(0xffffffffu, y, 0));
         irr = __shfl_sync(0xffffffffu, y, 1);
     } else {
-        na = rr / pw;
+        na = res_divide(rr, pw);
     }
     const double x = fma(na, fma(na, ww, m2), rr);
     rho = res_positive(x) ? x : 0.0;
-    if (res_positive(rr)) nb = plain ? res_quotient(rho, rr, irr) : rho / rr;
+    if (res_positive(rr)) nb = plain ? res_quotient<EXACT>(rho, rr, irr) : res_divide(rho, rr);
     return 0;
 }
 
@@ -260,18 +263,28 @@ __device__ __forceinline__ bool rec_ld(const ulonglong2 *p, unsigned long long t
     v = __longlong_as_double(a);
     return b == tag;
 }
-// wait for a record's tag; false after limit_ns
-__device__ __forceinline__ bool rec_wait(const ulonglong2 *p, unsigned long long tag, double &v, uint64_t limit_ns) {
-    if (rec_ld(p, tag, v)) return true;
+__device__ __forceinline__ uint64_t res_limit(const volatile uint64_t *limit_ns) { return limit_ns ? *limit_ns : RES_WAIT_NS; }
+// Wait for a record's tag; false after *limit_ns (in shared memory: a limit in a register of the
+// vector warps cost 1 %; null: RES_WAIT_NS).  The wait proper is a function of its own, out of the
+// scalar warp's loop: with x kept 300 x 200 Matern 7.12 -> 7.04 us an iteration.
+static __device__ __noinline__ bool rec_poll(const ulonglong2 *p, unsigned long long tag, double *out,
+                                             const volatile uint64_t *limit_ns) {
     uint64_t t0 = 0;
+    double v;
     for (unsigned it = 0;; ++it) {
-        if (rec_ld(p, tag, v)) return true;
+        if (rec_ld(p, tag, v)) {
+            *out = v;
+            return true;
+        }
         if ((it & 255) == 0) {
             const uint64_t t = global_ns();
             if (it == 0) t0 = t;
-            else if (t - t0 > limit_ns) return false;
+            else if (t - t0 > res_limit(limit_ns)) return false;
         }
     }
+}
+__device__ __forceinline__ bool rec_wait(const ulonglong2 *p, unsigned long long tag, double &v, const volatile uint64_t *limit_ns) {
+    return rec_ld(p, tag, v) || rec_poll(p, tag, &v, limit_ns);
 }
 
 // ---- private vectors in tensor memory: 16 bytes a lane, the warp's own 32 lanes
@@ -401,8 +414,8 @@ __device__ __forceinline__ void st_async(uint32_t addr, uint32_t bar, const ResI
                  "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(bar)
                  : "memory");
 }
-// wait for a phase of this CTA's mbarrier, with the remote stores it counted; false after limit_ns
-__device__ __forceinline__ bool res_bar_wait(uint32_t bar, unsigned parity, uint64_t limit_ns) {
+// wait for a phase of this CTA's mbarrier, with the remote stores it counted; false after *limit_ns
+__device__ __forceinline__ bool res_bar_wait(uint32_t bar, unsigned parity, const volatile uint64_t *limit_ns) {
     uint64_t t0 = 0;
     for (unsigned it = 0;; ++it) {
         unsigned ok;
@@ -416,7 +429,7 @@ __device__ __forceinline__ bool res_bar_wait(uint32_t bar, unsigned parity, uint
         if ((it & 63) == 0) {
             const uint64_t t = global_ns();
             if (it == 0) t0 = t;
-            else if (t - t0 > limit_ns) return false;
+            else if (t - t0 > res_limit(limit_ns)) return false;
         }
     }
 }
@@ -438,6 +451,7 @@ struct ResCtl {
     volatile int done;           // queue entries processed when the last column's shifts converged
     volatile int head, tail;     // queue entries posted, processed
     int bad;                     // a vector warp's wait ran out
+    volatile uint64_t wait_ns;   // limit of a wait
     uint64_t bar[2];             // exchange barriers by iteration parity
     double dflag[2];             // done flag of the team's first CTA, by parity
     double tot[4];               // the team's rr, pw, rw, ww
@@ -592,11 +606,13 @@ static __device__ __noinline__ void res_shift_role(const Solve &s, int stride, i
 }
 
 // ------------------------------------------------------------------ scalar warp
-template <int NT>
+// BATCH: every team is a cluster and the limits are literals, so the cooperative code goes (eight
+// lattices of 40^2 to 400^2: 13.3 -> 12.6 ms)
+template <int NT, bool EXACT, bool BATCH>
 __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team, int m,
                                              ResCtl *ctl, const double *part, int NP, unsigned in_bytes) {
     const int lane = threadIdx.x & 31, M = pl.M;
-    const bool clustered = pl.clustered;
+    const bool clustered = BATCH || pl.clustered;
     const double ds = s.precision == 0 ? s.op.scale : (double)s.op.scale_f;
     const double ds2 = ds * ds;
     const bool scaled = ds != 1.0;
@@ -630,7 +646,7 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
                     st_async(mapa(smem_u32(&ctl->dflag[par]), lane), mapa(smem_u32(&ctl->bar[par]), lane), fl);
             } else {
                 if (m == 0 && lane == 0) rec_st(rp + 5, fl, tag);
-                ok = rec_wait(rp + 5, tag, fl, ar.wait_ns);
+                ok = rec_wait(rp + 5, tag, fl, BATCH ? nullptr : &ctl->wait_ns);
             }
             bar_sync(3, 160);                 // the sums of vector warps 0 to 3
             if (clustered) {
@@ -651,7 +667,7 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
                 ww *= ds2;
             }
             double na, nb, rho;
-            const int ncode = res_scalars(rr, pw, rw, ww, na, nb, rho);
+            const int ncode = res_scalars<EXACT>(rr, pw, rw, ww, na, nb, rho);
             if (lane == 0) {
                 ctl->alpha = na;
                 ctl->beta = nb;
@@ -666,7 +682,7 @@ __device__ __noinline__ void res_scalar_role(const Solve &s, const ResPlan &pl, 
                     for (int q = lane; q < (clustered ? NP : M); q += 32) {
                         double v = 0.0;
                         if (clustered) v = pp[(size_t)4 * NP + q];
-                        else ok = rec_wait(rp + (size_t)q * 8 + 4, tag, v, ar.wait_ns) && ok;
+                        else ok = rec_wait(rp + (size_t)q * 8 + 4, tag, v, BATCH ? nullptr : &ctl->wait_ns) && ok;
                         vr_sum += v;
                     }
                     __syncwarp();
@@ -729,7 +745,7 @@ __device__ __noinline__ void res_replay_role(const Solve &s, const ResPlan &pl, 
             // a neighbour's rows may be here before this CTA's own warps have come that far
             bar_sync(3, NT + 32);
             if (clustered) {
-                ok = res_bar_wait(smem_u32(&ctl->bar[par]), (unsigned)(tick >> 1) & 1u, ar.wait_ns);
+                ok = res_bar_wait(smem_u32(&ctl->bar[par]), (unsigned)(tick >> 1) & 1u, &ctl->wait_ns);
                 __syncwarp();
                 if (lane == 0) mbar_arrive_tx(&ctl->bar[par], in_bytes);      // armed for tick + 2
             } else {
@@ -737,7 +753,7 @@ __device__ __noinline__ void res_replay_role(const Solve &s, const ResPlan &pl, 
                 ulonglong2 *rp = rec + (size_t)par * M * 8;
                 if (lane == 0) rec_st(rp + (size_t)m * 8, 0.0, tick + 1);
                 double v;
-                if (lane < 4 && bk.has[lane]) ok = rec_wait(rp + (size_t)bk.nb(lane) * 8, tick + 1, v, ar.wait_ns);
+                if (lane < 4 && bk.has[lane]) ok = rec_wait(rp + (size_t)bk.nb(lane) * 8, tick + 1, v, &ctl->wait_ns);
                 __threadfence();
             }
             if (!__all_sync(0xffffffffu, ok)) {
@@ -759,9 +775,10 @@ __device__ __noinline__ void res_replay_role(const Solve &s, const ResPlan &pl, 
 // ------------------------------------------------------------------ vector warps
 // RP: replay of a finished solve (vector form): alpha, beta from its records, no dots,
 // y += coef_k r_k
-template <typename V, int KIND, int NT, bool KX, bool RP>
+template <typename V, int KIND, int NT, bool KX, bool RP, bool BATCH>
 __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team, int m,
-                                                unsigned char *smem, const ResSmem &lay, ResCtl *ctl) {
+                                                unsigned char *smem, const ResSmem &lay, ResCtl *ctl,
+                                                const volatile uint64_t *limit_ns) {
     constexpr int E = res_epi<V>(), NW = NT / 32;
     constexpr bool MAT = KIND == KIND_2D13_SQ, D3 = KIND == KIND_3D7;
     constexpr int H = MAT ? 2 : 1, NB = D3 ? 6 : 4;
@@ -771,7 +788,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
     using It = ResItem<V>;
     using PM = PackMath<V, E>;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const bool clustered = pl.clustered;
+    const bool clustered = BATCH || pl.clustered;
     const int M = pl.M, G = pl.G, GE = G * E, pitch = pl.pitch, cmax = pl.cmax;
     const ResBlock<KIND> bk(s, pl, m);
     const int nx = bk.nx, L = bk.L, Ly = bk.Ly;
@@ -1302,7 +1319,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                         for (int q = lane & 3; q < M; q += 4) st_async(mapa(slot, q), mapa(bar_addr, q), tot);
                     }
                     if (wid < 4) {
-                        if (!res_bar_wait(bar_addr, (unsigned)(tick >> 1) & 1u, ar.wait_ns)) ctl->bad = 1;
+                        if (!res_bar_wait(bar_addr, (unsigned)(tick >> 1) & 1u, limit_ns)) ctl->bad = 1;
                         const double *pp = part + (size_t)(par * RES_NDOT + wid) * NP;
                         double a = lane < NP ? pp[lane] : 0.0;
                         for (int q = lane + 32; q < NP; q += 32) a += pp[q];
@@ -1342,7 +1359,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                                 if ((spin & 255) == 255) {
                                     const uint64_t t = global_ns();
                                     if (t0 == 0) t0 = t;
-                                    else if (t - t0 > ar.wait_ns) {
+                                    else if (t - t0 > res_limit(limit_ns)) {
                                         ok = false;
                                         break;
                                     }
@@ -1425,7 +1442,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
 
 // ------------------------------------------------------------------ kernel
 // NT vector threads, then the scalar warp and the shift warp
-template <typename V, int KIND, int NT, bool KX, bool RP>
+template <typename V, int KIND, int NT, bool KX, bool RP, bool BATCH>
 __device__ __forceinline__ void resident_body(const Solve &s, const ResPlan &pl, const ResArgs &ar, int team, int m,
                                               unsigned char *smem) {
     constexpr int NW = NT / 32;
@@ -1449,6 +1466,7 @@ __device__ __forceinline__ void resident_body(const Solve &s, const ResPlan &pl,
             ctl->done = 0;
             ctl->head = ctl->tail = 0;
             ctl->bad = 0;
+            ctl->wait_ns = ar.wait_ns;
             if (pl.clustered) {
                 mbar_init(&ctl->bar[0], 1);
                 mbar_init(&ctl->bar[1], 1);
@@ -1462,11 +1480,11 @@ __device__ __forceinline__ void resident_body(const Solve &s, const ResPlan &pl,
     __syncthreads();
     if (pl.clustered) cluster_sync_all();          // barriers armed before any remote store
     if (wid < NW)
-        res_vector_role<V, KIND, NT, KX, RP>(s, pl, ar, team, m, smem, lay, ctl);
+        res_vector_role<V, KIND, NT, KX, RP, BATCH>(s, pl, ar, team, m, smem, lay, ctl, BATCH ? nullptr : &ctl->wait_ns);
     else if (RP && wid == NW)
         res_replay_role<NT, KIND>(s, pl, ar, team, m, ctl, in_bytes);
     else if (wid == NW)
-        res_scalar_role<NT>(s, pl, ar, team, m, ctl, reinterpret_cast<const double *>(smem + lay.part), NP, in_bytes);
+        res_scalar_role<NT, sizeof(V) == 8, BATCH>(s, pl, ar, team, m, ctl, reinterpret_cast<const double *>(smem + lay.part), NP, in_bytes);
     else if (m == 0 && !RP)
         res_shift_role(s, pl.J, ar.cb + team, ar, ctl->q, &ctl->head, &ctl->tail, &ctl->done,
                        reinterpret_cast<double2 *>(smem + lay.shift));
@@ -1482,7 +1500,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident(const __grid_constant__
                                                          const __grid_constant__ ResArgs ar) {
     extern __shared__ __align__(16) unsigned char smem[];
     const int team = blockIdx.x / pl.M;
-    resident_body<V, KIND, NT, KX, RP>(s, pl, ar, team, blockIdx.x - team * pl.M, smem);
+    resident_body<V, KIND, NT, KX, RP, false>(s, pl, ar, team, blockIdx.x - team * pl.M, smem);
 }
 
 // A batch's items (instance, column) of one kind and cluster size: a cluster solves one item.
@@ -1504,7 +1522,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident_batch(const Solve *solv
     ar.ce = it.y + 1;
     ar.cap = cap;
     ar.terms = 1;
-    resident_body<V, KIND, NT, false, false>(s, pl, ar, 0, blockIdx.x % M, smem);
+    resident_body<V, KIND, NT, false, false, true>(s, pl, ar, 0, blockIdx.x % M, smem);
 }
 
 }  // namespace ld

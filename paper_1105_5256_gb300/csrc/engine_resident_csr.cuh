@@ -33,6 +33,7 @@ struct CsrCtl {
     uint32_t tm;
     volatile int done, head, tail;
     int bad;                     // a vector warp's wait ran out
+    volatile uint64_t wait_ns;   // limit of a wait
     ResCtl::Entry q[4];
     double alpha[RES_CSR_T], beta[RES_CSR_T];
     double tot[4];               // rr, pw, rw, ww of the vector this CTA owns
@@ -40,7 +41,7 @@ struct CsrCtl {
 static_assert(sizeof(CsrCtl) <= RES_CSR_CTL_BYTES, "control block");
 
 // ------------------------------------------------------------------ scalar warp
-template <int NT>
+template <int NT, bool EXACT>
 __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, const ResArgs &ar, int team, int m,
                                              CsrCtl *ctl) {
     const int lane = threadIdx.x & 31, M = pl.M, T = pl.T;
@@ -53,7 +54,7 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
     auto timed = [&](uint64_t &t0) -> bool {     // the limit, from the first call
         const uint64_t t = global_ns();
         if (t0 == 0) t0 = t;
-        return t - t0 > ar.wait_ns;
+        return t - t0 > ctl->wait_ns;
     };
     for (int c0 = ar.cb + team * T; c0 < ar.ce; c0 += pl.J * T) {
         const int c = c0 + m;
@@ -82,7 +83,7 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
                 fin = !live;
                 const double rr = ctl->tot[0], pw = ctl->tot[1], rw = ctl->tot[2], ww = ctl->tot[3];
                 rho = rr;
-                if (live) ncode = res_scalars(rr, pw, rw, ww, na, nb, rho);
+                if (live) ncode = res_scalars<EXACT>(rr, pw, rw, ww, na, nb, rho);
                 if (lane < 3) rec_st(rec2 + ((size_t)par * T + m) * 4 + lane, lane == 0 ? na : lane == 1 ? nb : (double)fin, tag);
             }
             // every vector's alpha, beta and finished flag
@@ -118,7 +119,7 @@ __device__ __noinline__ void csr_scalar_role(const Solve &s, const CsrPlan &pl, 
                     double vr_sum = 0.0;
                     for (int q = lane; q < M; q += 32) {
                         double v = 0.0;
-                        ok = rec_wait(rp + (size_t)q * 6 + 4, tag, v, ar.wait_ns) && ok;
+                        ok = rec_wait(rp + (size_t)q * 6 + 4, tag, v, &ctl->wait_ns) && ok;
                         vr_sum += v;
                     }
                     __syncwarp();
@@ -377,7 +378,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
                         if ((spin & 255) == 255) {
                             const uint64_t t = global_ns();
                             if (t0 == 0) t0 = t;
-                            else if (t - t0 > ar.wait_ns) {
+                            else if (t - t0 > ctl->wait_ns) {
                                 ok = false;
                                 break;
                             }
@@ -445,6 +446,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident_csr(const __grid_consta
             ctl->done = 0;
             ctl->head = ctl->tail = 0;
             ctl->bad = 0;
+            ctl->wait_ns = ar.wait_ns;
         }
         __syncwarp();
     }
@@ -452,7 +454,7 @@ __global__ void __launch_bounds__(NT + 64, 1) k_resident_csr(const __grid_consta
     if (wid < NW) {
         csr_vector_role<V, NG, NT>(s, pl, ar, team, m, smem, lay, ctl);
     } else if (wid == NW) {
-        csr_scalar_role<NT>(s, pl, ar, team, m, ctl);
+        csr_scalar_role<NT, sizeof(V) == 8>(s, pl, ar, team, m, ctl);
     } else if (m < pl.T) {
         res_shift_role(s, pl.J * pl.T, ar.cb + team * pl.T + m, ar, ctl->q, &ctl->head, &ctl->tail, &ctl->done,
                        reinterpret_cast<double2 *>(smem + lay.shift));

@@ -130,8 +130,6 @@ struct ResPlan {
 };
 constexpr uint64_t RES_WAIT_NS = 2000000000;   // limit of every device wait of the resident engines
 struct ResArgs {
-    uint64_t wait_ns;     // limit of a device wait: RES_WAIT_NS but in the self-test
-    int missing;          // self-test: CTAs of a cooperative launch left out at its end
     int cb, ce;           // colour range
     int cap;              // iterations at most
     int terms;            // 1: the shift warp also writes s.terms (batches)
@@ -145,6 +143,8 @@ struct ResArgs {
     double2 *hist;        // [column][iteration][shift][3]: alpha^sigma, beta^sigma, zeta
     double2 *ab;          // [column][iteration]: alpha, beta
     double *coef;         // [column][iteration]: y = sum_k coef_k r_k
+    uint64_t wait_ns;     // limit of a device wait: RES_WAIT_NS but in the self-test
+    int missing;          // self-test: CTAs of a cooperative launch left out at its end
 };
 // vector form on chip: y = Re sum_l weight_l (Q - sigma_l)^{-1} v for the columns of a.rhs;
 // plan with engine_resident_plan_vec.  DEV_OVERFLOW in *s.status: more than hcap iterations
@@ -217,7 +217,7 @@ int engine_apply(const Operator &op, int precision, int T, int ntiles, const voi
                  void *stream);
 int engine_grad_params(const Solve &s, int nparam, const int *ids, double *out_dev, void *stream);
 // the resident engines' scalar step on given dots: {rr, pw, rw, ww} -> {alpha, beta, rho, DEV_ code}
-int engine_resident_scalar_selftest(int64_t count, const double *dots_dev, double *out_dev, void *stream);
+int engine_resident_scalar_selftest(int64_t count, bool exact, const double *dots_dev, double *out_dev, void *stream);
 // one CTA waits on an mbarrier nothing arrives at, giving up after limit_ns: writes
 // DEV_TIMEOUT (or DEV_OK) to *status_dev
 int engine_wait_selftest(uint64_t limit_ns, int32_t *status_dev, void *stream);
