@@ -287,7 +287,8 @@ __device__ __forceinline__ bool rec_wait(const ulonglong2 *p, unsigned long long
     return rec_ld(p, tag, v) || rec_poll(p, tag, &v, limit_ns);
 }
 
-// ---- private vectors in tensor memory: 16 bytes a lane, the warp's own 32 lanes
+// ---- private vectors in tensor memory: 16 bytes a lane, the warp's own 32 lanes.  These are
+// .sync.aligned: a __syncwarp() stands between them and a branch on a thread's own lines or rows
 struct TmItem {
     uint32_t r[4];
 };
@@ -1015,6 +1016,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     TmItem tw[U], ta[PRIV ? U : 1];
                     V *line[U];
                     It old[U];
+                    __syncwarp();
 #pragma unroll
                     for (int k = 0; k < U; ++k) {
                         const int i = min(i0 + k, cmax - 1);
@@ -1030,20 +1032,23 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     for (int k = 0; k < U; ++k) {
                         const int i = i0 + k;
                         if (i >= items) break;
-                        const bool act = i < cnt;
                         const It wv = tm_get<V>(tw[k]);
                         if constexpr (RP) y_add(i, RS ? old[k] : tm_get<V>(ta[PRIV ? k : 0]), wv);
+                        It &next = old[k];          // r, or p
                         if constexpr (RS) {
-                            const It r = PM::fma(nas, wv, old[k]);
-                            if (act) put(line[k], g, r);
+                            next = PM::fma(nas, wv, old[k]);
                         } else {
                             if constexpr (keepx) x_add(i, aa, old[k]);
                             const It r = PM::fma(nas, wv, tm_get<V>(ta[k]));
                             tm_st<V>(tma + 4u * i, r);
-                            if (act) put(line[k], g, PM::fma(bb, old[k], r));
+                            next = PM::fma(bb, old[k], r);
                         }
                     }
+#pragma unroll
+                    for (int k = 0; k < U; ++k)
+                        if (i0 + k < cnt) put(line[k], g, old[k]);
                 }
+                __syncwarp();
                 tm_wait_st();
                 if (RP && it == last) break;          // y has its last term
                 const V *in = clustered ? HB + (size_t)(par ^ 1) * hstride : hglob + (size_t)(2 * m + (par ^ 1)) * hstride;
@@ -1171,6 +1176,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     l = row[-1];
                     r = row[E];
                 }
+                __syncwarp();
                 TmItem ta, td;
                 if constexpr (PRIV) tm_ld(ta, tma);
                 if (!MAT && d_tm) tm_ld(td, tmd);
@@ -1180,6 +1186,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     const bool act = i < cnt;
                     It cc;
                     const int in = min(i + 1, cmax - 1);
+                    if constexpr (!RS) __syncwarp();
                     if constexpr (PRIV) {
                         if (!MAT && d_tm) tm_wait(ta, td);
                         else tm_wait(ta);
@@ -1246,6 +1253,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     }
                     clip(wv);
                     if constexpr (RS) clip(rv);    // a torus ghost inside a partial item is not r
+                    __syncwarp();
                     tm_st<V>(tmw + 4u * i, wv);
                     if (act) {
                         if constexpr (!RP) {
@@ -1288,6 +1296,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     r = !D3 && rfix ? re : r2;
                     row = nrow;
                 }
+                __syncwarp();
                 if constexpr (PRIV) {
                     if (!MAT && d_tm) tm_wait(ta, td);     // the load past the last item
                     else tm_wait(ta);

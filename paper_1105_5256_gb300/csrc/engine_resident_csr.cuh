@@ -217,6 +217,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
                 r = init(colour[row] - c0);
                 ri_st(P + ((size_t)row * NG + g) * E, zz);
             }
+            __syncwarp();
             tm_st<V>(tmw + 4u * i, zz);
             tm_st<V>(tmr + 4u * i, r);
             if (keepx) tm_st<V>(tmx + 4u * i, zz);
@@ -228,6 +229,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
                 r = init(s.colour[pl.ext[e0 + q]] - c0);
                 ri_st(P + ((size_t)(own + q) * NG + g) * E, zz);
             }
+            __syncwarp();
             tm_st<V>(tme + 4u * i, r);
         }
         tm_wait_st();
@@ -253,6 +255,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
                 for (int k = 0; k < U; ++k) {
                     const int i = i0 + k, q = i * RS + rs;
                     if (i >= ie) break;
+                    __syncwarp();
                     TmItem tr;
                     tm_ld(tr, tme + 4u * i);
                     V *pp = P + ((size_t)(own + min(q, ext - 1)) * NG + g) * E;
@@ -266,6 +269,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
 #pragma unroll 2
             for (int i = 0; i < io; ++i) {
                 const int row = i * RS + rs;
+                __syncwarp();
                 TmItem tw, tr;
                 tm_ld(tw, tmw + 4u * i);
                 tm_ld(tr, tmr + 4u * i);
@@ -282,6 +286,7 @@ __device__ __forceinline__ void csr_vector_role(const Solve &s, const CsrPlan &p
                 }
                 if (row < own) ri_st(pp, PM::fma(be, old, r));
             }
+            __syncwarp();
             tm_wait_st();
             bar_sync(1, NT);
             // ---- w = Q p, dots
