@@ -648,7 +648,13 @@ ld_status matfree_grad(ld_ctx *c, int n_params, const int *ids, double *grad) {
     return LD_OK;
 }
 
-std::mutex g_coop_mu;   // cooperative resident solves of this process
+// cooperative resident solves of this process: one at a time on a device
+std::mutex &coop_mutex() {
+    static std::mutex mu[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+    return mu[dev & 63];
+}
 
 // One probed solve over colours [cb, ce).  On LD_OK, result[0..1] hold
 // sum of terms and sum of seed projections on the device and in *out.
@@ -754,9 +760,9 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         ra.rec = c->d_res_rec.as<ulonglong2>();
         ra.halo = c->d_res_halo.p;
         // Teams of a cooperative launch wait on one another, so two such launches must not share
-        // the SMs half each: one at a time in this process, until its results are here.
+        // the SMs half each: one at a time on a device, until its results are here.
         // (A cluster's CTAs are scheduled together: clustered plans need no such rule.)
-        if (c->kind == LD_CSR || !c->res_plan[want_x0].clustered) coop = std::unique_lock<std::mutex>(g_coop_mu);
+        if (c->kind == LD_CSR || !c->res_plan[want_x0].clustered) coop = std::unique_lock<std::mutex>(coop_mutex());
         // the engine writes the seed solutions of the colours it solves; the others' are zero
         if (keep_x0 && (cb > 0 || ce < c->ncolours)) CUDA_TRY(cudaMemsetAsync(c->d_x.p, 0, c->d_x.bytes, c->stream));
         CUDA_TRY(cudaEventRecord(c->ev2, c->stream));
@@ -1667,7 +1673,7 @@ static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y
     ra.ab = reinterpret_cast<double2 *>(w + o_ab);
     ra.coef = reinterpret_cast<double *>(w + o_coef);
     std::unique_lock<std::mutex> coop;
-    if (!plan.clustered) coop = std::unique_lock<std::mutex>(g_coop_mu);
+    if (!plan.clustered) coop = std::unique_lock<std::mutex>(coop_mutex());
     CUDA_TRY(cudaMemcpyAsync(const_cast<double *>(s.class_size), norm2.data(), C * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(cudaMemcpyAsync(w + o_rhs, V, (size_t)n * C * 8, cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(cudaMemsetAsync(w + o_y, 0, (size_t)n * C * 8, c->stream));
