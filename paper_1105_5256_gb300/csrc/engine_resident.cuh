@@ -49,8 +49,10 @@
 //
 // Where x, r or w live was tried three ways: registers with unrolled loops (12 items a
 // thread spilled, half the capacity), shared memory only (two thirds of the capacity), and
-// tensor memory (kept).  A driver limit makes one CTA an SM of any kernel that allocates
-// tensor memory, so a team's iterations are not overlapped with another team's.
+// tensor memory (kept).  The runtime's occupancy query gives one CTA an SM to any kernel that
+// allocates tensor memory (a 288-thread, 12-register kernel with 1 KB of shared memory: 7 without
+// the tcgen05.alloc of 256 columns, 1 with it), and the registers here allow no second one
+// either, so a team's iterations are not overlapped with another team's.
 #pragma once
 #include "engine_device.cuh"
 #include "resident.h"
@@ -1032,9 +1034,11 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     for (int k = 0; k < U; ++k) {
                         const int i = i0 + k;
                         if (i >= items) break;
+                        const bool act = i < cnt;
                         const It wv = tm_get<V>(tw[k]);
+                        if constexpr (!RS || RP) __syncwarp();
                         if constexpr (RP) y_add(i, RS ? old[k] : tm_get<V>(ta[PRIV ? k : 0]), wv);
-                        It &next = old[k];          // r, or p
+                        It next;                    // r, or p
                         if constexpr (RS) {
                             next = PM::fma(nas, wv, old[k]);
                         } else {
@@ -1043,10 +1047,8 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                             tm_st<V>(tma + 4u * i, r);
                             next = PM::fma(bb, old[k], r);
                         }
+                        if (act) put(line[k], g, next);
                     }
-#pragma unroll
-                    for (int k = 0; k < U; ++k)
-                        if (i0 + k < cnt) put(line[k], g, old[k]);
                 }
                 __syncwarp();
                 tm_wait_st();
@@ -1186,7 +1188,7 @@ __device__ __forceinline__ void res_vector_role(const Solve &s, const ResPlan &p
                     const bool act = i < cnt;
                     It cc;
                     const int in = min(i + 1, cmax - 1);
-                    if constexpr (!RS) __syncwarp();
+                    __syncwarp();
                     if constexpr (PRIV) {
                         if (!MAT && d_tm) tm_wait(ta, td);
                         else tm_wait(ta);
