@@ -56,7 +56,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
                      *inc, "-c", os.path.join(CSRC, s), "-o", o])
     for s in CXX_SOURCES:
         o = os.path.join(BUILD, s + ".o")
-        jobs.append(["g++", "-O2", "-std=c++17", "-fPIC", *inc,
+        # aligned functions: the colouring's inner loop runs 4.7 or 5.6 ms on a 512^2 lattice by
+        # where the linker happens to put it otherwise (64 lattices: creation 135 or 155 ms)
+        jobs.append(["g++", "-O2", "-falign-functions=64", "-std=c++17", "-fPIC", *inc,
                      "-I" + os.path.join(cuda, "include"), "-c", os.path.join(CSRC, s), "-o", o])
 
     def run(cmd):
