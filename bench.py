@@ -210,14 +210,12 @@ def timed_evals(L, ctx, count, params=None, grad=None):
 
 
 def roofline_entry(kernel, n, T, word, r, keep_x, bq_per_pass, peak, src, traffic=None):
-    alg = algorithmic_bytes(n, T, word, r["tile_iters"], keep_x, bq_per_pass, r["passes"])
     info = r["info"]
-    if info["engine"] == 4:     # the resident engine moves no state: what its algorithm would, over the time
-        return {"bound": "alu", "kernel": "resident engine (state on chip)", "traffic": None,
-                "us_per_pass": 1e3 * r["iter_ms"] / max(r["passes"], 1),
-                "algorithmic_bytes_per_pass": alg / max(r["passes"], 1), "peak": peak, "unit": "GB/s",
-                "achieved": alg / (r["iter_ms"] / 1e3) / 1e9, "frac": alg / (r["iter_ms"] / 1e3) / 1e9 / peak,
-                "pass_words": info["pass_words"], "peak_source": src}
+    if info["engine"] == 4:     # the resident engine moves no state: no byte rate describes it
+        return {"bound": "alu", "kernel": "resident engine (state on chip)", "traffic": None, "frac": None,
+                "us_per_pass": 1e3 * r["iter_ms"] / max(r["passes"], 1), "pass_words": info["pass_words"],
+                "note": "state on chip: issue- and exchange-bound, no fraction of a byte rate"}
+    alg = algorithmic_bytes(n, T, word, r["tile_iters"], keep_x, bq_per_pass, r["passes"])
     lean = info["pass_words"] == 4 + (2 if keep_x else 0)     # the lean pass moves the algorithmic words
     achieved = alg / (r["iter_ms"] / 1e3) / 1e9
     return {"bound": "hbm", "kernel": kernel, "achieved": achieved, "peak": peak, "unit": "GB/s",
@@ -438,16 +436,16 @@ def config_batch(L, steps, warmup, peak, src, fp64=True):
             ms += info["ms"]
             vti += info["vertex_tile_iters"]
         word = 4 if prec == L.LD_MIXED else 8
-        # the active bytes: 4 state words a vertex and column of every pass each tile ran
-        alg = 4 * word * info["tile_width"] * vti
-        achieved = alg / (ms / 1e3) / 1e9
-        out[name] = {"value": 256 * steps / (ms / 1e3), "ms_per_step": ms / steps,
-                     "vals": vals, "tile_width": info["tile_width"],
-                     "roofline": {"bound": "alu", "kernel": "k_resident_batch (state on chip)",
-                                  "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                                  "traffic": None, "algorithmic_bytes_per_step": alg / steps,
-                                  "peak_source": src,
-                                  "note": "whole batch wall time over the bytes a streamed pass would move"}}
+        roof = {"bound": "alu", "kernel": "k_resident_batch (state on chip)", "traffic": None, "frac": None,
+                "note": "state on chip: issue- and exchange-bound, no fraction of a byte rate"}
+        if info["engine"] != 4:     # some instances stream: the active bytes, 4 state words a vertex and column
+            alg = 4 * word * info["tile_width"] * vti
+            roof = {"bound": "hbm", "kernel": "k_batch_solve + grid engine + k_resident_batch", "traffic": None,
+                    "achieved": alg / (ms / 1e3) / 1e9, "peak": peak, "unit": "GB/s",
+                    "frac": alg / (ms / 1e3) / 1e9 / peak, "algorithmic_bytes_per_step": alg / steps, "peak_source": src,
+                    "note": "whole batch wall time over the active bytes of all its instances"}
+        out[name] = {"value": 256 * steps / (ms / 1e3), "ms_per_step": ms / steps, "vals": vals,
+                     "tile_width": info["tile_width"], "roofline": roof}
         del b
     res = {"workload": "256 grids, sides U{32..512}, 5-pt d=4 / 13-pt d=2, N=20, tol 1e-6",
            "value": out["mixed"]["value"], "unit": UNIT, "evaluations": 256 * steps,

@@ -398,12 +398,14 @@ ld_status ld_hht_nodes(double lmin, double lmax, int N, double *sigma, double *a
 /* Spectral interval the library uses for a grid kind (Weyl bounds). */
 ld_status ld_grid_bounds(const ld_matrix *Q, double *lmin, double *lmax);
 
-/* Batched evaluation of many independent grid GMRFs of uneven size in one persistent
- * launch (each (instance, tile) a work item).  Qs[count] (grid kinds), distances[count]
- * as in ld_create; every instance gets its own colouring, spectral bounds and nodes.
- * opt: precision, max_iter, tile_width (0: instances whose columns a thread-block cluster can
- * hold run on the resident engine; the width of any others is chosen by timing short runs of
- * the persistent launch per candidate, cached per batch shape), cuda_stream.  An instance whose one-CTA
+/* Batched evaluation of many independent grid GMRFs of uneven size.  Qs[count] (grid kinds),
+ * distances[count] as in ld_create; every instance gets its own colouring, spectral bounds and
+ * nodes.  opt: precision, max_iter, tile_width, cuda_stream.  tile_width 0 (and engine 0):
+ * instances whose columns a thread-block cluster can hold run on the resident engine, one launch
+ * per kind and cluster size with a cluster per (instance, column).  The others, and all
+ * instances where a width is given, share one persistent launch with (instance, tile) as work
+ * items; their width is chosen by timing short runs of it per candidate, cached per shape of
+ * those instances.  Of them an instance whose one-CTA
  * solve would outlast the batch (estimated from its size, its condition number and the
  * measured time of a CTA step) runs on the multi-CTA grid engine instead, several at once
  * on their own streams from host threads; for those to overlap, the process should set
@@ -415,12 +417,15 @@ ld_status ld_batch_create(int count, const ld_matrix *Qs, const int *distances, 
 
 /* Evaluate every instance: logdets[count]; grads[count] = d log det / d kappa2 for
  * scalar-kappa2 5/7-point instances (tr Q^{-1} probed, from the projected seed sums),
- * NaN for the others; grads and info may be NULL.  One CUDA-graph launch: a queue
- * reset, a per-instance prep kernel, the persistent solve (CTAs pull (instance, tile)
- * items, longest first, and run each tile's whole CG-M in one CTA) and a per-instance
- * sum; beside it the grid-engine instances.  info: ms is the host wall time of the whole
- * batch, tile_iters and vertex_tile_iters the exact passes every tile ran.  Errors: the
- * first failing instance's status (no outputs written). */
+ * NaN for the others; grads and info may be NULL.  Side by side on their own streams: the
+ * resident engine's launches, longest columns first; one CUDA graph for the instances of the
+ * persistent launch (a queue reset, a per-instance prep kernel, the solve, whose CTAs pull
+ * (instance, tile) items, longest first, and run each tile's whole CG-M in one CTA, and a
+ * per-instance sum); the grid-engine instances.  info: ms is the host wall time of the whole
+ * batch; engine 4 when every instance ran on the resident engine, else 2; tile_width the width
+ * of the others (with none, the columns that tile_iters counts together: 1 FP64, 2 mixed);
+ * tile_iters and vertex_tile_iters the exact passes every tile ran.  Errors: the first
+ * failing instance's status (no outputs written). */
 ld_status ld_batch_logdet(ld_ctx *ctx, double *logdets, double *grads, ld_info *info);
 
 /* ---------------------------------------------------------------------------
