@@ -101,7 +101,7 @@ struct ld_ctx {
     double kappa2 = 0, tau = 0, scale = 1;
     bool has_field = false, has_mask = false, mask_any = false;
     // the field's range: kappa2 >= 0, so its products' range is kappa2 times this, rounding
-    // included, and ld_set_params need not read the field back and scan it (128^3: about 3 of 140 ms a step)
+    // included, and ld_set_params need not read the field back (16 MB at 128^3) and scan it
     double field_min = NAN, field_max = NAN, field_some = NAN;   // field_some: any finite value
     int distance = 0, nshift = 0;
     bool auto_shift = false;   // n_shifts = 0: N chosen from the quadrature certificate

@@ -41,9 +41,9 @@
 // warps an SM) or by their FP64 units (19 clocks a warp instruction), plus one exchange of 2
 // to 4.5 us an iteration, most of it dependent FP64 instructions; the state costs no DRAM or
 // L2 traffic at all.  Measured a CG iteration over all vectors (before: the streaming or the
-// one-CTA engine): 48 x 40 Matern FP64, 52 vectors, with x 63 -> 9.2 us; 128^2 5-point FP64,
-// 18, with x 143 -> 13.5; 300 x 200 Matern FP32, 19, with x 22.6 -> 8.0; 500 x 333 torus
-// field FP32, 26, with x 29.6 -> 16; 512 x 384 Matern FP64, 18 (FP64 units busy in both) 137
+// one-CTA engine): 48 x 40 Matern FP64, 52 vectors, with x 63 -> 8.5 us; 128^2 5-point FP64,
+// 18, with x 143 -> 13.5; 300 x 200 Matern FP32, 19, with x 22.6 -> 7.2; 500 x 333 torus
+// field FP32, 26, with x 29.6 -> 17.5; 512 x 384 Matern FP64, 18 (FP64 units busy in both) 137
 // -> 114.  Large FP32 problems stay with the lean passes: 1024^2 Matern, 18 vectors: 77 us
 // here, 60 streamed.
 //

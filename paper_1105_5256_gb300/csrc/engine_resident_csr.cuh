@@ -20,7 +20,7 @@
 // shared-memory wavefronts of the gathers (FP32) or the FP64 units on larger ones.  Measured
 // a CG iteration over all vectors (before: one CTA a tile, or the streaming step and product):
 // 64^2 torus FP64, 25 vectors 38.7 -> 11 us; second-order FEM mesh of 13K vertices, 31
-// vectors, FP32 220 -> 10.2, FP64 80 -> 38; of 90K vertices, 33 vectors, FP32 85 -> 44 (the
+// vectors, FP32 220 -> 10.6, FP64 80 -> 39; of 90K vertices, 33 vectors, FP32 85 -> 46 (the
 // last vector of 33 runs in a round of its own, on four vectors a team); FP64 of that size
 // stays with the streaming passes (270 against 206).
 #pragma once
