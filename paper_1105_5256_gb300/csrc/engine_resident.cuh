@@ -139,7 +139,8 @@ struct Sum2 {
     __device__ __forceinline__ Sum2() {}
     __device__ __forceinline__ Sum2(float v) : hi(v), lo(0.f) {}
     __device__ __forceinline__ Sum2(float h, float l) : hi(h), lo(l) {}
-    __device__ __forceinline__ explicit operator double() const { return (double)hi + (double)lo; }
+    // an overflowed sum is infinite, whatever its errors
+    __device__ __forceinline__ explicit operator double() const { return isfinite(hi) ? (double)hi + (double)lo : (double)hi; }
 };
 __device__ __forceinline__ Sum2 operator+(const Sum2 &a, const Sum2 &b) {
     const float s = a.hi + b.hi, t = s - a.hi;

@@ -24,3 +24,15 @@ def test_first_step_length_is_exact(n, prec):
     assert info["engine"] == 4 and info["iters"] == 1
     seed = L.ld_column_terms(ctx)[1][0]
     assert abs(seed - n * (n / d.sum())) <= 1e-12 * n
+
+
+@pytest.mark.parametrize("engine", [0, 1])
+def test_dots_beyond_fp32_are_reported(engine):
+    """|w|^2 of entries 1e20 overflows FP32: infinite, and so is the predicted residual."""
+    n = 700
+    d = 1e20 * (1.0 + synth.rng(n).random(n))
+    ctx = L.ld_create(L.csr_matrix(np.arange(n + 1), np.arange(n), d), 1, 12, 0.5,
+                      L.options(precision=L.LD_MIXED, engine=engine, colouring=np.zeros(n, np.int32), lambda_min=1e20, lambda_max=2e20))
+    with pytest.raises(L.LogDetError) as e:
+        L.ld_logdet(ctx)
+    assert e.value.status == L.LD_ENUMERIC
