@@ -1971,6 +1971,11 @@ ld_status ld_csr_layout(int64_t n, const int64_t *rowptr, const int32_t *colidx,
     if (n < 1 || !rowptr || !colidx || !fits || ncolours < 1 || sms < 1 || n_shifts < 1 || n_shifts > 256)
         return fail(LD_EINVAL, "bad arguments");
     if (precision != LD_FP64 && precision != LD_MIXED) return fail(LD_EINVAL, "bad precision");
+    if (rowptr[0] != 0) return fail(LD_EINVAL, "rowptr[0] must be 0");
+    for (int64_t i = 0; i < n; ++i)
+        if (rowptr[i + 1] < rowptr[i]) return fail(LD_EINVAL, "rowptr not monotone at %lld", (long long)i);
+    for (int64_t e = 0; e < rowptr[n]; ++e)
+        if (colidx[e] < 0 || colidx[e] >= n) return fail(LD_EINVAL, "colidx out of range at %lld", (long long)e);
     ld::CsrPlan p{};
     std::vector<int32_t> r0, e0, e;
     std::vector<uint16_t> lc;

@@ -5,6 +5,7 @@ import resource
 import subprocess
 import sys
 
+import numpy as np
 import pytest
 
 import paper_1105_5256_gb300 as L
@@ -28,6 +29,14 @@ def test_a_matrix_that_fits_is_laid_out(prec):
     rp, ci = torus(64, 64)
     fits, ctas, scanned = L.ld_csr_layout(rp, ci, prec, 25, 20, 152)
     assert fits and 1 < ctas <= 152 and 0 < scanned
+
+
+def test_a_broken_pattern_is_refused():
+    rp, ci = torus(8, 8)
+    for r, c in ((rp + 1, ci), (rp[::-1].copy(), ci), (rp, np.where(np.arange(ci.size) == 7, 64, ci)), (rp, ci - 1)):
+        with pytest.raises(L.LogDetError) as e:
+            L.ld_csr_layout(r, c, L.LD_FP64, 4, 20, 152)
+        assert e.value.status == L.LD_EINVAL
 
 
 CHILD = """
