@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(256) k_residual_sweep(Solve s, int set, int cb
     const int tile = blockIdx.z;
     // y blocks (3D) and segments of the marching axis share blockIdx.y
     const int yb = D3 ? (ny + 7) / 8 : 1;
-    const int m0 = ((int)blockIdx.y / yb) * seg, m1 = min(m0 + seg, nm);
+    const int m0 = ((int)blockIdx.y / yb) * seg, m1 = m0 + min(seg, nm - m0);
     const SweepLane<D3, DIFF> me(nx, ny, blockIdx.x, (int)blockIdx.y % yb, wid, lane);
     const int gx = me.gx, gy = me.gy;
     const bool own = me.own, in = me.in;

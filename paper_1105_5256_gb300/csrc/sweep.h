@@ -29,7 +29,7 @@ struct SweepLane {
 
 // Launch of the sweep: xb x (yb * number of segments) blocks a tile; segments of the marching
 // axis for about eight blocks an SM, at least 16 positions each.  ok: the grid's y and z
-// extents hold it.
+// extents hold it, and no lane's column or count leaves int (one block of columns is 256 wide).
 struct SweepGrid {
     int xb, yb, seg;
     unsigned by;
@@ -37,7 +37,9 @@ struct SweepGrid {
 };
 inline SweepGrid sweep_grid(bool d3, bool diff, int nx, int ny, int nz, int ntiles) {
     constexpr int64_t MAX = 65535;
-    SweepGrid g;
+    SweepGrid g{};
+    constexpr int EDGE = 2147483647 - 512;
+    if (nx > EDGE || ny > EDGE || nz > EDGE) return g;
     const int nm = d3 ? nz : ny, W = (d3 ? 1 : SWEEP_WARPS) * (diff ? 31 : 32);
     g.xb = (nx + W - 1) / W;
     g.yb = d3 ? (ny + SWEEP_WARPS - 1) / SWEEP_WARPS : 1;
@@ -45,7 +47,7 @@ inline SweepGrid sweep_grid(bool d3, bool diff, int nx, int ny, int nz, int ntil
     segs = std::max<int64_t>(1, std::min<int64_t>(segs, (nm + 15) / 16));
     while (segs > 1 && segs * g.yb > MAX) segs = (segs + 1) / 2;
     g.seg = (int)((nm + segs - 1) / segs);
-    g.by = (unsigned)(g.yb * ((nm + g.seg - 1) / g.seg));
+    g.by = (unsigned)(g.yb * (((int64_t)nm + g.seg - 1) / g.seg));
     g.ok = g.yb <= MAX && ntiles <= MAX;
     return g;
 }

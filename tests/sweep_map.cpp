@@ -39,12 +39,18 @@ static int walk(int nx, int ny, int nz, bool per) {
 // gather kernel) exactly where its y blocks or tiles exceed a grid's extent.
 static int launch(bool d3, bool diff, int nx, int ny, int nz, int ntiles) {
     const ld::SweepGrid g = ld::sweep_grid(d3, diff, nx, ny, nz, ntiles);
-    const int nm = d3 ? nz : ny, want = d3 ? (ny + 7) / 8 : 1;
-    int bad = g.ok != (want <= 65535 && ntiles <= 65535);
+    const int nm = d3 ? nz : ny;
+    const int64_t want = d3 ? ((int64_t)ny + 7) / 8 : 1;
+    const int64_t edge = 2147483647 - 512;            // lane columns and block counts beyond it leave int
+    int bad = g.ok != (want <= 65535 && ntiles <= 65535 && nx <= edge && ny <= edge && nz <= edge);
     if (g.ok) {
         const int segs = (int)g.by / g.yb;
         bad += g.by < 1 || g.by > 65535 || (int)g.by % g.yb != 0;
         bad += g.seg < 1 || (int64_t)segs * g.seg < nm || (int64_t)(segs - 1) * g.seg >= nm;
+    }
+    if (g.ok) {              // the last lane of the last warp still has a column number
+        const int64_t last = ((int64_t)g.xb * (d3 ? 1 : ld::SWEEP_WARPS)) * (diff ? 31 : 32);
+        bad += g.xb < 1 || last > 2147483647;
     }
     if (bad) std::printf("launch of %dx%dx%d, %d tiles: %d faults\n", nx, ny, nz, ntiles, bad);
     return bad;
@@ -56,6 +62,11 @@ int main() {
         for (int ntiles : {1, 3, 9, 152, 5000, 65535, 65536})
             for (int nx : {1, 31, 32, 33, 500, 70000}) {
                 for (int ny : {1, 15, 16, 17, 333, 100000, 2000000}) bad += launch(false, diff, nx, ny, 1, ntiles);
+                for (int big : {2147483647, 2147483647 - 500, 2147483647 - 512}) {
+                    bad += launch(false, diff, big, 1, 1, ntiles) + launch(false, diff, 1, big, 1, ntiles);
+                    bad += launch(true, diff, big, 1, 1, ntiles) + launch(true, diff, 1, big, 1, ntiles) +
+                           launch(true, diff, 1, 1, big, ntiles);
+                }
                 for (int ny : {1, 8, 9, 333, 30000, 262144, 524279, 524280, 524281, 600000})
                     for (int nz : {1, 2, 17, 400, 100000}) bad += launch(true, diff, nx, ny, nz, ntiles);
             }
