@@ -325,9 +325,11 @@ ld_status ld_wait_selftest(int64_t limit_ns);
 
 /* The same for whole teams: the solve of ld_logdet on the resident engine's cooperative
  * teams, with the launch's last CTA left out and waits of limit_ns (1e6 .. 1e10).  The
- * CTAs that wait for it give up, the kernel ends, and the call returns LD_ETIMEOUT; the
- * context stays usable.  LD_EUNSUPPORTED: the context's solves use no cooperative teams. */
-ld_status ld_team_wait_selftest(ld_ctx *ctx, int64_t limit_ns);
+ * CTAs that wait for it give up and the kernel ends.  With logdet NULL the call returns
+ * LD_ETIMEOUT; else it goes on as ld_logdet does, on the engine that waits for nobody, and
+ * writes *logdet and info (may be NULL).  The context stays usable.  LD_EUNSUPPORTED: the
+ * context's solves use no cooperative teams. */
+ld_status ld_team_wait_selftest(ld_ctx *ctx, int64_t limit_ns, double *logdet, ld_info *info);
 
 /* The scalar step of the resident engines on count (1 .. 2^24) given sets of dots, host
  * arrays of 4 doubles a set: {|r|^2, p.w, r.w, |w|^2} -> {alpha, beta, predicted

@@ -116,7 +116,7 @@ def library(build_if_missing: bool = False):
         "ld_select_distance": ([vp, i64, dbl, C.c_int, P(i32), vp, P(Info)], st),
         "ld_hutchinson": ([vp, C.c_int, vp, P(dbl), P(dbl), vp, P(Info)], st),
         "ld_wait_selftest": ([i64], st),
-        "ld_team_wait_selftest": ([vp, i64], st),
+        "ld_team_wait_selftest": ([vp, i64, P(dbl), P(Info)], st),
         "ld_scalar_selftest": ([i64, C.c_int, vp, vp], st),
         "ld_invsqrt_mv": ([vp, C.c_int, vp, vp, P(Info)], st),
         "ld_csr_layout": ([i64, vp, vp, C.c_int, C.c_int, C.c_int, C.c_int, P(i32), P(i32), P(i64)], st),
@@ -392,10 +392,16 @@ def ld_wait_selftest(limit_ns: int):
     _check(library().ld_wait_selftest(int(limit_ns)))
 
 
-def ld_team_wait_selftest(ctx: Context, limit_ns: int):
+def ld_team_wait_selftest(ctx: Context, limit_ns: int, go_on: bool = False):
     """The same on a context's cooperative teams, one CTA of which is left out: raises
-    LogDetError(LD_ETIMEOUT) when its team gave up."""
-    _check(library().ld_team_wait_selftest(ctx.handle, int(limit_ns)))
+    LogDetError(LD_ETIMEOUT) when its team gave up; with go_on returns (logdet, info) of the other
+    engine, which takes the solve then."""
+    if not go_on:
+        _check(library().ld_team_wait_selftest(ctx.handle, int(limit_ns), None, None))
+        return None
+    v, info = C.c_double(), Info()
+    _check(library().ld_team_wait_selftest(ctx.handle, int(limit_ns), C.byref(v), C.byref(info)))
+    return v.value, info.as_dict()
 
 
 def ld_scalar_selftest(dots: np.ndarray, precision: int = LD_FP64) -> np.ndarray:

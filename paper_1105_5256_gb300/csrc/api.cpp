@@ -658,8 +658,12 @@ std::mutex &coop_mutex() {
 
 // One probed solve over colours [cb, ce).  On LD_OK, result[0..1] hold
 // sum of terms and sum of seed projections on the device and in *out.
-// test_wait_ns > 0: self-test, see ld_team_wait_selftest.
-ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_info *info, uint64_t test_wait_ns = 0) {
+struct SolveMode {
+    uint64_t test_wait_ns = 0;   // > 0: self-test, see ld_team_wait_selftest
+    bool fall_back = true;       // cooperative teams whose waits ran out: solve on the other engine
+    bool resident = true;        // the resident engine may take the solve
+};
+ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_info *info, SolveMode mode = SolveMode()) {
     Range range("ld solve");
     int64_t launches = 0;
     int iters = 0;
@@ -704,11 +708,11 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         return false;
     };
     if (c->kind == LD_CSR) {
-        if (c->res_state[0] == 1 && c->nshift <= (c->auto_shift ? 64 : c->nshift)) {
+        if (mode.resident && c->res_state[0] == 1 && c->nshift <= (c->auto_shift ? 64 : c->nshift)) {
             const size_t hb = (size_t)c->csr_plan.J * 2 * c->n * c->csr_plan.T * (c->opt.precision == LD_FP64 ? 8 : 4);
             resident = room(c->d_res_rec, ld::engine_csr_rec_bytes(c->csr_plan)) && room(c->d_res_halo, hb);
         }
-    } else if (c->opt.engine == 0 && c->opt.lattice_pass == 0 && !ru) {
+    } else if (mode.resident && c->opt.engine == 0 && c->opt.lattice_pass == 0 && !ru) {
         int &state = c->res_state[want_x0];
         if (state == 0)
             state = ld::engine_resident_plan(c->s, c->ncolours, keep_x0, c->engine == 1, &c->res_plan[want_x0]) == 0 ? 1 : 2;
@@ -719,9 +723,10 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
             resident = room(c->d_res_rec, rb) && room(c->d_res_halo, hb);
         }
     }
-    if (test_wait_ns > 0) {
-        const bool teams = resident && (c->kind == LD_CSR ? c->csr_plan.M : c->res_plan[want_x0].clustered ? 1 : c->res_plan[want_x0].M) > 1;
-        if (!teams) return fail(LD_EUNSUPPORTED, "the context does not run on cooperative teams");
+    const bool coop_teams = resident && (c->kind == LD_CSR || !c->res_plan[want_x0].clustered);
+    if (mode.test_wait_ns > 0) {
+        if (!coop_teams || (c->kind == LD_CSR ? c->csr_plan.M : c->res_plan[want_x0].M) < 2)
+            return fail(LD_EUNSUPPORTED, "the context does not run on cooperative teams");
     }
     // the lean lattice pass (four state words per vertex and column) wherever it applies;
     // the stored-w pass otherwise (FP64, other kinds, the Matern kind with a kept x0)
@@ -751,8 +756,8 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
     }
     if (resident) {
         ld::ResArgs ra{};
-        ra.wait_ns = test_wait_ns > 0 ? test_wait_ns : ld::RES_WAIT_NS;
-        ra.missing = test_wait_ns > 0 ? 1 : 0;
+        ra.wait_ns = mode.test_wait_ns > 0 ? mode.test_wait_ns : ld::RES_WAIT_NS;
+        ra.missing = mode.test_wait_ns > 0 ? 1 : 0;
         ra.cb = cb;
         ra.ce = ce;
         // the iteration cap of the engine this context would otherwise run (whole chunks)
@@ -762,7 +767,7 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
         // Teams of a cooperative launch wait on one another, so two such launches must not share
         // the SMs half each: one at a time on a device, until its results are here.
         // (A cluster's CTAs are scheduled together: clustered plans need no such rule.)
-        if (c->kind == LD_CSR || !c->res_plan[want_x0].clustered) coop = std::unique_lock<std::mutex>(coop_mutex());
+        if (coop_teams) coop = std::unique_lock<std::mutex>(coop_mutex());
         // the engine writes the seed solutions of the colours it solves; the others' are zero
         if (keep_x0 && (cb > 0 || ce < c->ncolours)) CUDA_TRY(cudaMemsetAsync(c->d_x.p, 0, c->d_x.bytes, c->stream));
         CUDA_TRY(cudaEventRecord(c->ev2, c->stream));
@@ -882,6 +887,16 @@ ld_status run_solve(ld_ctx *c, int cb, int ce, bool keep_x0, double out[2], ld_i
     }
     const int dev_status = c->h_pinned[1];
     const int remaining = c->h_pinned[0];
+    if (coop_teams && dev_status == ld::DEV_TIMEOUT && mode.fall_back) {
+        // A team's CTAs may have become resident piecemeal beside another stream's long launch: the
+        // other engines wait for nobody.
+        coop.unlock();
+        mode = SolveMode();
+        mode.resident = false;
+        const ld_status other = run_solve(c, cb, ce, keep_x0, out, info, mode);
+        if (info) info->gpu_launches += launches;
+        return other;
+    }
     for (int v : it) iters = std::max(iters, v);
     int64_t tile_iters = 0;
     for (int t = 0; t < c->ntiles; ++t) {
@@ -1695,6 +1710,14 @@ static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y
     if (status == ld::DEV_OVERFLOW) status = 0;                            // max_iter itself
     *taken = true;
     int64_t launches = 2;
+    // cooperative teams whose waits ran out (see run_solve): the streaming form
+    auto give_up = [&](int s2) {
+        if (plan.clustered || s2 != ld::DEV_TIMEOUT) return false;
+        *taken = false;
+        *launched = launches;
+        return true;
+    };
+    if (give_up(status)) return LD_OK;
     if (status == 0 && remaining == 0) {
         ENGINE_TRY(ld::engine_resident_funmv(s, plan, ra, ncols, c->stream));
         launches += 3;
@@ -1707,6 +1730,7 @@ static ld_status funmv_resident(ld_ctx *c, int ncols, const double *V, double *Y
         CUDA_TRY(cudaMemcpyAsync(Y, ra.y, (size_t)n * C * 8, cudaMemcpyDeviceToHost, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));
     if (good) status = c->h_pinned[1];
+    if (give_up(status)) return LD_OK;
     float ms = 0.f;
     CUDA_TRY(cudaEventElapsedTime(&ms, c->ev0, c->ev1));
     ld_status st = LD_OK;
@@ -1900,12 +1924,17 @@ ld_status ld_scalar_selftest(int64_t count, int precision, const double *dots, d
     return LD_OK;
 }
 
-ld_status ld_team_wait_selftest(ld_ctx *c, int64_t limit_ns) {
+ld_status ld_team_wait_selftest(ld_ctx *c, int64_t limit_ns, double *logdet, ld_info *info) {
     if (!c || limit_ns < 1000000 || limit_ns > 10000000000LL) return fail(LD_EINVAL, "limit_ns out of range");
     if (c->is_batch) return fail(LD_EINVAL, "batched context");
     REJECT_MATFREE(c);
+    SolveMode mode;
+    mode.test_wait_ns = (uint64_t)limit_ns;
+    mode.fall_back = logdet != nullptr;
     double out[2];
-    return run_solve(c, 0, c->ncolours, c->opt.keep_x0 != 0, out, nullptr, (uint64_t)limit_ns);
+    const ld_status st = run_solve(c, 0, c->ncolours, c->opt.keep_x0 != 0, out, info, mode);
+    if (st == LD_OK && logdet) *logdet = out[0];
+    return st;
 }
 
 ld_status ld_hutchinson(ld_ctx *c, int s, const double *Z, double *estimate, double *std_error,

@@ -62,6 +62,30 @@ def test_a_csr_team_gives_up_with_empty_colour_classes(prec):
     assert L.ld_logdet(ctx)[0] == v
 
 
+@pytest.mark.parametrize("keep", [0, 1])
+@pytest.mark.parametrize("csr", [False, True])
+def test_a_solve_whose_teams_gave_up_goes_on_on_the_other_engine(csr, keep):
+    """As ld_logdet does when a team's CTAs become resident piecemeal: the value and seed
+    solutions of the one-CTA engine (both stop at tol: 50 tol of the terms' magnitudes)."""
+    if csr:
+        rp, ci, vv = synth.csr_from_edges(3001, *synth.random_sparse_spd_pattern(9, 3001), 0.3)
+        make = lambda engine: L.ld_create(L.csr_matrix(rp, ci, vv), 1, 16, 1e-8, L.options(engine=engine, keep_x0=keep))
+    else:
+        make = lambda engine: L.ld_create(L.grid_matrix(L.LD_STENCIL_2D13_SQ, (200, 150), 0.3), 2, 20, 1e-8,
+                                          L.options(engine=engine, keep_x0=keep))
+    ctx, ref = make(0), make(2)
+    want, _ = L.ld_logdet(ref)
+    terms, _ = L.ld_column_terms(ref)
+    first, info = L.ld_logdet(ctx)
+    assert info["engine"] == 4
+    got, info = L.ld_team_wait_selftest(ctx, 30_000_000, go_on=True)
+    assert info["engine"] == 2 and abs(got - want) <= 50e-8 * np.abs(terms).sum()
+    if keep:
+        assert np.allclose(L.ld_grad(ctx, [L.LD_P_SCALE]), L.ld_grad(ref, [L.LD_P_SCALE]), rtol=50e-8, atol=0)
+    again, info = L.ld_logdet(ctx)
+    assert info["engine"] == 4 and again == first
+
+
 def test_the_self_test_needs_teams():
     ctx = L.ld_create(L.grid_matrix(L.LD_STENCIL_2D5, (32, 16), 0.5), 1, 16, 1e-8, L.options(engine=1))
     with pytest.raises(L.LogDetError) as e:
